@@ -110,6 +110,7 @@ DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base) {
   dt.d.a_lo = nullptr;
   dt.d.c_lo = nullptr;
   dt.red_f = pl->has_tri ? nullptr : (const float*)(base + pl->off_red);
+  dt.low_rb = pl->low >= 0 ? (double*)(base + pl->off_low) : nullptr;
   dt.status = (int*)(base + pl->off_status);
   dt.acc = (double*)(base + pl->off_acc);
   dt.tri_d = TriFactors<double>{};
@@ -293,8 +294,8 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   if (d->precision == PP_FP32_REFINED) off = align_up(off + 4 * (size_t)ny * g.nz * g.nx, 256);
   pl->off_r1 = off;      // the first correction's residual (FP32 pair per cell) for the later ones
   if (pl->refine >= 2) off = align_up(off + 8 * (size_t)ny * g.nz * g.nx, 256);
-  pl->off_scratch = off;
-  if (L >= 0) off = align_up(off + 16 * (size_t)ny * (L + 1) * (2 * L + 1), 256);
+  pl->off_low = off;     // pivots of the FP64 low modes
+  if (L >= 0) off = align_up(off + 8 * (size_t)ny * (L + 1) * (2 * L + 1), 256);
   pl->off_tables = off; off = align_up(off + tab_bytes, 256);
   pl->off_status = off; off = align_up(off + 256, 256);
   pl->off_acc = off;    off = align_up(off + 256, 256);
@@ -338,16 +339,13 @@ poisson_status poisson_set_workspace(poisson_plan_t pl, void* ws, size_t bytes, 
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return PS_ECUDA;
   pl->ws = base;
   pl->dt = pp::bind_tables(pl, base);
-  if (!pl->has_tri && pl->parts > 1) {
-    if (launch_reduced_setup(pl->g, pl->dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, (float*)(base + pl->off_red),
-                             st) != cudaSuccess)
-      return PS_ECUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return PS_ECUDA;
-  }
-  if (pl->has_tri) {
-    if (launch_tridiag_setup(pl->g, pl->dt, pl->parts, st) != cudaSuccess) return PS_ECUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return PS_ECUDA;
-  }
+  if (pp::launch_low_setup(pl->g, pl->dt, pl->low, st) != cudaSuccess) return PS_ECUDA;
+  if (!pl->has_tri && pl->parts > 1 &&
+      launch_reduced_setup(pl->g, pl->dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, (float*)(base + pl->off_red),
+                           st) != cudaSuccess)
+    return PS_ECUDA;
+  if (pl->has_tri && launch_tridiag_setup(pl->g, pl->dt, pl->parts, st) != cudaSuccess) return PS_ECUDA;
+  if (cudaStreamSynchronize(st) != cudaSuccess) return PS_ECUDA;
   return PS_OK;
 }
 
@@ -407,7 +405,8 @@ void timer_end(Exec& ex, const char* name) {
   } while (0)
 
 // Spectral middle of a solve on the x-transformed spectral buffer (Sec. 3.2 steps (4)-(6)):
-// forward z-transform, wall-normal systems, the (0, 0) mode, inverse z-transform.
+// forward z-transform, wall-normal systems (the (0, 0) mode and the FP64 low modes among them),
+// inverse z-transform.
 template <typename T>
 poisson_status spectral_mid(Exec& ex, cplx<T>* spec, GaugeMode gauge);
 
@@ -417,8 +416,8 @@ poisson_status spectral_mid<double>(Exec& ex, cplx<double>* spec, GaugeMode gaug
   const Geometry& g = pl->g;
   cudaStream_t st = ex.st;
   PP_TRY_N("fft_z_fwd", launch_fft_z<double>(g, ex.dt, pl->fz, -1, spec, st));
-  PP_TRY_N("tridiag_pdd", launch_tridiag_factored(g, ex.dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, spec, st));
-  PP_TRY_N("mode00", launch_mode00<double>(g, ex.dt, gauge, spec, st));
+  PP_TRY_N("tridiag_pdd", launch_tridiag_factored(g, ex.dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, spec,
+                                                  side_args(ex.dt, -1, gauge), st));
   PP_TRY_N("fft_z_inv", launch_fft_z<double>(g, ex.dt, pl->fz, +1, spec, st));
   return PS_OK;
 }
@@ -436,7 +435,9 @@ poisson_status spectral_chain_f32(Exec& ex, cplx<float>* spec, GaugeMode gauge) 
   cudaStream_t st = ex.st;
   const int sw = pl->slab_cols;
   const bool two = pl->chain_streams > 1 && pl->chain_st != nullptr;
-  cplx<double>* scr = (cplx<double>*)(ex.ws + pl->off_scratch);
+  const SideArgs side = side_args(ex.dt, pl->low, gauge);
+  SideArgs none = side;
+  none.nsys = 0;
   const bool timed = timer_begin(ex);
   if (two) {
     if (cudaEventRecord(pl->chain_ev[0], st) != cudaSuccess) return PS_ECUDA;
@@ -446,11 +447,7 @@ poisson_status spectral_chain_f32(Exec& ex, cplx<float>* spec, GaugeMode gauge) 
     const int hi = lo + sw < g.ncols ? lo + sw : g.ncols;
     cudaStream_t s = (two && (k & 1)) ? pl->chain_st : st;
     PP_TRY_Q(launch_fft_z_fast<float>(g, ex.dt.f, -1, spec, s, lo, hi));
-    PP_TRY_Q(launch_tridiag_reg_f32(g, ex.dt, pl->parts, pl->low, spec, s, lo, hi));
-    if (lo == 0) {
-      if (pl->low >= 0) PP_TRY_Q(launch_tridiag_low64(g, ex.dt, pl->parts, pl->low, spec, scr, s));
-      PP_TRY_Q(launch_mode00<float>(g, ex.dt, gauge, spec, s));
-    }
+    PP_TRY_Q(launch_tridiag_reg_f32(g, ex.dt, pl->parts, pl->low, spec, lo == 0 ? side : none, s, lo, hi));
     PP_TRY_Q(launch_fft_z_fast<float>(g, ex.dt.f, +1, spec, s, lo, hi));
   }
   if (two) {
@@ -468,15 +465,11 @@ poisson_status spectral_mid<float>(Exec& ex, cplx<float>* spec, GaugeMode gauge)
   cudaStream_t st = ex.st;
   if (pl->slab_cols > 0) return spectral_chain_f32(ex, spec, gauge);
   PP_TRY_N("fft_z_fwd", launch_fft_z<float>(g, ex.dt, pl->fz, -1, spec, st));
+  const SideArgs side = side_args(ex.dt, pl->low, gauge);
   if (pl->has_tri)
     PP_TRY_N("tridiag_pdd", launch_tridiag_factored_f32(g, ex.dt, pl->parts, pl->low, pl->tridiag == PT_PDD_TRUNCATED,
-                                                        spec, st));
-  else PP_TRY_N("tridiag_pdd", launch_tridiag_reg_f32(g, ex.dt, pl->parts, pl->low, spec, st));
-  if (pl->low >= 0) {
-    cplx<double>* scr = (cplx<double>*)(ex.ws + pl->off_scratch);
-    PP_TRY_N("tridiag_low64", launch_tridiag_low64(g, ex.dt, pl->parts, pl->low, spec, scr, st));
-  }
-  PP_TRY_N("mode00", launch_mode00<float>(g, ex.dt, gauge, spec, st));
+                                                        spec, side, st));
+  else PP_TRY_N("tridiag_pdd", launch_tridiag_reg_f32(g, ex.dt, pl->parts, pl->low, spec, side, st));
   PP_TRY_N("fft_z_inv", launch_fft_z<float>(g, ex.dt, pl->fz, +1, spec, st));
   return PS_OK;
 }

@@ -47,6 +47,16 @@ struct DevTables {
   TriFactors<double> tri_d;  // FP64 plans
   TriFactors<float> tri_f;   // FP32 and FP32-refined plans
   const float* red_f;        // FP32 register-kernel plans: per-mode LU of the reduced interface system
+  double* low_rb;            // FP32 forms: pivots 1/beta_j of the FP64 low modes, [system of the list][row]
+};
+
+// The modes solved by extra CTAs of the wall-normal launch (low_modes.cuh): the (0, 0) mode and,
+// with low >= 0, the FP64 systems with kx <= low, |kz| <= low: nsys systems, `threads` threads to
+// each, `per` systems to a CTA, n CTAs (0: none in this launch).
+struct SideArgs {
+  int n, nsys, per, threads, low, gauge;
+  const double *a, *c, *rb, *dy, *h;
+  double* acc;
 };
 
 struct Geometry {
@@ -130,24 +140,14 @@ cudaError_t launch_fft_z_fast(const Geometry& g, const Tables<T>& tt, int sign, 
 template <typename T>
 int fft_z_fast_tile(const Geometry& g);
 
-template <typename TD, typename TC>
-cudaError_t launch_tridiag(const Geometry& g, const DevTables& tb, int parts, int low_modes, bool low_list,
-                           cplx<TD>* spec, cudaStream_t st);
-
-template <>
-cudaError_t launch_tridiag<double, double>(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                           bool low_list, cplx<double>* spec, cudaStream_t st);
-template <>
-cudaError_t launch_tridiag<float, float>(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                         bool low_list, cplx<float>* spec, cudaStream_t st);
-
 // PDD with the precomputed factors tb.tri_d / tb.tri_f (setup once per plan, then per solve).
 cudaError_t launch_tridiag_setup(const Geometry& g, const DevTables& tb, int parts, cudaStream_t st);
 // trunc: the truncated reduced system of Sec. 2.2 (framed coupling entries dropped).
+// sd: the modes solved by the launch's extra CTAs (side_args; nsys = 0 for none).
 cudaError_t launch_tridiag_factored(const Geometry& g, const DevTables& tb, int parts, bool trunc, cplx<double>* spec,
-                                    cudaStream_t st);
+                                    const SideArgs& sd, cudaStream_t st);
 cudaError_t launch_tridiag_factored_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes, bool trunc,
-                                        cplx<float>* spec, cudaStream_t st);
+                                        cplx<float>* spec, const SideArgs& sd, cudaStream_t st);
 
 // FP32 PDD with each block of m = ny/P rows held in one thread's registers and its factors
 // computed on the fly (no factor tables): m in {1, 2, 3, 4, 6, 8, 12, 16, 24}, P <= 256, S = 256/P
@@ -162,24 +162,21 @@ __host__ __device__ inline int reg_systems_per_cta(int P) { return P >= 256 ? 1 
 // warp-scan variant only (P a power of two <= 32), with kx_lo a multiple of
 // reg_systems_per_cta(P), and is refused (cudaErrorNotSupported) otherwise.
 cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                   cplx<float>* spec, cudaStream_t st, int kx_lo = 0, int kx_hi = -1);
+                                   cplx<float>* spec, SideArgs sd, cudaStream_t st, int kx_lo = 0, int kx_hi = -1);
 __host__ __device__ inline bool scan_tridiag_ok(int ny, int P) { return reg_tridiag_ok(ny, P) && P <= 32 && (P & (P - 1)) == 0; }
 // Bytes of the reduced-system table of the register kernel, and its FP64 set-up (once per plan).
 size_t reduced_table_bytes(const Geometry& g, int parts);
 cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int parts, bool trunc, float* tab,
                                  cudaStream_t st);
 
-// FP64 re-solve of the low-mode list on FP32 spectral data (intermediates in FP64 scratch).
-cudaError_t launch_tridiag_low64(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                 cplx<float>* spec, cplx<double>* scratch, cudaStream_t st);
-
 // Gauge modes of the (0, 0) solve: plain zero weighted mean; GAUGE_STORE_MEAN also stores the
 // rhs mean <f> in tb.acc[0]; GAUGE_OFFSET shifts the result so that the running pressure
 // total (weighted sum tb.acc[1]) plus this correction has zero weighted mean.
 enum GaugeMode { GAUGE_ZERO = 0, GAUGE_STORE_MEAN = 1, GAUGE_OFFSET = 2 };
-template <typename TD>
-cudaError_t launch_mode00(const Geometry& g, const DevTables& tb, GaugeMode gauge, cplx<TD>* spec,
-                          cudaStream_t st);
+// The modes solved apart: the (0, 0) mode with the gauge, and the FP64 low modes (low >= 0).
+SideArgs side_args(const DevTables& tb, int low, GaugeMode gauge);
+// Their FP64 pivots tb.low_rb (once per plan; low >= 1).
+cudaError_t launch_low_setup(const Geometry& g, const DevTables& tb, int low, cudaStream_t st);
 
 template <typename T>
 cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, T* u, T* v, T* w, double dt,
@@ -252,7 +249,7 @@ struct poisson_plan_s {
   std::vector<double> faces, dy, h, a, c, lamx, lamz;
   std::vector<unsigned char> host_tables;   // staging image of the device tables
   // workspace layout (byte offsets)
-  size_t off_spec, off_pbuf, off_pbuf2, off_r1, off_scratch, off_tables, off_status, off_acc, off_tri, off_red,
+  size_t off_spec, off_pbuf, off_pbuf2, off_r1, off_low, off_tables, off_status, off_acc, off_tri, off_red,
       ws_bytes;
   bool has_tri;   // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans with m = ny/P outside the register kernel's set)
   size_t tab_offsets[32];

@@ -21,173 +21,13 @@
 // e_j = beta_j - c_j,  e_j = sigma + a_j e_{j-1} / beta_{j-1}  (all terms >= 0), so the
 // weakly dominant low modes keep full relative accuracy.
 //
-// The singular (0, 0) mode is skipped here and solved by k_mode00.  In the FP32 forms the
-// lowest modes are skipped by the FP32 pass and re-solved in FP64 by a list pass whose
-// intermediates live in an FP64 scratch buffer.
+// The singular (0, 0) mode and, in the FP32 forms, the lowest modes (FP64 systems) are skipped by
+// the main pass and solved by extra CTAs at the head of its grid (low_modes.cuh).
 #include "internal.h"
+#include "low_modes.cuh"
 #include "tridiag_scan.cuh"
 
 namespace pp {
-
-struct TriParams {
-  int P, m, S;        // blocks per system, rows per block, systems per CTA
-  int low;            // low-mode half-width L (-1: none)
-  int list;           // 1: iterate the low-mode list instead of all modes
-  int nsys;           // number of systems addressed by the grid
-};
-
-template <typename TD, typename TC, bool SCR>
-__global__ void __launch_bounds__(512) k_tridiag(Geometry g, TriParams tp, const TC* __restrict__ a,
-                                                 const TC* __restrict__ c, const double* __restrict__ lamx,
-                                                 const double* __restrict__ lamz, cplx<TD>* __restrict__ spec,
-                                                 cplx<TC>* __restrict__ scratch) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int P = tp.P, m = tp.m, S = tp.S;
-  const int nth = P * S;
-  const int tid = threadIdx.x;
-  const int b = tid / S, s = tid - b * S;
-  TC* rbs = reinterpret_cast<TC*>(smem_raw);          // [m][nth] pivots 1/beta_j
-  TC* gvs = rbs + (size_t)m * nth;                      // [m][nth] forward-eliminated spike
-  TC* itf = gvs + (size_t)m * nth;                      // interface arrays, [18][P*S]
-  const int PS = P * S;
-  TC* xFr = itf;          TC* xFi = itf + PS;      TC* xLr = itf + 2 * PS;  TC* xLi = itf + 3 * PS;
-  TC* vFs = itf + 4 * PS; TC* vLs = itf + 5 * PS;  TC* wFs = itf + 6 * PS;  TC* wLs = itf + 7 * PS;
-  TC* alr = itf + 8 * PS; TC* ali = itf + 9 * PS;  TC* ber = itf + 10 * PS; TC* bei = itf + 11 * PS;
-  TC* y0r = itf + 12 * PS; TC* y0i = itf + 13 * PS; TC* y1r = itf + 14 * PS; TC* y1i = itf + 15 * PS;
-  TC* X01s = itf + 16 * PS; TC* X11s = itf + 17 * PS;
-
-  const int sys = blockIdx.x * S + s;
-  int kx = 0, kz = 0;
-  bool active = sys < tp.nsys;
-  if (active) {
-    if (tp.list) {
-      const int nlx = tp.low + 1;
-      kx = sys % nlx;
-      const int q = sys / nlx;
-      kz = q <= tp.low ? q : g.nz - (q - tp.low);
-    } else {
-      kz = sys / g.ncols;
-      kx = sys - kz * g.ncols;
-      if (is_low(kx, kz, g.nz, tp.low)) active = false;
-    }
-    if (kx == 0 && kz == 0) active = false;
-  }
-  const TC sigma = active ? TC(-(lamx[kx] + lamz[kz])) : TC(1);
-  const size_t rstride = (size_t)g.nz * g.pitch;
-  cplx<TD>* col = spec + (size_t)kz * g.pitch + kx;
-  cplx<TC>* scol = SCR ? scratch + sys : nullptr;
-  const size_t sstride = SCR ? (size_t)tp.nsys : 0;
-  const int r0 = b * m;
-
-  // ---- 1. forward elimination ------------------------------------------------------------
-  cplx<TC> gg = mk<TC>(TC(0), TC(0));
-  TC e = TC(0), rbp = TC(0), gvv = TC(0);
-  cplx<TC> xL = mk<TC>(TC(0), TC(0));
-  TC vL = TC(0), wL = TC(0);
-  if (active) {
-    e = a[r0] + sigma;
-    gvv = a[r0];
-    for (int i = 0; i < m; ++i) {
-      const int j = r0 + i;
-      const cplx<TD> F = ld_c(col + (size_t)j * rstride);
-      const cplx<TC> rhs = mk<TC>(-TC(F.x), -TC(F.y));
-      if (i == 0) {
-        gg = rhs;
-      } else {
-        const TC mult = a[j] * rbp;
-        e = sigma + mult * e;
-        gg = mk<TC>(rhs.x + mult * gg.x, rhs.y + mult * gg.y);
-        gvv = mult * gvv;
-      }
-      const TC rb = TC(1) / (c[j] + e);
-      rbs[(size_t)i * nth + tid] = rb;
-      gvs[(size_t)i * nth + tid] = gvv;
-      if constexpr (SCR) st_c(scol + (size_t)j * sstride, gg);
-      else st_c(col + (size_t)j * rstride, gg);
-      rbp = rb;
-    }
-    xL = scale(gg, rbp);
-    vL = gvv * rbp;
-    wL = c[r0 + m - 1] * rbp;
-  }
-
-  auto gload = [&](int j) -> cplx<TC> {
-    if constexpr (SCR) return ld_c(scol + (size_t)j * sstride);
-    else return ld_c(col + (size_t)j * rstride);
-  };
-
-  cplx<TC> alpha = mk<TC>(TC(0), TC(0)), beta = mk<TC>(TC(0), TC(0));
-  if (P > 1) {
-    // ---- 2. first-row values of x~, v, w --------------------------------------------------
-    cplx<TC> xn = xL;
-    TC vn = vL, wn = wL;
-    if (active) {
-      for (int i = m - 2; i >= 0; --i) {
-        const int j = r0 + i;
-        const TC rb = rbs[(size_t)i * nth + tid];
-        const TC cj = c[j];
-        const cplx<TC> gj = gload(j);
-        xn = mk<TC>((gj.x + cj * xn.x) * rb, (gj.y + cj * xn.y) * rb);
-        vn = (gvs[(size_t)i * nth + tid] + cj * vn) * rb;
-        wn = cj * rb * wn;
-      }
-    }
-    const int me = b * S + s;
-    xFr[me] = xn.x; xFi[me] = xn.y; xLr[me] = xL.x; xLi[me] = xL.y;
-    vFs[me] = vn; vLs[me] = vL; wFs[me] = wn; wLs[me] = wL;
-    __syncthreads();
-    // ---- 3. exact reduced system over the P-1 interfaces (unknowns L_i, F_{i+1}) --------------
-    // L_i     = x~L_i + vL_i L_{i-1} + wL_i F_{i+1}
-    // F_{i+1} = x~F_{i+1} + vF_{i+1} L_i + wF_{i+1} F_{i+2}
-    if (b == 0 && active) {
-      TC pX01 = TC(0);
-      cplx<TC> py0 = mk<TC>(TC(0), TC(0));
-      for (int i = 0; i < P - 1; ++i) {
-        const int ii = i * S + s, in = (i + 1) * S + s;
-        const TC vLi = vLs[ii], wLi = wLs[ii], vFn = vFs[in], wFi = wFs[ii];
-        // eliminating z_{i-1} fills entry (0,1): L_i reaches F_{i+1} through L_{i-1} and F_i
-        const TC d01 = -wLi - vLi * wFi * pX01, d10 = -vFn;
-        const TC inv = TC(1) / (TC(1) - d01 * d10);
-        const TC X00 = inv, X01 = -d01 * inv, X10 = -d10 * inv, X11 = inv;
-        const cplx<TC> q0 = mk<TC>(xLr[ii] + vLi * py0.x, xLi[ii] + vLi * py0.y);
-        const cplx<TC> q1 = mk<TC>(xFr[in], xFi[in]);
-        const cplx<TC> y0 = mk<TC>(X00 * q0.x + X01 * q1.x, X00 * q0.y + X01 * q1.y);
-        const cplx<TC> y1 = mk<TC>(X10 * q0.x + X11 * q1.x, X10 * q0.y + X11 * q1.y);
-        y0r[ii] = y0.x; y0i[ii] = y0.y; y1r[ii] = y1.x; y1i[ii] = y1.y;
-        X01s[ii] = X01; X11s[ii] = X11;
-        pX01 = X01;
-        py0 = y0;
-      }
-      cplx<TC> z1n = mk<TC>(TC(0), TC(0));   // F_{i+2}
-      for (int i = P - 2; i >= 0; --i) {
-        const int ii = i * S + s;
-        const TC t = (i == P - 2) ? TC(0) : wFs[(i + 1) * S + s];
-        const cplx<TC> z0 = mk<TC>(y0r[ii] + t * z1n.x * X01s[ii], y0i[ii] + t * z1n.y * X01s[ii]);
-        const cplx<TC> z1 = mk<TC>(y1r[ii] + t * z1n.x * X11s[ii], y1i[ii] + t * z1n.y * X11s[ii]);
-        alr[(i + 1) * S + s] = z0.x; ali[(i + 1) * S + s] = z0.y;   // alpha of block i+1 = L_i
-        ber[ii] = z1.x; bei[ii] = z1.y;                              // beta of block i = F_{i+1}
-        z1n = z1;
-      }
-    }
-    __syncthreads();
-    if (b > 0) alpha = mk<TC>(alr[me], ali[me]);
-    if (b < P - 1) beta = mk<TC>(ber[me], bei[me]);
-  }
-
-  // ---- 4. final backward sweep with the neighbour values folded in --------------------------
-  if (active) {
-    cplx<TC> xn = beta;   // x_{r1+1}; multiplied by c_{r1} (0 for the last block)
-    for (int i = m - 1; i >= 0; --i) {
-      const int j = r0 + i;
-      const TC rb = rbs[(size_t)i * nth + tid];
-      const TC gv = gvs[(size_t)i * nth + tid];
-      const TC cj = c[j];
-      const cplx<TC> gj = gload(j);
-      xn = mk<TC>((gj.x + alpha.x * gv + cj * xn.x) * rb, (gj.y + alpha.y * gv + cj * xn.y) * rb);
-      st_c(col + (size_t)j * rstride, mk<TD>(TD(xn.x), TD(xn.y)));
-    }
-  }
-}
 
 // ---- PDD with per-mode factors (the production path) ----------------------------------------
 // The RHS-independent part of each block's elimination (pivots, spikes, first-row weights)
@@ -252,9 +92,14 @@ __global__ void __launch_bounds__(256) k_tridiag_setup(Geometry g, int P, int m,
 template <typename T, bool FULL>
 __global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int m, int S, int low, int trunc,
                                                           const T* __restrict__ a, const T* __restrict__ c,
-                                                          TriFactors<T> tf, cplx<T>* __restrict__ spec) {
+                                                          TriFactors<T> tf, cplx<T>* __restrict__ spec,
+                                                          SideArgs sd) {
   constexpr int CH = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x < sd.n) {
+    low_system<T>(g, sd, spec, blockIdx.x, smem_raw);
+    return;
+  }
   T* sm = reinterpret_cast<T*>(smem_raw);
   const int PS = P * S;
   T* xFr = sm;          T* xFi = sm + PS;      T* xLr = sm + 2 * PS;  T* xLi = sm + 3 * PS;
@@ -264,7 +109,7 @@ __global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int
   const int nsys = tf.nsys;
   const int tid = threadIdx.x;
   const int b = tid / S, s = tid - b * S;
-  const int sys = blockIdx.x * S + s;
+  const int sys = ((int)blockIdx.x - sd.n) * S + s;
   int kx = 0, kz = 0;
   bool active = sys < nsys;
   if (active) {
@@ -481,10 +326,14 @@ template <int M>
 __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S, int low, const float* __restrict__ a,
                                                         const float* __restrict__ c, const double* __restrict__ lamx,
                                                         const double* __restrict__ lamz, const float* __restrict__ rtab,
-                                                        cplx<float>* __restrict__ spec) {
+                                                        cplx<float>* __restrict__ spec, SideArgs sd) {
   // shared: the interface arrays (6 x NT floats), the CTA's slice of the reduced-system table
   // (5 (P-1) S floats, [i][k][s]), then the blocks' rows [row][thread]
   extern __shared__ __align__(16) float red_s[];
+  if ((int)blockIdx.x < sd.n) {
+    low_system<float>(g, sd, spec, blockIdx.x, reinterpret_cast<unsigned char*>(red_s));
+    return;
+  }
   enum { R_XFR, R_XFI, R_XLR, R_XLI, R_ZR, R_ZI };
   const int NT = P * S;
 #define RED(k, idx) red_s[(k) * NT + (idx)]
@@ -493,7 +342,7 @@ __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S
   const int nsys = g.nz * g.ncols;
   const int tid = threadIdx.x;
   const int b = tid / S, s = tid - b * S;
-  const int sys0 = blockIdx.x * S;
+  const int sys0 = ((int)blockIdx.x - sd.n) * S;
   const int sys = sys0 + s;
   int kx = 0, kz = 0;
   bool active = sys < nsys;
@@ -599,63 +448,92 @@ __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S
   }
 }
 
+// Pivots of the modes solved apart, one thread per system of the list (low_system's order):
+// rb[sys ny + j] = 1 / beta_j by the margin recurrence, in FP64.
+__global__ void __launch_bounds__(32) k_low_setup(Geometry g, int n, int low, const double* __restrict__ a,
+                                                  const double* __restrict__ c, const double* __restrict__ lamx,
+                                                  const double* __restrict__ lamz, double* __restrict__ rb) {
+  const int sys = blockIdx.x * blockDim.x + threadIdx.x;
+  if (sys < 1 || sys >= n) return;
+  const int kx = sys % (low + 1), q = sys / (low + 1);
+  const int kz = q <= low ? q : g.nz - (q - low);
+  const double sigma = -(lamx[kx] + lamz[kz]);
+  double e = 0.0, r = 0.0;
+  for (int j = 0; j < g.ny; ++j) {
+    e = j > 0 ? sigma + a[j] * e * r : sigma;
+    r = 1.0 / (c[j] + e);
+    rb[(size_t)sys * g.ny + j] = r;
+  }
+}
+
 // ------------------------------------------------------------------------------ launchers
 template <typename K>
 static cudaError_t prep(K kernel, size_t smem) {
   return ensure_smem_limit((const void*)kernel, smem);
 }
 
-template <typename TC> static const TC* coef_a(const DevTables& tb);
-template <> const double* coef_a<double>(const DevTables& tb) { return tb.d.a; }
-template <> const float* coef_a<float>(const DevTables& tb) { return tb.f.a; }
-template <typename TC> static const TC* coef_c(const DevTables& tb);
-template <> const double* coef_c<double>(const DevTables& tb) { return tb.d.c; }
-template <> const float* coef_c<float>(const DevTables& tb) { return tb.f.c; }
+// The modes solved apart (low_modes.cuh): as extra CTAs of the main launch while a system's work
+// area (16 bytes per row) stays below the 48 KB that every launch may ask for without lowering the
+// main pass's occupancy, else (ny > 3072) as a launch of their own before it.
+static constexpr size_t kSideFusedBytes = 48 * 1024;
 
-static size_t tridiag_smem(int P, int m, int S, size_t tc) {
-  return ((size_t)2 * m * P * S + (size_t)18 * P * S) * tc;
+template <typename TD>
+__global__ void __launch_bounds__(128) k_tridiag_side(Geometry g, SideArgs sd, cplx<TD>* __restrict__ spec) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  low_system<TD>(g, sd, spec, blockIdx.x, smem_raw);
 }
 
-static int pick_systems_per_cta(int P, int m, size_t tc) {
-  int S = 32;
-  while (S > 8 && (tridiag_smem(P, m, S, tc) > 100 * 1024 || P * S > 512)) S /= 2;
-  while (S > 1 && (tridiag_smem(P, m, S, tc) > 200 * 1024 || P * S > 512)) S /= 2;
-  return S;
+// Groups of sd for CTAs of `threads` threads: a warp per system up to 256 rows, else 128 threads.
+static void side_groups(const Geometry& g, SideArgs& sd, int threads) {
+  const int whole = threads & ~31;
+  sd.threads = g.ny <= 256 ? 32 : (whole < 128 ? whole : 128);
+  sd.per = whole / sd.threads;
+  while (sd.per > 1 && (size_t)16 * g.ny * sd.per > kSideFusedBytes) --sd.per;
+  sd.n = (sd.nsys + sd.per - 1) / sd.per;
 }
 
-template <typename TD, typename TC, bool SCR>
-cudaError_t launch_tridiag_impl(const Geometry& g, const DevTables& tb, int parts, int low_modes, bool low_list,
-                                cplx<TD>* spec, cplx<TC>* scratch, cudaStream_t st) {
-  TriParams tp;
-  tp.P = parts;
-  tp.m = g.ny / parts;
-  tp.low = low_modes;
-  tp.list = low_list ? 1 : 0;
-  tp.nsys = low_list ? (low_modes + 1) * (2 * low_modes + 1) : g.nz * g.ncols;
-  tp.S = pick_systems_per_cta(tp.P, tp.m, sizeof(TC));
-  const size_t smem = tridiag_smem(tp.P, tp.m, tp.S, sizeof(TC));
-  const dim3 grid((tp.nsys + tp.S - 1) / tp.S);
-  auto kern = k_tridiag<TD, TC, SCR>;
-  cudaError_t e;
-  if ((e = prep(kern, smem)) != cudaSuccess) return e;
-  kern<<<grid, tp.P * tp.S, smem, st>>>(g, tp, coef_a<TC>(tb), coef_c<TC>(tb), tb.lamx, tb.lamz, spec, scratch);
+// sd for a main launch of CTAs of `threads` threads (n = 0 after a launch of its own); smem
+// raised to the work area.
+template <typename TD>
+static cudaError_t prepare_side(const Geometry& g, SideArgs& sd, int threads, size_t& smem, cplx<TD>* spec,
+                                cudaStream_t st) {
+  sd.n = 0;
+  if (sd.nsys == 0) return cudaSuccess;
+  if ((size_t)16 * g.ny <= kSideFusedBytes) {
+    side_groups(g, sd, threads);
+    const size_t need = (size_t)16 * g.ny * sd.per;
+    if (smem < need) smem = need;
+    return cudaSuccess;
+  }
+  side_groups(g, sd, 128);
+  const size_t need = (size_t)16 * g.ny;
+  cudaError_t e = prep(k_tridiag_side<TD>, need);
+  if (e != cudaSuccess) return e;
+  k_tridiag_side<TD><<<sd.n, 128, need, st>>>(g, sd, spec);
+  sd.n = 0;
   return cudaGetLastError();
 }
 
-template <>
-cudaError_t launch_tridiag<double, double>(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                           bool low_list, cplx<double>* spec, cudaStream_t st) {
-  return launch_tridiag_impl<double, double, false>(g, tb, parts, low_modes, low_list, spec, nullptr, st);
-}
-template <>
-cudaError_t launch_tridiag<float, float>(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                         bool low_list, cplx<float>* spec, cudaStream_t st) {
-  return launch_tridiag_impl<float, float, false>(g, tb, parts, low_modes, low_list, spec, nullptr, st);
+SideArgs side_args(const DevTables& tb, int low, GaugeMode gauge) {
+  SideArgs sd;
+  sd.nsys = low >= 0 ? (low + 1) * (2 * low + 1) : 1;
+  sd.n = sd.per = sd.threads = 0;   // set for each launch (prepare_side)
+  sd.low = low;
+  sd.gauge = (int)gauge;
+  sd.a = tb.d.a;
+  sd.c = tb.d.c;
+  sd.rb = tb.low_rb;
+  sd.dy = tb.dy;
+  sd.h = tb.h;
+  sd.acc = tb.acc;
+  return sd;
 }
 
-cudaError_t launch_tridiag_low64(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                 cplx<float>* spec, cplx<double>* scratch, cudaStream_t st) {
-  return launch_tridiag_impl<float, double, true>(g, tb, parts, low_modes, true, spec, scratch, st);
+cudaError_t launch_low_setup(const Geometry& g, const DevTables& tb, int low, cudaStream_t st) {
+  if (low < 1) return cudaSuccess;   // low = 0: the (0, 0) mode only
+  const int n = (low + 1) * (2 * low + 1);
+  k_low_setup<<<(n + 31) / 32, 32, 0, st>>>(g, n, low, tb.d.a, tb.d.c, tb.lamx, tb.lamz, tb.low_rb);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_tridiag_setup(const Geometry& g, const DevTables& tb, int parts, cudaStream_t st) {
@@ -674,16 +552,17 @@ cudaError_t launch_tridiag_setup(const Geometry& g, const DevTables& tb, int par
 
 template <typename T, bool FULL>
 static cudaError_t launch_factored(const Geometry& g, const T* a, const T* c, const TriFactors<T>& tf, int parts,
-                                   int low, bool trunc, cplx<T>* spec, cudaStream_t st) {
+                                   int low, bool trunc, cplx<T>* spec, SideArgs sd, cudaStream_t st) {
   int S = 256 / parts;
   if (S < 1) S = 1;
   if (S > 32) S = 32;
-  const size_t smem = (size_t)14 * parts * S * sizeof(T);
+  size_t smem = (size_t)14 * parts * S * sizeof(T);
   const int blocks = (tf.nsys + S - 1) / S;
   auto kern = k_tridiag_factored<T, FULL>;
   cudaError_t e;
+  if ((e = prepare_side<T>(g, sd, parts * S, smem, spec, st)) != cudaSuccess) return e;
   if ((e = prep(kern, smem)) != cudaSuccess) return e;
-  kern<<<blocks, parts * S, smem, st>>>(g, parts, g.ny / parts, S, low, trunc ? 1 : 0, a, c, tf, spec);
+  kern<<<sd.n + blocks, parts * S, smem, st>>>(g, parts, g.ny / parts, S, low, trunc ? 1 : 0, a, c, tf, spec, sd);
   return cudaGetLastError();
 }
 
@@ -701,7 +580,7 @@ cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int par
 }
 
 cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes,
-                                   cplx<float>* spec, cudaStream_t st, int kx_lo, int kx_hi) {
+                                   cplx<float>* spec, SideArgs sd, cudaStream_t st, int kx_lo, int kx_hi) {
   if (!reg_tridiag_ok(g.ny, parts)) return cudaErrorNotSupported;
   const int m = g.ny / parts;
   const int S = reg_systems_per_cta(parts);
@@ -711,14 +590,16 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
   if (!whole && (!scan_tridiag_ok(g.ny, parts) || kx_lo % S)) return cudaErrorNotSupported;
   if (scan_tridiag_ok(g.ny, parts)) {   // warp-scan variant
     const int nt = parts * S;
-    const size_t smem = (size_t)parts * (m * S + 1) * 8 + (size_t)2 * parts * (m | 1) * 4;
+    size_t smem = (size_t)parts * (m * S + 1) * 8 + (size_t)2 * parts * (m | 1) * 4;
     const int blocks = g.nz * ((kx_hi - kx_lo + S - 1) / S);
+    cudaError_t es = prepare_side<float>(g, sd, nt, smem, spec, st);
+    if (es != cudaSuccess) return es;
 #define PP_SCAN_CASE(MM)                                                                                       \
   case MM: {                                                                                                   \
     cudaError_t e = prep(k_tridiag_scan<MM>, smem);                                                            \
     if (e != cudaSuccess) return e;                                                                            \
-    k_tridiag_scan<MM><<<blocks, nt, smem, st>>>(g, parts, S, low_modes, tb.f.a, tb.f.c, tb.lamx, tb.lamz,     \
-                                                 tb.red_f, spec, kx_lo, kx_hi);                                \
+    k_tridiag_scan<MM><<<sd.n + blocks, nt, smem, st>>>(g, parts, S, low_modes, tb.f.a, tb.f.c, tb.lamx,       \
+                                                        tb.lamz, tb.red_f, spec, kx_lo, kx_hi, sd);            \
     return cudaGetLastError();                                                                                 \
   }
     switch (m) {
@@ -730,15 +611,17 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
   }
   const int nt = parts * S;
   const size_t tabf = ((size_t)5 * (parts - 1) * S + 1) & ~(size_t)1;
-  const size_t smem = (size_t)6 * nt * sizeof(float) + tabf * sizeof(float) + (size_t)m * 8 * nt;
+  size_t smem = (size_t)6 * nt * sizeof(float) + tabf * sizeof(float) + (size_t)m * 8 * nt;
   const int nsys = g.nz * g.ncols;
   const int blocks = (nsys + S - 1) / S;
+  const cudaError_t es = prepare_side<float>(g, sd, nt, smem, spec, st);
+  if (es != cudaSuccess) return es;
 #define PP_REG_CASE(MM)                                                                                         \
   case MM: {                                                                                                    \
     cudaError_t e = prep(k_tridiag_reg<MM>, smem);                                                              \
     if (e != cudaSuccess) return e;                                                                             \
-    k_tridiag_reg<MM><<<blocks, nt, smem, st>>>(g, parts, S, low_modes, tb.f.a, tb.f.c, tb.lamx, tb.lamz,       \
-                                                tb.red_f, spec);                                                \
+    k_tridiag_reg<MM><<<sd.n + blocks, nt, smem, st>>>(g, parts, S, low_modes, tb.f.a, tb.f.c, tb.lamx,         \
+                                                       tb.lamz, tb.red_f, spec, sd);                            \
     break;                                                                                                      \
   }
   switch (m) {
@@ -751,26 +634,13 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
 }
 
 cudaError_t launch_tridiag_factored(const Geometry& g, const DevTables& tb, int parts, bool trunc, cplx<double>* spec,
-                                    cudaStream_t st) {
-  return launch_factored<double, true>(g, tb.d.a, tb.d.c, tb.tri_d, parts, -1, trunc, spec, st);
+                                    const SideArgs& sd, cudaStream_t st) {
+  return launch_factored<double, true>(g, tb.d.a, tb.d.c, tb.tri_d, parts, -1, trunc, spec, sd, st);
 }
 
 cudaError_t launch_tridiag_factored_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes, bool trunc,
-                                        cplx<float>* spec, cudaStream_t st) {
-  return launch_factored<float, false>(g, tb.f.a, tb.f.c, tb.tri_f, parts, low_modes, trunc, spec, st);
+                                        cplx<float>* spec, const SideArgs& sd, cudaStream_t st) {
+  return launch_factored<float, false>(g, tb.f.a, tb.f.c, tb.tri_f, parts, low_modes, trunc, spec, sd, st);
 }
-
-template <typename TD>
-cudaError_t launch_mode00(const Geometry& g, const DevTables& tb, GaugeMode gauge, cplx<TD>* spec, cudaStream_t st) {
-  const size_t smem = 2 * (size_t)g.ny * sizeof(double);
-  auto kern = k_mode00<TD>;
-  cudaError_t e;
-  if ((e = prep(kern, smem)) != cudaSuccess) return e;
-  kern<<<1, 32, smem, st>>>(g, tb.dy, tb.h, spec, tb.acc, (int)gauge);
-  return cudaGetLastError();
-}
-template cudaError_t launch_mode00<double>(const Geometry&, const DevTables&, GaugeMode, cplx<double>*,
-                                           cudaStream_t);
-template cudaError_t launch_mode00<float>(const Geometry&, const DevTables&, GaugeMode, cplx<float>*, cudaStream_t);
 
 }  // namespace pp

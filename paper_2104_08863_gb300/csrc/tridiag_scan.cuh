@@ -1,10 +1,11 @@
 // Wall-normal pieces shared by the standalone kernels (k_tridiag.cu) and the persistent batched
 // kernel (batch_persistent.cu): the low-mode test, the reciprocal, 8- and 4-byte asynchronous
-// copies, the warp-scan FP32 PDD tile (Sec. 2.2, Eqs. 10-21, exact reduced system) and the exact
-// solve of the singular (0, 0) mode.
+// copies, the warp-scan FP32 PDD tile (Sec. 2.2, Eqs. 10-21, exact reduced system) and, for the
+// persistent kernel, the exact solve of the singular (0, 0) mode by one warp.
 #pragma once
 
 #include "internal.h"
+#include "low_modes.cuh"
 
 namespace pp {
 
@@ -170,16 +171,15 @@ __device__ __forceinline__ void tridiag_scan_tile(const Geometry& g, int P, int 
     csm[bj * MS + ij] = c[j];
   }
   // a CTA owns the S systems kx0 .. kx0+S-1 of one kz, within the launch's columns
-  // [kx_lo, kx_hi) (kx_lo a multiple of S); columns past the padded row (pitch) are not touched,
-  // columns in [ncols, pitch) are padding and go back unchanged (the last slab copies them)
+  // [kx_lo, kx_hi) (kx_lo a multiple of S); the columns of the modes solved apart (by other CTAs
+  // of the launch) are neither read nor written
   const int ntile = (kx_hi - kx_lo + S - 1) / S;
   const int kz = tile_id / ntile;
   const int kx0 = kx_lo + (tile_id - kz * ntile) * S;
-  const int copy_hi = kx_hi >= g.ncols ? g.pitch : kx_hi;
   const size_t rstride = (size_t)g.nz * g.pitch;
   // ---- coalesced copy-in: thread t copies block t / S of system t % S (S-system row segments)
   const int cpb = threadIdx.x / S, cps = threadIdx.x - cpb * S;
-  const bool cvalid = kx0 + cps < copy_hi;
+  const bool cvalid = kx0 + cps < kx_hi && !(kx0 + cps == 0 && kz == 0) && !is_low(kx0 + cps, kz, g.nz, low);
   const float2* gsrc = reinterpret_cast<const float2*>(spec) + (size_t)kz * g.pitch + kx0 + cps +
                        (size_t)cpb * M * rstride;
   float2* tsrc = tile + cpb * BS + cps;
@@ -214,9 +214,14 @@ template <int M>
 __global__ void __launch_bounds__(256, 2) k_tridiag_scan(Geometry g, int P, int S, int low, const float* __restrict__ a,
                                                          const float* __restrict__ c, const double* __restrict__ lamx,
                                                          const double* __restrict__ lamz, const float* __restrict__ rtab,
-                                                         cplx<float>* __restrict__ spec, int kx_lo, int kx_hi) {
+                                                         cplx<float>* __restrict__ spec, int kx_lo, int kx_hi,
+                                                         SideArgs sd) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  tridiag_scan_tile<M>(g, P, S, low, a, c, lamx, lamz, rtab, spec, kx_lo, kx_hi, blockIdx.x, smem_raw);
+  if ((int)blockIdx.x < sd.n) {
+    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
+    return;
+  }
+  tridiag_scan_tile<M>(g, P, S, low, a, c, lamx, lamz, rtab, spec, kx_lo, kx_hi, blockIdx.x - sd.n, smem_raw);
 }
 
 // The (0, 0) mode: T p = F - mean with sum_j dy_j p_j = 0 (compatibility and gauge), by the
@@ -304,14 +309,6 @@ __device__ __forceinline__ void mode00_warp(const Geometry& g, const double* __r
   if (gauge == GAUGE_OFFSET) mr2 += acc[1] / sw;
   for (int j = lo; j < hi; ++j)
     st_c(spec + (size_t)j * rstride, mk<TD>(TD(fr[j] - mr2), TD(fi[j] - mi2)));
-}
-
-template <typename TD>
-__global__ void __launch_bounds__(32) k_mode00(Geometry g, const double* __restrict__ dy,
-                                               const double* __restrict__ h, cplx<TD>* __restrict__ spec,
-                                               double* __restrict__ acc, int gauge) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  mode00_warp<TD>(g, dy, h, spec, acc, gauge, reinterpret_cast<double*>(smem_raw));
 }
 
 }  // namespace pp
