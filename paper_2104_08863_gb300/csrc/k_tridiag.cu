@@ -448,6 +448,134 @@ __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S
   }
 }
 
+// ---- FP32 PDD with the blocks in registers (P a power of two <= 32) --------------------------
+// A CTA owns S = 256 / P consecutive systems of the flattened (kz, padded kx) index, thread
+// (s, b) = (tid mod S, tid div S) block b of system s: it loads its M rows straight into registers
+// (S-system row segments of 64 bytes or more, every load in flight before the first use), sweeps
+// forward keeping per row rb_i gg_i, rb_i c_i and rb_i gv_i (4 registers), and after the reduced
+// system sweeps back and stores each row as it is final.  Only the block-end values cross shared
+// memory, twice: into system-major order, where the P interfaces of a system are P lanes of a
+// warp and the reduced system is the pair of warp scans of tridiag_scan.cuh, and back.
+//
+// The form that staged the rows in shared memory and swept them there made 14 shared-memory
+// wavefronts per warp and row; it took 278 us per pass at 768x384x512 and 2.73 ms at
+// 1536x768x1024, this one 250 us and 2.58 ms (1.21 and 9.78 GB each).  What is left is the
+// access pattern: 64-byte row segments (S = 8 at P = 32) several MB apart.  The same operations in
+// the same order: bit-identical results.
+template <int M> constexpr int rows_min_ctas() { return M <= 8 ? 4 : (M <= 12 ? 3 : 2); }
+
+template <int M>
+__global__ void __launch_bounds__(256, rows_min_ctas<M>())
+    k_tridiag_rows(Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
+                   const double* __restrict__ lamx, const double* __restrict__ lamz, const float* __restrict__ rtab,
+                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, SideArgs sd) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x < sd.n) {
+    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
+    return;
+  }
+  constexpr int MS = M | 1;   // odd stride of a block's (a, c) pairs
+  const int P = 1 << lgP, S = 256 >> lgP;
+  const int tid = threadIdx.x;
+  const int s = tid & (S - 1), b = tid >> (8 - lgP);
+  float4* ex = reinterpret_cast<float4*>(smem_raw);                   // [s][b], stride P + 1
+  float* rec = reinterpret_cast<float*>(ex + (size_t)S * (P + 1));    // interface records [k][tid]
+  float2* ac = reinterpret_cast<float2*>(rec + 5 * 256);              // [b][i]
+  const int idx0 = ((int)blockIdx.x - sd.n) * S, total = g.nz * width;
+  // mode of system index q of the flattened (kz, kx - kx_lo) order; false for padding, columns
+  // outside the launch and the modes solved apart
+  auto mode = [&](int q, int& kx, int& kz) {
+    kz = q / width;
+    kx = kx_lo + q - kz * width;
+    return q < total && kx < kx_hi && !(kx == 0 && kz == 0) && !is_low(kx, kz, g.nz, low);
+  };
+  int kx, kz;
+  const bool active = mode(idx0 + s, kx, kz);
+  const size_t rstride = (size_t)g.nz * g.pitch;
+  float2* p = reinterpret_cast<float2*>(spec) + (size_t)kz * g.pitch + kx + (size_t)b * M * rstride;
+  float2 v[M];
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < M; ++i) v[i] = __ldcg(p + (size_t)i * rstride);
+  }
+  // interface role: thread (s2, b2) of the system-major order, its record fetched meanwhile
+  const int s2 = tid >> lgP, b2 = tid & (P - 1);
+  bool iface = false;
+  if (P > 1 && b2 < P - 1) {
+    int kx2, kz2;
+    iface = mode(idx0 + s2, kx2, kz2);
+    if (iface) {
+      const float* t = rtab + ((size_t)(kz2 * g.ncols + kx2) * (P - 1) + b2) * 5;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) cp_async4(rec + k * 256 + tid, t + k);
+    }
+  }
+  for (int j = tid; j < g.ny; j += 256) {
+    const int bj = j / M;
+    ac[bj * MS + j - bj * M] = make_float2(a[j], c[j]);
+  }
+  const float sigma = active ? float(-(lamx[kx] + lamz[kz])) : 0.f;
+  __syncthreads();
+  const float2* co = ac + b * MS;
+  float rcv[M], rgv[M];
+  float2 xF = make_float2(0.f, 0.f), xL = make_float2(0.f, 0.f);
+  if (active) {
+    float2 cf = co[0];
+    float e = cf.x + sigma, gv = cf.x, rb = rcp_nr(cf.y + e);
+    float run = 1.f;
+    float2 gg = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      float mult = 0.f;
+      if (i > 0) {
+        cf = co[i];
+        mult = cf.x * rb;
+        e = fmaf(mult, e, sigma);
+        gv = mult * gv;
+        rb = rcp_nr(cf.y + e);
+      }
+      gg = make_float2(fmaf(mult, gg.x, -v[i].x), fmaf(mult, gg.y, -v[i].y));
+      v[i] = make_float2(gg.x * rb, gg.y * rb);
+      const float crb = cf.y * rb;
+      rcv[i] = crb;
+      rgv[i] = gv * rb;
+      const float kap = run * rb;
+      xF.x = fmaf(kap, gg.x, xF.x);
+      xF.y = fmaf(kap, gg.y, xF.y);
+      run *= crb;
+    }
+    xL = v[M - 1];
+  }
+  float2 alpha = make_float2(0.f, 0.f), beta = make_float2(0.f, 0.f);
+  if (P > 1) {
+    ex[s * (P + 1) + b] = make_float4(xF.x, xF.y, xL.x, xL.y);
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    float4* mine = ex + s2 * (P + 1) + b2;
+    const float4 x = *mine;
+    float vL = 0.f, inv = 0.f, X01 = 0.f, X10 = 0.f, tw = 0.f;
+    if (iface) {
+      vL = rec[tid]; inv = rec[256 + tid]; X01 = rec[512 + tid]; X10 = rec[768 + tid]; tw = rec[1024 + tid];
+    }
+    float2 al, be;
+    scan_interfaces(P, b2, make_float2(x.x, x.y), make_float2(x.z, x.w), vL, inv, X01, X10, tw, al, be);
+    *mine = make_float4(al.x, al.y, be.x, be.y);
+    __syncthreads();
+    const float4 y = ex[s * (P + 1) + b];
+    alpha = make_float2(y.x, y.y);
+    beta = make_float2(y.z, y.w);
+  }
+  if (active) {
+    float2 xn = beta;
+#pragma unroll
+    for (int i = M - 1; i >= 0; --i) {
+      xn = make_float2(fmaf(rcv[i], xn.x, fmaf(rgv[i], alpha.x, v[i].x)),
+                       fmaf(rcv[i], xn.y, fmaf(rgv[i], alpha.y, v[i].y)));
+      p[(size_t)i * rstride] = xn;
+    }
+  }
+}
+
 // Pivots of the modes solved apart, one thread per system of the list (low_system's order):
 // rb[sys ny + j] = 1 / beta_j by the margin recurrence, in FP64.
 __global__ void __launch_bounds__(32) k_low_setup(Geometry g, int n, int low, const double* __restrict__ a,
@@ -588,26 +716,29 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
   const bool whole = kx_lo == 0 && kx_hi == g.ncols;
   if (kx_lo < 0 || kx_hi > g.ncols || kx_hi <= kx_lo) return cudaErrorInvalidValue;
   if (!whole && (!scan_tridiag_ok(g.ny, parts) || kx_lo % S)) return cudaErrorNotSupported;
-  if (scan_tridiag_ok(g.ny, parts)) {   // warp-scan variant
-    const int nt = parts * S;
-    size_t smem = (size_t)parts * (m * S + 1) * 8 + (size_t)2 * parts * (m | 1) * 4;
-    const int blocks = g.nz * ((kx_hi - kx_lo + S - 1) / S);
-    cudaError_t es = prepare_side<float>(g, sd, nt, smem, spec, st);
+  if (scan_tridiag_ok(g.ny, parts)) {   // P a power of two <= 32: the blocks in registers
+    int lgP = 0;
+    while ((1 << lgP) < parts) ++lgP;
+    // the launch's columns; a whole row with its padding keeps every CTA's segments 64-byte aligned
+    const int width = (kx_hi == g.ncols ? g.pitch : kx_hi) - kx_lo;
+    const int blocks = (g.nz * width + S - 1) / S;
+    size_t smem = (size_t)S * (parts + 1) * 16 + 5 * 256 * 4 + (size_t)parts * (m | 1) * 8;
+    const cudaError_t es = prepare_side<float>(g, sd, 256, smem, spec, st);
     if (es != cudaSuccess) return es;
-#define PP_SCAN_CASE(MM)                                                                                       \
+#define PP_ROWS_CASE(MM)                                                                                       \
   case MM: {                                                                                                   \
-    cudaError_t e = prep(k_tridiag_scan<MM>, smem);                                                            \
+    cudaError_t e = prep(k_tridiag_rows<MM>, smem);                                                            \
     if (e != cudaSuccess) return e;                                                                            \
-    k_tridiag_scan<MM><<<sd.n + blocks, nt, smem, st>>>(g, parts, S, low_modes, tb.f.a, tb.f.c, tb.lamx,       \
-                                                        tb.lamz, tb.red_f, spec, kx_lo, kx_hi, sd);            \
+    k_tridiag_rows<MM><<<sd.n + blocks, 256, smem, st>>>(g, lgP, low_modes, tb.f.a, tb.f.c, tb.lamx, tb.lamz,  \
+                                                         tb.red_f, spec, kx_lo, kx_hi, width, sd);             \
     return cudaGetLastError();                                                                                 \
   }
     switch (m) {
-      PP_SCAN_CASE(1) PP_SCAN_CASE(2) PP_SCAN_CASE(3) PP_SCAN_CASE(4) PP_SCAN_CASE(6) PP_SCAN_CASE(8)
-      PP_SCAN_CASE(12) PP_SCAN_CASE(16) PP_SCAN_CASE(24)
+      PP_ROWS_CASE(1) PP_ROWS_CASE(2) PP_ROWS_CASE(3) PP_ROWS_CASE(4) PP_ROWS_CASE(6) PP_ROWS_CASE(8)
+      PP_ROWS_CASE(12) PP_ROWS_CASE(16) PP_ROWS_CASE(24)
       default: break;
     }
-#undef PP_SCAN_CASE
+#undef PP_ROWS_CASE
   }
   const int nt = parts * S;
   const size_t tabf = ((size_t)5 * (parts - 1) * S + 1) & ~(size_t)1;

@@ -5,7 +5,6 @@
 #pragma once
 
 #include "internal.h"
-#include "low_modes.cuh"
 
 namespace pp {
 
@@ -73,6 +72,33 @@ __device__ __forceinline__ float2 shfl_down2(float2 v, int d) {
   return make_float2(__shfl_down_sync(0xffffffffu, v.x, d), __shfl_down_sync(0xffffffffu, v.y, d));
 }
 
+// The reduced system of one system on the P consecutive lanes of its blocks: lane b with its
+// block's end values xF, xL of x~ and the record (vL, inv, X01, X10, tw) of interface b (zeros in
+// the last lane) gets its neighbour values alpha = z0_{b-1}, beta = z1_b.  Every lane takes part.
+__device__ __forceinline__ void scan_interfaces(int P, int b, float2 xF, float2 xL, float vL, float inv, float X01,
+                                                float X10, float tw, float2& alpha, float2& beta) {
+  alpha = beta = make_float2(0.f, 0.f);
+  const float2 xFn = shfl_down2(xF, 1);                 // xF_{i+1}
+  float A = inv * vL;
+  float2 B = make_float2(fmaf(inv, xL.x, X01 * xFn.x), fmaf(inv, xL.y, X01 * xFn.y));
+  scan_up(P, b, A, B);                                  // B = y0_i
+  const float2 y0 = B;
+  float2 y0m = shfl_up2(y0, 1);                         // y0_{i-1}
+  if (b == 0) y0m = make_float2(0.f, 0.f);
+  const float2 q0 = make_float2(fmaf(vL, y0m.x, xL.x), fmaf(vL, y0m.y, xL.y));
+  float G = tw * inv;
+  float2 Y = make_float2(fmaf(X10, q0.x, inv * xFn.x), fmaf(X10, q0.y, inv * xFn.y));
+  if (b == P - 1) { G = 0.f; Y = make_float2(0.f, 0.f); }
+  scan_down(P, b, G, Y);                                // Y = z1_i
+  const float2 z1 = Y;
+  const float2 z1n = shfl_down2(z1, 1);                 // z1_{i+1}
+  const float a0 = tw * X01;
+  const float2 z0 = make_float2(fmaf(a0, z1n.x, y0.x), fmaf(a0, z1n.y, y0.y));
+  const float2 z0m = shfl_up2(z0, 1);                   // z0_{b-1}
+  if (b > 0) alpha = z0m;
+  if (b < P - 1) beta = z1;
+}
+
 // The sweeps of one system's block and the reduced interface system, on a staged tile: thread
 // (s, b) with `blk` its block's first row (row i at blk[i * S], updated in place), `ab`, `cb` the
 // block's a and c (a_{bM+i} at ab[i]); `active` false for the (0, 0) mode, the FP64 low modes
@@ -82,7 +108,6 @@ template <int M>
 __device__ __forceinline__ void scan_sweeps(int P, int S, float2* blk, const float* ab, const float* cb, int b,
                                             bool active, float sigma, float vL, float inv, float X01, float X10,
                                             float tw) {
-  const int lseg = b;
   // The backward sweep x_i = rb_i (gg_i + alpha gv_i + c_i x_{i+1}) takes its three products with
   // the pivot reciprocal rb_i from the forward sweep: rb_i gg_i in the tile (in place of gg_i),
   // rb_i c_i and rb_i gv_i in registers, so that it loads no coefficient from shared memory (whose
@@ -117,28 +142,7 @@ __device__ __forceinline__ void scan_sweeps(int P, int S, float2* blk, const flo
     xL = make_float2(gg.x * rb, gg.y * rb);
   }
   float2 alpha = make_float2(0.f, 0.f), beta = make_float2(0.f, 0.f);
-  if (P > 1) {
-    // interface i = b (lanes b <= P-2); every lane takes part in the shuffles
-    const float2 xFn = shfl_down2(xF, 1);                 // xF_{i+1}
-    float A = inv * vL;
-    float2 B = make_float2(fmaf(inv, xL.x, X01 * xFn.x), fmaf(inv, xL.y, X01 * xFn.y));
-    scan_up(P, lseg, A, B);                               // B = y0_i
-    const float2 y0 = B;
-    float2 y0m = shfl_up2(y0, 1);                         // y0_{i-1}
-    if (lseg == 0) y0m = make_float2(0.f, 0.f);
-    const float2 q0 = make_float2(fmaf(vL, y0m.x, xL.x), fmaf(vL, y0m.y, xL.y));
-    float G = tw * inv;
-    float2 Y = make_float2(fmaf(X10, q0.x, inv * xFn.x), fmaf(X10, q0.y, inv * xFn.y));
-    if (lseg == P - 1) { G = 0.f; Y = make_float2(0.f, 0.f); }
-    scan_down(P, lseg, G, Y);                             // Y = z1_i
-    const float2 z1 = Y;
-    const float2 z1n = shfl_down2(z1, 1);                 // z1_{i+1}
-    const float a0 = tw * X01;
-    const float2 z0 = make_float2(fmaf(a0, z1n.x, y0.x), fmaf(a0, z1n.y, y0.y));
-    const float2 z0m = shfl_up2(z0, 1);                   // z0_{b-1}
-    if (lseg > 0) alpha = z0m;
-    if (lseg < P - 1) beta = z1;
-  }
+  if (P > 1) scan_interfaces(P, b, xF, xL, vL, inv, X01, X10, tw, alpha, beta);
   if (active) {
     float2 xn = beta;
 #pragma unroll
@@ -208,20 +212,6 @@ __device__ __forceinline__ void tridiag_scan_tile(const Geometry& g, int P, int 
 #pragma unroll
     for (int i = 0; i < M; ++i) gdst[(size_t)i * rstride] = tsrc[i * S];
   }
-}
-
-template <int M>
-__global__ void __launch_bounds__(256, 2) k_tridiag_scan(Geometry g, int P, int S, int low, const float* __restrict__ a,
-                                                         const float* __restrict__ c, const double* __restrict__ lamx,
-                                                         const double* __restrict__ lamz, const float* __restrict__ rtab,
-                                                         cplx<float>* __restrict__ spec, int kx_lo, int kx_hi,
-                                                         SideArgs sd) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if ((int)blockIdx.x < sd.n) {
-    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
-    return;
-  }
-  tridiag_scan_tile<M>(g, P, S, low, a, c, lamx, lamz, rtab, spec, kx_lo, kx_hi, blockIdx.x - sd.n, smem_raw);
 }
 
 // The (0, 0) mode: T p = F - mean with sum_j dy_j p_j = 0 (compatibility and gauge), by the
