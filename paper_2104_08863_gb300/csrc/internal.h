@@ -62,6 +62,7 @@ struct SideArgs {
 struct Geometry {
   int nx, ny, nz, M, ncols, pitch;
   double dx, dz;
+  double inv_dx, inv_dz;   // from the host: an FP64 division costs a thread more than its loads
   int generic_fft;   // 1: use the runtime-generic FFT kernels (POISSON_GENERIC_FFT)
   int selftest_wait; // 1: the bulk-copy-staged x-transform skips its first copy (POISSON_SELFTEST_WAIT)
 };

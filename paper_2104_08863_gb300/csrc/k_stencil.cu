@@ -9,87 +9,167 @@
 //  k_check_finite : sets the device status word when a value is NaN or Inf.
 //  k_divergence : f = D(u)/dt of Eq. 7 on the cell centres (the right-hand side of the
 //                pressure equation), for callers that want it as a field.
+#include <string.h>
+
 #include "fpconv.cuh"
 #include "internal.h"
 
 namespace pp {
 
-// Lines [lbeg, lend) of the (ny + 1) nz face lines (line = j nz + k).
-template <typename T>
-__global__ void __launch_bounds__(256) k_gradient(Geometry g, const T* __restrict__ p, T* __restrict__ u,
-                                                  T* __restrict__ v, T* __restrict__ w,
-                                                  const T* __restrict__ inv_h, T dt, int lbeg, int lend) {
+// The passes below stream whole fields with a few operations per value, so HBM bounds them (FP64
+// gradient: its six FP64 instructions per point, too).  A thread takes V consecutive x values of
+// one line as one 16-byte access per field (V = 4 FP32, 2 FP64; nx not a multiple of V: V = 2,
+// nx is even), with every access of the line in flight before the first use; a CTA covers
+// STENCIL_THREADS / tx lines of tx vectors, and what depends on the grid only comes from the host
+// (two FP64 divisions per thread took 50 us of these).  FP32 gradient and adjoint epilogue of
+// 256x192x256 (352 MB each): 59 and 58 us (6.0 TB/s), with one scalar per thread and line in
+// flight 102 and 100; FP64 gradient of 512x384x512 (5.6 GB): 1.23 ms, before 1.37.
+template <typename T, int V> struct Vec { T x[V]; };
+template <typename T, int V>
+__device__ __forceinline__ Vec<T, V> vload(const T* p) {
+  Vec<T, V> r;
+  if constexpr (sizeof(T) * V == 16) {
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    memcpy(&r, &q, 16);
+  } else {
+    const uint2 q = *reinterpret_cast<const uint2*>(p);
+    memcpy(&r, &q, 8);
+  }
+  return r;
+}
+template <typename T, int V>
+__device__ __forceinline__ void vstore(T* p, const Vec<T, V>& r) {
+  if constexpr (sizeof(T) * V == 16) {
+    uint4 q;
+    memcpy(&q, &r, 16);
+    *reinterpret_cast<uint4*>(p) = q;
+  } else {
+    uint2 q;
+    memcpy(&q, &r, 8);
+    *reinterpret_cast<uint2*>(p) = q;
+  }
+}
+
+constexpr int STENCIL_THREADS = 256;
+
+// The pressure at V cells, their x - 1, z - 1 and y - 1 neighbours.
+template <typename T, int V> struct PNeigh { Vec<T, V> c, xm, zm, ym; };
+template <typename T, int V>
+__device__ __forceinline__ PNeigh<T, V> pload(const Geometry& g, const T* __restrict__ p, int j, int k, size_t idx,
+                                              int i0, bool cell, bool ym) {
+  PNeigh<T, V> n;
   const size_t plane = (size_t)g.nz * g.nx;
-  const T cx = T(dt / g.dx), cz = T(dt / g.dz);
-  for (int line = lbeg + blockIdx.x; line < lend; line += gridDim.x)
-  for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-    const int j = line / g.nz, k = line - j * g.nz;
-    const size_t idx = (size_t)line * g.nx + i;
-    if (j < g.ny) {
-      const T pc = p[idx];
-      const T pxm = p[idx - i + (i == 0 ? g.nx - 1 : i - 1)];
-      const T pzm = p[(size_t)j * plane + (size_t)(k == 0 ? g.nz - 1 : k - 1) * g.nx + i];
-      u[idx] -= cx * (pc - pxm);
-      w[idx] -= cz * (pc - pzm);
+  T left = T(0);
+  if (cell) {
+    n.c = vload<T, V>(p + idx);
+    left = p[idx + (i0 == 0 ? g.nx - 1 : -1)];
+    n.zm = vload<T, V>(p + idx + (k == 0 ? plane - g.nx : -(size_t)g.nx));
+  }
+  if (ym) n.ym = vload<T, V>(p + idx - plane);
+#pragma unroll
+  for (int q = 0; q < V; ++q) n.xm.x[q] = q ? n.c.x[q - 1] : left;
+  return n;
+}
+
+// Lines [lbeg, lend) of the ny nz cell lines (line = j nz + k).
+template <typename T, int V>
+__global__ void __launch_bounds__(STENCIL_THREADS) k_gradient(Geometry g, const T* __restrict__ p, T* __restrict__ u,
+                                                              T* __restrict__ v, T* __restrict__ w,
+                                                              const T* __restrict__ inv_h, T dt, T cx, T cz, int lbeg,
+                                                              int lend) {
+  const int line = lbeg + blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= lend) return;
+  const int j = line / g.nz, k = line - j * g.nz;
+  const bool inner = j >= 1;   // v's wall faces are boundary values
+  const T cy = inner ? dt * inv_h[j] : T(0);
+  for (int i0 = threadIdx.x * V; i0 < g.nx; i0 += blockDim.x * V) {
+    const size_t idx = (size_t)line * g.nx + i0;
+    const PNeigh<T, V> n = pload<T, V>(g, p, j, k, idx, i0, true, inner);
+    Vec<T, V> uu = vload<T, V>(u + idx), ww = vload<T, V>(w + idx), vv;
+    if (inner) vv = vload<T, V>(v + idx);
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      uu.x[q] -= cx * (n.c.x[q] - n.xm.x[q]);
+      ww.x[q] -= cz * (n.c.x[q] - n.zm.x[q]);
     }
-    if (j >= 1 && j <= g.ny - 1) {
-      const T cy = dt * inv_h[j];
-      v[idx] -= cy * (p[idx] - p[idx - plane]);
+    vstore<T, V>(u + idx, uu);
+    vstore<T, V>(w + idx, ww);
+    if (inner) {
+#pragma unroll
+      for (int q = 0; q < V; ++q) vv.x[q] -= cy * (n.c.x[q] - n.ym.x[q]);
+      vstore<T, V>(v + idx, vv);
     }
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_adj_epi(Geometry g, const T* __restrict__ pp_, T* __restrict__ gu,
-                                                 T* __restrict__ gv, T* __restrict__ gw,
-                                                 const double* __restrict__ dy) {
-  const size_t plane = (size_t)g.nz * g.nx;
-  const int nlines = (g.ny + 1) * g.nz;
-  const T ix = T(1.0 / g.dx), iz = T(1.0 / g.dz);
-  for (int line = blockIdx.x; line < nlines; line += gridDim.x)
-  for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-    const int j = line / g.nz, k = line - j * g.nz;
-    const size_t idx = (size_t)line * g.nx + i;
-    if (j < g.ny) {
-      const T dyj = T(dy[j]);
-      const T pc = pp_[idx];
-      const T pxm = pp_[idx - i + (i == 0 ? g.nx - 1 : i - 1)];
-      const T pzm = pp_[(size_t)j * plane + (size_t)(k == 0 ? g.nz - 1 : k - 1) * g.nx + i];
-      gu[idx] -= dyj * (pxm - pc) * ix;
-      gw[idx] -= dyj * (pzm - pc) * iz;
+template <typename T, int V>
+__global__ void __launch_bounds__(STENCIL_THREADS) k_adj_epi(Geometry g, const T* __restrict__ pp_, T* __restrict__ gu,
+                                                             T* __restrict__ gv, T* __restrict__ gw,
+                                                             const double* __restrict__ dy, T ix, T iz) {
+  const int line = blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= (g.ny + 1) * g.nz) return;
+  const int j = line / g.nz, k = line - j * g.nz;
+  const bool cell = j < g.ny, below = j >= 1;
+  const T dyj = cell ? T(dy[j]) : T(0);
+  for (int i0 = threadIdx.x * V; i0 < g.nx; i0 += blockDim.x * V) {
+    const size_t idx = (size_t)line * g.nx + i0;
+    const PNeigh<T, V> n = pload<T, V>(g, pp_, j, k, idx, i0, cell, below);
+    Vec<T, V> vv = vload<T, V>(gv + idx), uu, ww;
+    if (cell) {
+      uu = vload<T, V>(gu + idx);
+      ww = vload<T, V>(gw + idx);
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        uu.x[q] -= dyj * (n.xm.x[q] - n.c.x[q]) * ix;
+        ww.x[q] -= dyj * (n.zm.x[q] - n.c.x[q]) * iz;
+      }
+      vstore<T, V>(gu + idx, uu);
+      vstore<T, V>(gw + idx, ww);
     }
     // (D_y^T q)_f = q_{f-1}/dy_{f-1} - q_f/dy_f = p'_{f-1} - p'_f  (terms outside 0..ny-1 vanish)
-    T t = T(0);
-    if (j >= 1) t += pp_[idx - plane];
-    if (j <= g.ny - 1) t -= pp_[idx];
-    gv[idx] -= t;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+      T t = T(0);
+      if (below) t += n.ym.x[q];
+      if (cell) t -= n.c.x[q];
+      vv.x[q] -= t;
+    }
+    vstore<T, V>(gv + idx, vv);
   }
 }
 
 // out[j][k][i] = in[j][k][i] * s_j with s_j = 1/dy_j (to_weighted = false) or dy_j (true): the
-// diagonal volume weights W^-1 and W of the transposed solve (L_h^T = W L_h W^-1).
-template <typename T>
-__global__ void __launch_bounds__(256) k_scale_planes(Geometry g, const T* __restrict__ in, T* __restrict__ out,
-                                                      const double* __restrict__ dy, int to_weighted) {
-  const int nlines = g.ny * g.nz;
-  for (int line = blockIdx.x; line < nlines; line += gridDim.x) {
-    const int j = line / g.nz;
-    const T sj = to_weighted ? T(dy[j]) : T(1.0 / dy[j]);
-    const size_t base = (size_t)line * g.nx;
-    for (int i = threadIdx.x; i < g.nx; i += blockDim.x) out[base + i] = in[base + i] * sj;
+// diagonal volume weights W^-1 and W of the transposed solve (L_h^T = W L_h W^-1).  1/dy_j comes
+// from the plan's table: a division per thread cost more FP64 time than the pass's traffic.
+template <typename T, int V>
+__global__ void __launch_bounds__(STENCIL_THREADS) k_scale_planes(Geometry g, const T* __restrict__ in,
+                                                                  T* __restrict__ out, const double* __restrict__ sc) {
+  const int line = blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= g.ny * g.nz) return;
+  const T sj = T(sc[line / g.nz]);
+  const size_t base = (size_t)line * g.nx;
+  for (int i0 = threadIdx.x * V; i0 < g.nx; i0 += blockDim.x * V) {
+    Vec<T, V> x = vload<T, V>(in + base + i0);
+#pragma unroll
+    for (int q = 0; q < V; ++q) x.x[q] *= sj;
+    vstore<T, V>(out + base + i0, x);
   }
 }
 
 // q[j][k][i] = dy_j (hi + lo): the FP64 value of the refined solve's FP32 pair, weighted.
-__global__ void __launch_bounds__(256) k_weighted_pair(Geometry g, const float* __restrict__ hi,
-                                                       const float* __restrict__ lo, double* __restrict__ q,
-                                                       const double* __restrict__ dy) {
-  const int nlines = g.ny * g.nz;
-  for (int line = blockIdx.x; line < nlines; line += gridDim.x) {
-    const double w = dy[line / g.nz];
-    const size_t base = (size_t)line * g.nx;
-    for (int i = threadIdx.x; i < g.nx; i += blockDim.x)
-      q[base + i] = w * f32_add_to_f64(hi[base + i], lo ? lo[base + i] : 0.0f);
+__global__ void __launch_bounds__(STENCIL_THREADS) k_weighted_pair(Geometry g, const float* __restrict__ hi,
+                                                                   const float* __restrict__ lo,
+                                                                   double* __restrict__ q,
+                                                                   const double* __restrict__ dy) {
+  const int line = blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= g.ny * g.nz) return;
+  const double w = dy[line / g.nz];
+  const size_t base = (size_t)line * g.nx;
+  for (int i0 = threadIdx.x * 2; i0 < g.nx; i0 += blockDim.x * 2) {
+    const float2 h = *reinterpret_cast<const float2*>(hi + base + i0);
+    const float2 l = *reinterpret_cast<const float2*>(lo + base + i0);
+    *reinterpret_cast<double2*>(q + base + i0) =
+        make_double2(w * f32_add_to_f64(h.x, l.x), w * f32_add_to_f64(h.y, l.y));
   }
 }
 
@@ -107,7 +187,7 @@ __global__ void __launch_bounds__(256) k_divergence(Geometry g, const T* __restr
                                                     const T* __restrict__ inv_dy, T inv_dt) {
   const size_t plane = (size_t)g.nz * g.nx;
   const int nlines = g.ny * g.nz;
-  const T ix = T(1.0 / g.dx), iz = T(1.0 / g.dz);
+  const T ix = T(g.inv_dx), iz = T(g.inv_dz);
   for (int line = blockIdx.x; line < nlines; line += gridDim.x) {
     const int j = line / g.nz, k = line - j * g.nz;
     const T iy = inv_dy[j];
@@ -142,37 +222,61 @@ template <typename T> static const T* inv_h_table(const DevTables& tb);
 template <> const double* inv_h_table<double>(const DevTables& tb) { return tb.d.inv_h; }
 template <> const float* inv_h_table<float>(const DevTables& tb) { return tb.f.inv_h; }
 
+// CTAs of tx vectors of V values by STENCIL_THREADS / tx lines, covering nlines lines.
+struct LineTiles { dim3 grid, block; };
+static LineTiles line_tiles(const Geometry& g, int V, int nlines) {
+  int tx = (g.nx + V - 1) / V;
+  tx = tx < STENCIL_THREADS ? tx : STENCIL_THREADS;
+  const int ty = STENCIL_THREADS / tx;
+  return LineTiles{dim3((nlines + ty - 1) / ty), dim3(tx, ty)};
+}
+template <typename T> static bool wide_vectors(const Geometry& g) { return g.nx % (16 / (int)sizeof(T)) == 0; }
+
 template <typename T>
 cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, T* u, T* v, T* w, double dt,
                             cudaStream_t st, int jlo, int jhi) {
   if (jhi < 0) jhi = g.ny;
   if (jlo < 0 || jhi > g.ny || jhi <= jlo) return cudaErrorInvalidValue;
-  const int lbeg = jlo * g.nz, lend = (jhi == g.ny ? g.ny + 1 : jhi) * g.nz;
-  const int cap = line_grid(g);
-  k_gradient<T><<<lend - lbeg < cap ? lend - lbeg : cap, line_block(g), 0, st>>>(g, p, u, v, w, inv_h_table<T>(tb),
-                                                                                  T(dt), lbeg, lend);
+  const int lbeg = jlo * g.nz, lend = jhi * g.nz;
+  constexpr int VW = 16 / (int)sizeof(T);
+  const int V = wide_vectors<T>(g) ? VW : 2;
+  const LineTiles t = line_tiles(g, V, lend - lbeg);
+  // dt/dx and dt/dz once on the host: two FP64 divisions per thread took as long as its traffic
+  const T d = T(dt), cx = T(d / g.dx), cz = T(d / g.dz);
+  const T* ih = inv_h_table<T>(tb);
+  if (V == VW) k_gradient<T, VW><<<t.grid, t.block, 0, st>>>(g, p, u, v, w, ih, d, cx, cz, lbeg, lend);
+  else k_gradient<T, 2><<<t.grid, t.block, 0, st>>>(g, p, u, v, w, ih, d, cx, cz, lbeg, lend);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_adjoint_epilogue(const Geometry& g, const DevTables& tb, const T* q, T* gu, T* gv, T* gw,
                                     cudaStream_t st) {
-  k_adj_epi<T><<<line_grid(g), line_block(g), 0, st>>>(g, q, gu, gv, gw, tb.dy);
+  constexpr int VW = 16 / (int)sizeof(T);
+  const int V = wide_vectors<T>(g) ? VW : 2;
+  const LineTiles t = line_tiles(g, V, (g.ny + 1) * g.nz);
+  const T ix = T(g.inv_dx), iz = T(g.inv_dz);
+  if (V == VW) k_adj_epi<T, VW><<<t.grid, t.block, 0, st>>>(g, q, gu, gv, gw, tb.dy, ix, iz);
+  else k_adj_epi<T, 2><<<t.grid, t.block, 0, st>>>(g, q, gu, gv, gw, tb.dy, ix, iz);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_scale_planes(const Geometry& g, const DevTables& tb, const T* in, T* out, bool to_weighted,
                                 cudaStream_t st) {
-  const int nlines = g.ny * g.nz, cap = 152 * 16;
-  k_scale_planes<T><<<nlines < cap ? nlines : cap, line_block(g), 0, st>>>(g, in, out, tb.dy, to_weighted ? 1 : 0);
+  constexpr int VW = 16 / (int)sizeof(T);
+  const int V = wide_vectors<T>(g) ? VW : 2;
+  const LineTiles t = line_tiles(g, V, g.ny * g.nz);
+  const double* sc = to_weighted ? tb.dy : tb.d.inv_dy;
+  if (V == VW) k_scale_planes<T, VW><<<t.grid, t.block, 0, st>>>(g, in, out, sc);
+  else k_scale_planes<T, 2><<<t.grid, t.block, 0, st>>>(g, in, out, sc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_weighted_pair(const Geometry& g, const DevTables& tb, const float* hi, const float* lo, double* q,
                                  cudaStream_t st) {
-  const int nlines = g.ny * g.nz, cap = 152 * 16;
-  k_weighted_pair<<<nlines < cap ? nlines : cap, line_block(g), 0, st>>>(g, hi, lo, q, tb.dy);
+  const LineTiles t = line_tiles(g, 2, g.ny * g.nz);
+  k_weighted_pair<<<t.grid, t.block, 0, st>>>(g, hi, lo, q, tb.dy);
   return cudaGetLastError();
 }
 

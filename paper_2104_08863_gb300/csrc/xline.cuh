@@ -160,13 +160,13 @@ __device__ __forceinline__ cplx<T> fwd_load(const Geometry& g, const FwdArgs& ar
     TI f0, f1;
     const TI s = TI(args.in_scale);
     divergence_pair<TI>(g, reinterpret_cast<const TI*>(args.u), reinterpret_cast<const TI*>(args.v),
-                        reinterpret_cast<const TI*>(args.w), j, k, i0, TI(1.0 / g.dx), TI(tt.inv_dy[j]),
-                        TI(1.0 / g.dz), f0, f1);
+                        reinterpret_cast<const TI*>(args.w), j, k, i0, TI(g.inv_dx), TI(tt.inv_dy[j]),
+                        TI(g.inv_dz), f0, f1);
     return mk<T>(T(f0 * s), T(f1 * s));
   } else if constexpr (MODE == FWD_GRADT) {
     TI f0, f1;
     gradT_pair<TI>(g, reinterpret_cast<const TI*>(args.u), reinterpret_cast<const TI*>(args.v),
-                   reinterpret_cast<const TI*>(args.w), j, k, i0, TI(1.0 / g.dx), TI(1.0 / g.dz),
+                   reinterpret_cast<const TI*>(args.w), j, k, i0, TI(g.inv_dx), TI(g.inv_dz),
                    TI(tt.inv_h[j]), TI(tt.inv_h[j + 1]), TI(tt.inv_dy[j]), f0, f1);
     return mk<T>(T(f0), T(f1));
   } else {  // FWD_RESID: FP64 rhs (or a stored residual), FP32 pressure field, double-float arithmetic
