@@ -107,6 +107,10 @@ DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base) {
   dt.f.inv_h = (const float*)(tb + to[17]);
   dt.f.a_lo = (const float*)(tb + to[18]);
   dt.f.c_lo = (const float*)(tb + to[19]);
+  dt.d.lf_m = (const cplx<double>*)(tb + to[20]);
+  dt.d.lf_post = (const cplx<double>*)(tb + to[21]);
+  dt.d.lf_z = (const cplx<double>*)(tb + to[22]);
+  dt.f.lf_m = dt.f.lf_post = dt.f.lf_z = nullptr;
   dt.d.a_lo = nullptr;
   dt.d.c_lo = nullptr;
   dt.red_f = pl->has_tri ? nullptr : (const float*)(base + pl->off_red);
@@ -252,12 +256,28 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   slot(14, 8 * (size_t)ny);   slot(15, 8 * (size_t)(ny + 1));
   slot(16, 4 * (size_t)ny);   slot(17, 4 * (size_t)(ny + 1));
   slot(18, 4 * (size_t)ny);   slot(19, 4 * (size_t)ny);
+  const bool lf = spec_is_fp64(pl);   // (cos, tan) tables of the FP64 transforms
+  slot(20, lf ? 16 * (size_t)g.M : 0); slot(21, lf ? 16 * (size_t)(g.M / 2 + 1) : 0); slot(22, lf ? 16 * (size_t)g.nz : 0);
   const size_t tab_bytes = off;
   pl->host_tables.assign(tab_bytes, 0);
   auto& img = pl->host_tables;
   put_cplx_table<double>(img, to[0], twm_r, twm_i);
   put_cplx_table<double>(img, to[1], twp_r, twp_i);
   put_cplx_table<double>(img, to[2], twz_r, twz_i);
+  if (lf) {
+    auto cos_tan = [&](int id, int L, int n) {
+      std::vector<double> c(n), t(n);
+      for (int q = 0; q < n; ++q) {
+        const double ang = 2.0 * M_PI * (double)q / (double)L;
+        c[q] = cos(ang);   // never 0: pi/2 is not a double
+        t[q] = sin(ang) / c[q];
+      }
+      put_cplx_table<double>(img, to[id], c, t);
+    };
+    cos_tan(20, g.M, g.M);
+    cos_tan(21, g.nx, g.M / 2 + 1);
+    cos_tan(22, g.nz, g.nz);
+  }
   put_real_table<double>(img, to[3], pl->a);
   put_real_table<double>(img, to[4], pl->c);
   put_cplx_table<float>(img, to[5], twm_r, twm_i);

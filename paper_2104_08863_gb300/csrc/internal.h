@@ -15,6 +15,10 @@ template <typename T> struct Tables {
   const cplx<T>* tw_m;     // e^{-2 pi i t / M}, t < M   (half-length complex FFT in x)
   const cplx<T>* tw_post;  // e^{-2 pi i k / Nx}, k <= M (real-to-complex packing)
   const cplx<T>* tw_z;     // e^{-2 pi i t / Nz}, t < Nz
+  // FP64 only (fft_lf.cuh): (cos, tan) of 2 pi t / M (t < M), 2 pi k / Nx (k <= M/2), 2 pi t / Nz
+  const cplx<T>* lf_m;
+  const cplx<T>* lf_post;
+  const cplx<T>* lf_z;
   const T* a;              // wall-normal sub-diagonal a_j  (0 for j = 0)
   const T* c;              // wall-normal super-diagonal c_j (0 for j = ny-1)
   const T* inv_dy;         // 1 / dy_j
@@ -87,7 +91,7 @@ struct FwdArgs {
   const void* v;
   const void* w;
   const void* p;         // FWD_RESID: the FP32 pressure field the residual is formed of
-  double in_scale;       // FWD_DIV: 1/dt; FWD_PLAIN: 1 (ignored for FP64 input to FP32)
+  double in_scale;       // factor of the right-hand side: 1/dt for FWD_DIV, else 1 (ignored for FP64 input to FP32)
   float idx2h, idx2l;    // FWD_RESID: 1/dx^2 and 1/dz^2 as double-floats
   float idz2h, idz2l;
   // FWD_RESID, later corrections: r = rin - L_h p with rin a stored residual (one FP32 pair per

@@ -13,6 +13,7 @@
 #include <utility>
 
 #include "bulk_copy.cuh"
+#include "fft_lf.cuh"
 #include "fft_static.cuh"
 #include "k_fft_x_reg.cuh"
 #include "xline.cuh"
@@ -38,24 +39,7 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
   const int line0 = blockIdx.x * LPB;
-  if constexpr (MODE == FWD_RESID && sizeof(T) == 4) {
-    // refinement residual: per-line setup, then pairs of cells
-    float mh, ml;
-    f64_split(tb.acc[0], mh, ml);
-    for (int t = 0; t < LPB; ++t) {
-      const int line = line0 + t;
-      if (line < nlines) {
-        const ResidLine R = resid_line(g, args, tt, tb, line, mh, ml);
-#pragma unroll
-        for (int n = threadIdx.x; n < M; n += THREADS) {
-          const float2 r = R.rin ? resid_pair_line2<true>(R, n) : resid_pair_line2<false>(R, n);
-          buf[padi<T>(t * M + n)] = mk<T>(r.x, r.y);
-        }
-      } else {
-        for (int n = threadIdx.x; n < M; n += THREADS) buf[padi<T>(t * M + n)] = mk<T>(T(0), T(0));
-      }
-    }
-  } else {
+  {
     // all of a thread's loads are issued before any shared-memory store
     constexpr int PER = (LPB * M + THREADS - 1) / THREADS;
     cplx<T> v[PER];
@@ -73,6 +57,31 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
     }
   }
   __syncthreads();
+  if constexpr (sizeof(T) == 8) {
+    // FP64: fused twiddles, two bins per item (the input carries the split's factor 1/2)
+    fft_lf<T, M, -1, LPB, THREADS, 1, M, false>(buf, tt.lf_m);
+    constexpr int H = M / 2;
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < LPB * H; idx += THREADS) {
+      const int t = idx / H, kx = idx % H;
+      const int line = line0 + t;
+      if (line >= nlines) continue;
+      cplx<T>* X = spec + (size_t)line * g.pitch;
+      const cplx<T> Zk = buf[padi<T>(t * M + kx)];
+      if (kx == 0) {   // the real bins 0 and M, and the middle bin, whose partner is itself
+        const cplx<T> Zh = buf[padi<T>(t * M + H)];
+        st_c(X, mk<T>(T(2) * (Zk.x + Zk.y), T(0)));
+        st_c(X + M, mk<T>(T(2) * (Zk.x - Zk.y), T(0)));
+        st_c(X + H, mk<T>(T(2) * Zh.x, T(-2) * Zh.y));
+      } else {
+        cplx<T> Xk, Xm;
+        fwd_post_pair(Zk, buf[padi<T>(t * M + M - kx)], ldg_c(tt.lf_post + kx), Xk, Xm);
+        st_c(X + kx, Xk);
+        st_c(X + M - kx, Xm);
+      }
+    }
+    return;
+  }
   fft_static<T, M, -1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
   constexpr int M1 = M + 1;
 #pragma unroll 4
@@ -95,7 +104,42 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
   const int line0 = blockIdx.x * LPB;
-  {
+  if constexpr (sizeof(T) == 8) {   // FP64: bins k and M - k loaded once and packed together
+    constexpr int H = M / 2;
+    constexpr int PER = (LPB * H + THREADS - 1) / THREADS;
+    cplx<T> Xk[PER], Xm[PER];
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int idx = threadIdx.x + q * THREADS;
+      const int t = idx / H, kx = idx % H;
+      const int line = line0 + t;
+      Xk[q] = Xm[q] = mk<T>(T(0), T(0));
+      if (idx < LPB * H && line < nlines) {
+        const cplx<T>* row = spec + (size_t)line * g.pitch;
+        Xk[q] = ld_c(row + kx);
+        Xm[q] = ld_c(row + (M - kx));
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int idx = threadIdx.x + q * THREADS;
+      const int t = idx / H, kx = idx % H;
+      const int line = line0 + t;
+      if (idx >= LPB * H) continue;
+      if (kx == 0) {
+        const cplx<T> Xh = line < nlines ? ld_c(spec + (size_t)line * g.pitch + H) : mk<T>(T(0), T(0));
+        buf[padi<T>(t * M)] = mk<T>(Xk[q].x + Xm[q].x, Xk[q].x - Xm[q].x);
+        buf[padi<T>(t * M + H)] = mk<T>(T(2) * Xh.x, T(-2) * Xh.y);
+      } else {
+        cplx<T> Zk, Zm;
+        inv_pre_pair(Xk[q], Xm[q], ldg_c(tt.lf_post + kx), Zk, Zm);
+        buf[padi<T>(t * M + kx)] = Zk;
+        buf[padi<T>(t * M + M - kx)] = Zm;
+      }
+    }
+    __syncthreads();
+    fft_lf<T, M, 1, LPB, THREADS, 1, M, false>(buf, tt.lf_m);
+  } else {
     constexpr int PER = (LPB * M + THREADS - 1) / THREADS;
     cplx<T> Xk[PER], Xm[PER];
 #pragma unroll
@@ -116,9 +160,9 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
       const int kx = idx % M;
       if (idx < LPB * M) buf[padi<T>(idx)] = inv_pre(kx, Xk[q], Xm[q], ldg_c(tt.tw_post + kx));
     }
+    __syncthreads();
+    fft_static<T, M, 1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
   }
-  __syncthreads();
-  fft_static<T, M, 1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
   const T s = T(scl);
   if constexpr (!ACC && MODE == INV_FINAL) {
     // refined pressure: the pair (hi, lo) of every element is loaded before any assembly
@@ -293,7 +337,7 @@ inline cudaError_t set_smem(K kernel, int smem) {
 }
 
 // FP32 spectra of FP32 fields: the two-pass register kernels (k_fft_x_reg.cuh); the refinement
-// residual (Nx/2 >= 256) too, with its residual formed warp by warp into shared memory first.
+// residual too, with its residual formed warp by warp into shared memory first.
 // For the plain FP64 right-hand side and the FP64 assembly of the refined pressure the Stockham
 // kernels measured faster: those passes are latency-bound on their FP64 streams and want the
 // finer-grained CTAs (two lines, 63-80 registers) that the register kernels do not give.
@@ -366,11 +410,13 @@ cudaError_t launch_fwd_x_stockham(const Geometry& g, const DevTables& tb, const 
   const int nlines = g.ny * g.nz;
   const dim3 grid((nlines + C::LPB - 1) / C::LPB);
   cudaError_t e = cudaSuccess;
+  FwdArgs fa = args;
+  if (sizeof(T) == 8) fa.in_scale *= 0.5;   // the even/odd split's factor (fwd_post_pair)
 #define PP_FWDF(MODEV)                                                                  \
   {                                                                                     \
     auto k = k_fwd_x_fast<T, TI, M, MODEV>;                                             \
     if ((e = set_smem(k, C::SMEM)) != cudaSuccess) return e;                            \
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, args, tt, tb, spec, nlines);                \
+    k<<<grid, C::THREADS, C::SMEM, st>>>(g, fa, tt, tb, spec, nlines);                  \
   }
   if constexpr (sizeof(T) == 4 && sizeof(TI) == 8 && M >= 256 && M != 384) {
     // FP64 right-hand side into the FP32 spectrum: the input is the widest stream of the solve,
@@ -387,8 +433,9 @@ cudaError_t launch_fwd_x_stockham(const Geometry& g, const DevTables& tb, const 
       return cudaGetLastError();
     }
   }
-  if constexpr (sizeof(T) == 4 && sizeof(TI) == 8 && M >= 256) {
+  if constexpr (sizeof(T) == 4 && sizeof(TI) == 8) {
     // refinement residual: warp-per-line residual into shared memory, then the register transform
+    // (192x96x192: 32 us, 49 us for the Stockham form that this one replaces at Nx/2 < 256, too)
     if (mode == FWD_RESID) {
       using R = XReg<M>;
       auto k = args.rin ? k_fwd_x_reg_resid<M, true> : k_fwd_x_reg_resid<M, false>;
@@ -407,7 +454,6 @@ cudaError_t launch_fwd_x_stockham(const Geometry& g, const DevTables& tb, const 
   } else {
     switch (mode) {
       case FWD_PLAIN: PP_FWDF(FWD_PLAIN) break;
-      case FWD_RESID: PP_FWDF(FWD_RESID) break;
       default: return cudaErrorNotSupported;
     }
   }

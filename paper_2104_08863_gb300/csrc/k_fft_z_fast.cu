@@ -1,11 +1,11 @@
 // Specialised z-transform kernel (step (4) / (6) of Sec. 3.2): a CTA transforms a tile of W
 // adjacent kx columns of one y-plane along z (Nz points each).  The tile is loaded with
 // coalesced row segments of W complex values, transformed in place in (padded) shared memory
-// by the compile-time Stockham engine, and stored back.  W and the thread count are chosen so
+// by the compile-time Stockham engine (FP64: its form with fused twiddles), and stored back.  W and the thread count are chosen so
 // that each thread stages 16 (FP32) or 8 (FP64) complex values per stage, which keeps two
 // CTAs resident per SM so that one CTA's loads overlap the other's arithmetic.  A launch may
 // cover only the kx columns [kx_lo, kx_hi) (one slab of the spectrum; kx_lo a multiple of W).
-#include "fft_static.cuh"
+#include "fft_lf.cuh"
 #include "internal.h"
 #include "z_reg.cuh"
 
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(ZTile<T, NZ>::THREADS, ZTile<T, NZ>::MINB) k_f
     }
   }
   __syncthreads();
-  fft_static<T, NZ, SIGN, W, THREADS, W, 1, true>(buf, tt.tw_z);
+  fft_lf<T, NZ, SIGN, W, THREADS, W, 1, true>(buf, tt.lf_z);
 #pragma unroll 4
   for (int idx = threadIdx.x; idx < NZ * W; idx += THREADS) {
     const int n = idx / W, c = idx % W;

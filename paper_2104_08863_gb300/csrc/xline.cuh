@@ -28,21 +28,35 @@ template <> struct RealIO<float> {
   }
 };
 
+// The five stencil pairs of the divergence and its transpose at cells (j, k, i0) and (j, k, i0+1):
+// every field as one pair per load (i0 is even and so is nx), the x-neighbour outside as a scalar.
+template <typename TI> struct FacePairs {
+  TI u0, u1, u2, vl0, vl1, vh0, vh1, w00, w01, w10, w11;
+};
+template <typename TI>
+__device__ __forceinline__ FacePairs<TI> face_pairs(const Geometry& g, const TI* __restrict__ u,
+                                                    const TI* __restrict__ v, const TI* __restrict__ w, int j, int k,
+                                                    int i0) {
+  const size_t nx = g.nx;
+  const size_t row = ((size_t)j * g.nz + k) * nx;
+  FacePairs<TI> f;
+  RealIO<TI>::load2(u + row + i0, f.u0, f.u1);
+  f.u2 = u[row + (i0 + 2 == g.nx ? 0 : i0 + 2)];
+  RealIO<TI>::load2(v + row + i0, f.vl0, f.vl1);
+  RealIO<TI>::load2(v + row + (size_t)g.nz * nx + i0, f.vh0, f.vh1);
+  RealIO<TI>::load2(w + row + i0, f.w00, f.w01);
+  RealIO<TI>::load2(w + ((size_t)j * g.nz + (k + 1 == g.nz ? 0 : k + 1)) * nx + i0, f.w10, f.w11);
+  return f;
+}
+
 // Divergence (Eq. 7) at cells (j, k, i) and (j, k, i+1); TI arithmetic.
 template <typename TI>
 __device__ __forceinline__ void divergence_pair(const Geometry& g, const TI* __restrict__ u,
                                                 const TI* __restrict__ v, const TI* __restrict__ w, int j, int k,
                                                 int i0, TI inv_dx, TI inv_dy, TI inv_dz, TI& f0, TI& f1) {
-  const size_t nx = g.nx;
-  const size_t row = ((size_t)j * g.nz + k) * nx;
-  const TI* ur = u + row;
-  const TI ui0 = ur[i0], ui1 = ur[i0 + 1], ui2 = ur[(i0 + 2) % g.nx];
-  const TI* vlo = v + row;
-  const TI* vhi = v + row + (size_t)g.nz * nx;
-  const TI* w0 = w + row;
-  const TI* w1 = w + ((size_t)j * g.nz + (k + 1 == g.nz ? 0 : k + 1)) * nx;
-  f0 = (ui1 - ui0) * inv_dx + (vhi[i0] - vlo[i0]) * inv_dy + (w1[i0] - w0[i0]) * inv_dz;
-  f1 = (ui2 - ui1) * inv_dx + (vhi[i0 + 1] - vlo[i0 + 1]) * inv_dy + (w1[i0 + 1] - w0[i0 + 1]) * inv_dz;
+  const FacePairs<TI> f = face_pairs<TI>(g, u, v, w, j, k, i0);
+  f0 = (f.u1 - f.u0) * inv_dx + (f.vh0 - f.vl0) * inv_dy + (f.w10 - f.w00) * inv_dz;
+  f1 = (f.u2 - f.u1) * inv_dx + (f.vh1 - f.vl1) * inv_dy + (f.w11 - f.w01) * inv_dz;
 }
 
 // (G^T g)_{jki} / dy_j at cells (j,k,i0) and (j,k,i0+1) (adjoint right-hand side).
@@ -50,19 +64,12 @@ template <typename TI>
 __device__ __forceinline__ void gradT_pair(const Geometry& g, const TI* __restrict__ gu, const TI* __restrict__ gv,
                                            const TI* __restrict__ gw, int j, int k, int i0, TI inv_dx, TI inv_dz,
                                            TI inv_hj, TI inv_hj1, TI inv_dy, TI& f0, TI& f1) {
-  const size_t nx = g.nx;
-  const size_t row = ((size_t)j * g.nz + k) * nx;
-  const TI* ur = gu + row;
-  const TI u0 = ur[i0], u1 = ur[i0 + 1], u2 = ur[(i0 + 2) % g.nx];
-  const TI* w0 = gw + row;
-  const TI* w1 = gw + ((size_t)j * g.nz + (k + 1 == g.nz ? 0 : k + 1)) * nx;
-  const TI* vlo = gv + row;                         // face j (bottom of cell j)
-  const TI* vhi = gv + row + (size_t)g.nz * nx;     // face j+1
+  const FacePairs<TI> f = face_pairs<TI>(g, gu, gv, gw, j, k, i0);
   TI ty0 = TI(0), ty1 = TI(0);
-  if (j >= 1) { ty0 += vlo[i0] * inv_hj; ty1 += vlo[i0 + 1] * inv_hj; }
-  if (j + 1 <= g.ny - 1) { ty0 -= vhi[i0] * inv_hj1; ty1 -= vhi[i0 + 1] * inv_hj1; }
-  f0 = ((u0 - u1) * inv_dx + (w0[i0] - w1[i0]) * inv_dz + ty0) * inv_dy;
-  f1 = ((u1 - u2) * inv_dx + (w0[i0 + 1] - w1[i0 + 1]) * inv_dz + ty1) * inv_dy;
+  if (j >= 1) { ty0 += f.vl0 * inv_hj; ty1 += f.vl1 * inv_hj; }
+  if (j + 1 <= g.ny - 1) { ty0 -= f.vh0 * inv_hj1; ty1 -= f.vh1 * inv_hj1; }
+  f0 = ((f.u0 - f.u1) * inv_dx + (f.w00 - f.w10) * inv_dz + ty0) * inv_dy;
+  f1 = ((f.u1 - f.u2) * inv_dx + (f.w01 - f.w11) * inv_dz + ty1) * inv_dy;
 }
 
 // Refinement residual r = (f - <f>) - L_h p at cells (j,k,i0) and (j,k,i0+1), where f is the
@@ -160,14 +167,14 @@ __device__ __forceinline__ cplx<T> fwd_load(const Geometry& g, const FwdArgs& ar
     TI f0, f1;
     const TI s = TI(args.in_scale);
     divergence_pair<TI>(g, reinterpret_cast<const TI*>(args.u), reinterpret_cast<const TI*>(args.v),
-                        reinterpret_cast<const TI*>(args.w), j, k, i0, TI(g.inv_dx), TI(tt.inv_dy[j]),
-                        TI(g.inv_dz), f0, f1);
-    return mk<T>(T(f0 * s), T(f1 * s));
+                        reinterpret_cast<const TI*>(args.w), j, k, i0, TI(g.inv_dx) * s, TI(tt.inv_dy[j]) * s,
+                        TI(g.inv_dz) * s, f0, f1);
+    return mk<T>(T(f0), T(f1));
   } else if constexpr (MODE == FWD_GRADT) {
     TI f0, f1;
     gradT_pair<TI>(g, reinterpret_cast<const TI*>(args.u), reinterpret_cast<const TI*>(args.v),
                    reinterpret_cast<const TI*>(args.w), j, k, i0, TI(g.inv_dx), TI(g.inv_dz),
-                   TI(tt.inv_h[j]), TI(tt.inv_h[j + 1]), TI(tt.inv_dy[j]), f0, f1);
+                   TI(tt.inv_h[j]), TI(tt.inv_h[j + 1]), TI(tt.inv_dy[j]) * TI(args.in_scale), f0, f1);
     return mk<T>(T(f0), T(f1));
   } else {  // FWD_RESID: FP64 rhs (or a stored residual), FP32 pressure field, double-float arithmetic
     if constexpr (sizeof(T) == 4) {
