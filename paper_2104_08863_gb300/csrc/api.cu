@@ -74,7 +74,7 @@ namespace pp {
 cudaError_t ensure_smem_limit(const void* kernel, size_t bytes) {
   static std::mutex mu;
   static std::unordered_map<const void*, size_t> granted;
-  if (bytes <= 48 * 1024) return cudaSuccess;
+  if (bytes <= 47 * 1024) return cudaSuccess;   // 48 KB less room for a kernel's static shared memory
   std::lock_guard<std::mutex> lock(mu);
   auto it = granted.find(kernel);
   if (it != granted.end() && it->second >= bytes) return cudaSuccess;
@@ -638,9 +638,7 @@ poisson_status projection_impl(Exec& ex, void* u, void* v, void* w, void* p_out,
 poisson_status projection_pairs(Exec& ex, void* u, void* v, void* w, void* p_out, double dt) {
   const poisson_plan_s* pl = ex.pl;
   PP_RET(check_finite_uvw<double>(ex, u, v, w));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)u, cell_count(pl), ex.st));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)v, vface_count(pl), ex.st));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)w, cell_count(pl), ex.st));
+  PP_TRY_N("to_pairs", launch_to_pairs(pl->g, (double*)u, (double*)v, (double*)w, ex.st));
   double* f = (double*)p_out;
   PP_TRY_N("divergence_df", launch_divergence_df(pl->g, ex.dt, (const float2*)u, (const float2*)v,
                                                  (const float2*)w, dt, f, ex.st));
@@ -674,9 +672,7 @@ poisson_status predictor_pairs(Exec& ex, void* u, void* v, void* w, void* ub, vo
                                double nu, double fx) {
   const poisson_plan_s* pl = ex.pl;
   PP_RET(check_finite_uvw<double>(ex, u, v, w));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)u, cell_count(pl), ex.st));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)v, vface_count(pl), ex.st));
-  PP_TRY_N("to_pairs", launch_to_pairs((double*)w, cell_count(pl), ex.st));
+  PP_TRY_N("to_pairs", launch_to_pairs(pl->g, (double*)u, (double*)v, (double*)w, ex.st));
   MomArgsDF s1{(const float2*)u, (const float2*)v, (const float2*)w, nullptr, nullptr, nullptr,
                (float2*)ub, (float2*)vb, (float2*)wb, 0.0, 1.0, dt, nu, fx};
   PP_TRY_N("momentum_df_1", launch_momentum_df(pl->g, ex.dt, s1, ex.st));
@@ -891,9 +887,7 @@ poisson_status momentum_predictor(poisson_plan_t pl, void* u, void* v, void* w, 
   Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
   if (pl->precision != PP_FP32_REFINED) return predictor_impl(ex, u, v, w, ub, vb, wb, dt, nu, fx);
   PP_RET(predictor_pairs(ex, u, v, w, ub, vb, wb, dt, nu, fx));
-  PP_TRY_N("from_pairs", launch_from_pairs((double*)u, cell_count(pl), ex.st));
-  PP_TRY_N("from_pairs", launch_from_pairs((double*)v, vface_count(pl), ex.st));
-  PP_TRY_N("from_pairs", launch_from_pairs((double*)w, cell_count(pl), ex.st));
+  PP_TRY_N("from_pairs", launch_from_pairs(pl->g, (double*)u, (double*)v, (double*)w, ex.st));
   return PS_OK;
 }
 

@@ -221,6 +221,9 @@ template <typename T>
 cudaError_t launch_momentum(const Geometry& g, const DevTables& tb, const MomArgs<T>& a, cudaStream_t st,
                             int jlo = 0, int jhi = -1);
 
+// Rows per chunk of a momentum launch whose x-z tiles are `tiles` CTAs (k_momentum.cu).
+int momentum_chunk_rows(long long tiles, int rows);
+
 // The FP64-accurate timestep on FP32 units (csrc/k_refined_ts.cu): the state as FP32 pairs
 // (hi, lo) in the FP64 buffers, double-float momentum stages, divergence and gradient.
 struct MomArgsDF {
@@ -229,8 +232,9 @@ struct MomArgsDF {
   float2 *ou, *ov, *ow;
   double alpha, beta, bdt, nu, fx;
 };
-cudaError_t launch_to_pairs(double* x, size_t n, cudaStream_t st);
-cudaError_t launch_from_pairs(double* x, size_t n, cudaStream_t st);
+// The velocity triple between FP64 and FP32 pairs, in place (one launch).
+cudaError_t launch_to_pairs(const Geometry& g, double* u, double* v, double* w, cudaStream_t st);
+cudaError_t launch_from_pairs(const Geometry& g, double* u, double* v, double* w, cudaStream_t st);
 cudaError_t launch_momentum_df(const Geometry& g, const DevTables& tb, const MomArgsDF& a, cudaStream_t st);
 cudaError_t launch_divergence_df(const Geometry& g, const DevTables& tb, const float2* u, const float2* v,
                                  const float2* w, double dt, double* f, cudaStream_t st);

@@ -29,6 +29,26 @@
 
 namespace pp {
 
+// Rows per chunk: the split of the rows that minimises (CTAs on the busiest SM) x (rows + the
+// chunk's own start, worth about one row), so that small grids fill the SMs and large ones do not
+// repeat the start; at least 4 rows.  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks
+// had at least 16 rows and filled 64 SMs.)
+int momentum_chunk_rows(long long tiles, int rows) {
+  int best = rows;
+  double cost = -1.0;
+  for (int chunks = 1; chunks <= (rows + 3) / 4; ++chunks) {
+    const int jc = (rows + chunks - 1) / chunks;
+    const long long ctas = tiles * ((rows + jc - 1) / jc);
+    const double t = (double)((ctas + 151) / 152) * (jc + 1.0);
+    if (cost < 0.0 || t < cost) {
+      cost = t;
+      best = jc;
+    }
+    if (ctas > 152LL * 64) break;
+  }
+  return best;
+}
+
 namespace {
 
 constexpr int MOM_THREADS = 256;
@@ -239,26 +259,6 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
   if (j1 == ny) vst<T, V>(a.ov + o, BASE ? vldv<T, V>(a.bv + o) : v_c);   // top wall face of v: boundary value
 }
 
-// Rows per chunk: the split of the rows that minimises (CTAs on the busiest SM) x (rows + the
-// chunk's own start, worth about one row), so that small grids fill the SMs and large ones do not
-// repeat the start; at least 4 rows.  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks
-// had at least 16 rows and filled 64 SMs.)
-int chunk_rows(long long tiles, int rows) {
-  int best = rows;
-  double cost = -1.0;
-  for (int chunks = 1; chunks <= (rows + 3) / 4; ++chunks) {
-    const int jc = (rows + chunks - 1) / chunks;
-    const long long ctas = tiles * ((rows + jc - 1) / jc);
-    const double t = (double)((ctas + 151) / 152) * (jc + 1.0);
-    if (cost < 0.0 || t < cost) {
-      cost = t;
-      best = jc;
-    }
-    if (ctas > 152LL * 64) break;
-  }
-  return best;
-}
-
 template <typename T, int V>
 cudaError_t launch_momentum_v(const Geometry& g, const DevTables& tb, const MomArgs<T>& a, const MomCoef& mc,
                               cudaStream_t st, int jlo, int jhi) {
@@ -267,7 +267,7 @@ cudaError_t launch_momentum_v(const Geometry& g, const DevTables& tb, const MomA
   while (tx > 1 && (tx / 2) * V >= g.nx) tx /= 2;
   const int tz = MOM_THREADS / tx;
   const int gx = (g.nx + tx * V - 1) / (tx * V), gz = (g.nz + tz - 1) / tz;
-  const int jc = chunk_rows((long long)gx * gz, rows);
+  const int jc = momentum_chunk_rows((long long)gx * gz, rows);
   const size_t smem = sizeof(RowCoef<T>) * (size_t)jc;
   const dim3 grid(gx, gz, (rows + jc - 1) / jc), block(tx, tz);
   const bool base = a.bu != nullptr;

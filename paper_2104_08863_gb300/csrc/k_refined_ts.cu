@@ -105,27 +105,49 @@ __device__ __forceinline__ void acc_out2(const Acc2& a, float2& x, float2& y) {
 
 constexpr int MTX = 32, MTZ = 8;
 
+// Stage constants split on the host: the FP64 divisions of every thread took 10 % of the stage
+// (512x384x512: 2.74 / 3.40 ms with them, 2.47 / 3.10 without).
+struct MomCoefDF {
+  double cdx, cdz, bdtnu;
+  df cDx, cDz, cAx, cAz, fterm, alpha;
+};
+
 struct RowCoefDF {
   df c0, ca, cc, cay;
   df v0, va, vc, vay;
 };
 
-__global__ void __launch_bounds__(256) k_to_pairs(double* __restrict__ x, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const df s = split(x[i]);
-    reinterpret_cast<float2*>(x)[i] = f2(s);
+// Two values (16 bytes) per thread and step, the velocity triple in one launch (field blockIdx.y; its
+// length is even): 740 us at 512x384x512 (6.5 TB/s), one value per step and a launch per field 865.
+struct Triple {
+  double* x[3];
+  size_t n[3];
+};
+
+__global__ void __launch_bounds__(256) k_to_pairs(Triple f) {
+  double* x = f.x[blockIdx.y];
+  const size_t n2 = f.n[blockIdx.y] / 2, step = (size_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += step) {
+    const double2 v = reinterpret_cast<const double2*>(x)[i];
+    const df p = split(v.x), q = split(v.y);
+    reinterpret_cast<float4*>(x)[i] = make_float4(p.hi, p.lo, q.hi, q.lo);
   }
 }
 
-__global__ void __launch_bounds__(256) k_from_pairs(double* __restrict__ x, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 v = reinterpret_cast<const float2*>(x)[i];
-    x[i] = f32_add_to_f64(v.x, v.y);
+__global__ void __launch_bounds__(256) k_from_pairs(Triple f) {
+  double* x = f.x[blockIdx.y];
+  const size_t n2 = f.n[blockIdx.y] / 2, step = (size_t)gridDim.x * blockDim.x;
+#pragma unroll 4
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += step) {
+    const float4 v = reinterpret_cast<const float4*>(x)[i];
+    reinterpret_cast<double2*>(x)[i] = make_double2(f32_add_to_f64(v.x, v.y), f32_add_to_f64(v.z, v.w));
   }
 }
 
 // out = alpha * base + beta * s + bdt * R(s) on pairs (see k_momentum for the stencil).
-__global__ void __launch_bounds__(MTX * MTZ) k_momentum_df(Geometry g, MomArgsDF a, const double* __restrict__ inv_dy,
+__global__ void __launch_bounds__(MTX * MTZ) k_momentum_df(Geometry g, MomArgsDF a, MomCoefDF mc,
+                                                          const double* __restrict__ inv_dy,
                                                           const double* __restrict__ inv_h,
                                                           const double* __restrict__ lo,
                                                           const double* __restrict__ up, int jc) {
@@ -134,8 +156,7 @@ __global__ void __launch_bounds__(MTX * MTZ) k_momentum_df(Geometry g, MomArgsDF
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int j0 = blockIdx.z * jc;
   const int j1 = min(ny, j0 + jc);
-  const double bdtnu = a.bdt * a.nu;
-  const double cdx = bdtnu / (g.dx * g.dx), cdz = bdtnu / (g.dz * g.dz);
+  const double bdtnu = mc.bdtnu, cdx = mc.cdx, cdz = mc.cdz;
   for (int r = threadIdx.y * MTX + threadIdx.x; r < j1 - j0; r += MTX * MTZ) {
     const int j = j0 + r;
     RowCoefDF c;
@@ -160,11 +181,9 @@ __global__ void __launch_bounds__(MTX * MTZ) k_momentum_df(Geometry g, MomArgsDF
   const int i = blockIdx.x * MTX + threadIdx.x;
   const int k = blockIdx.y * MTZ + threadIdx.y;
   if (i >= nx || k >= nz) return;
-  const df cDx = split(cdx), cDz = split(cdz);
-  const df cAx = split(-0.25 * a.bdt / g.dx), cAz = split(-0.25 * a.bdt / g.dz);
+  const df cDx = mc.cDx, cDz = mc.cDz, cAx = mc.cAx, cAz = mc.cAz;
   const df2 cD_xz = pk(cDx, cDz), cD_zx = pk(cDz, cDx), cA_xz = pk(cAx, cAz), cA_zx = pk(cAz, cAx);
-  const df fterm = split(a.bdt * a.fx);
-  const df alpha = split(a.alpha);
+  const df fterm = mc.fterm, alpha = mc.alpha;
   const bool has_base = a.bu != nullptr;
   const size_t plane = (size_t)nz * nx;
   const int im = i == 0 ? nx - 1 : i - 1, ip = i == nx - 1 ? 0 : i + 1;
@@ -268,122 +287,151 @@ __global__ void __launch_bounds__(MTX * MTZ) k_momentum_df(Geometry g, MomArgsDF
   }
 }
 
-// f = D(u*) / dt at every cell from the pairs, written as FP64 (faithful assembly).
+__device__ __forceinline__ df at0(float4 v) { return df{v.x, v.y}; }
+__device__ __forceinline__ df at1(float4 v) { return df{v.z, v.w}; }
+__device__ __forceinline__ float4 ld4(const float2* p) { return *reinterpret_cast<const float4*>(p); }
+
+// f = D(u*) / dt at every cell from the pairs, written as FP64 (faithful assembly).  A thread takes
+// two adjacent cells of a line, every field as 16-byte loads of two pairs, all in flight before the
+// first use; 1/(dt dx) and 1/(dt dz) come split from the host (HBM-bound: 32 bytes per point;
+// 512x384x512 620 us (5.2 TB/s), one cell per
+// thread with divisions on the device 770).
 __global__ void __launch_bounds__(256) k_divergence_df(Geometry g, const float2* __restrict__ u,
                                                       const float2* __restrict__ v, const float2* __restrict__ w,
-                                                      const double* __restrict__ inv_dy, double inv_dt,
+                                                      const double* __restrict__ inv_dy, df cx, df cz, df cdt,
                                                       double* __restrict__ f) {
   const size_t plane = (size_t)g.nz * g.nx;
-  const int nlines = g.ny * g.nz;
-  const df cx = split(inv_dt / g.dx), cz = split(inv_dt / g.dz), cdt = split(inv_dt);
-  for (int line = blockIdx.x; line < nlines; line += gridDim.x) {
-    const int j = line / g.nz, k = line - j * g.nz;
-    const df cy = dmul(cdt, split(inv_dy[j]));
-    for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-      const size_t idx = (size_t)line * g.nx + i;
-      const size_t oxp = idx - i + (i + 1 == g.nx ? 0 : i + 1);
-      const size_t ozp = (size_t)j * plane + (size_t)(k + 1 == g.nz ? 0 : k + 1) * g.nx + i;
-      df s = dmul(cx, dsub(ldp(u + oxp), ldp(u + idx)));
-      s = dfma(cz, dsub(ldp(w + ozp), ldp(w + idx)), s);
-      s = dfma(cy, dsub(ldp(v + idx + plane), ldp(v + idx)), s);
-      f[idx] = f32_add_to_f64(s.hi, s.lo);
-    }
+  const int line = blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= g.ny * g.nz) return;
+  const int j = line / g.nz, k = line - j * g.nz;
+  const df cy = dmul(cdt, split(inv_dy[j]));
+  const ptrdiff_t dzp = k + 1 == g.nz ? (ptrdiff_t)g.nx - (ptrdiff_t)plane : g.nx;
+  for (int i0 = 2 * threadIdx.x; i0 < g.nx; i0 += 2 * blockDim.x) {
+    const size_t idx = (size_t)line * g.nx + i0;
+    const float4 uc = ld4(u + idx), wc = ld4(w + idx), wp = ld4(w + idx + dzp), vc = ld4(v + idx), vp = ld4(v + idx + plane);
+    const df u2 = ldp(u + idx + (i0 + 2 == g.nx ? -(ptrdiff_t)i0 : 2));
+    auto cell = [&](df ul, df ur, df wl, df wr, df vl, df vr) {
+      df s = dmul(cx, dsub(ur, ul));
+      s = dfma(cz, dsub(wr, wl), s);
+      s = dfma(cy, dsub(vr, vl), s);
+      return f32_add_to_f64(s.hi, s.lo);
+    };
+    *reinterpret_cast<double2*>(f + idx) = make_double2(cell(at0(uc), at1(uc), at0(wc), at0(wp), at0(vc), at0(vp)),
+                                                        cell(at1(uc), u2, at1(wc), at1(wp), at1(vc), at1(vp)));
   }
 }
 
 // u = u* - dt G p (Eq. 4): u* as pairs, p = hi + lo the refined solve's FP32 pair, the result in
 // FP64 (v's walls copied); the pressure differences and the products run in double-float and the
-// sums are assembled into FP64 with integer operations (no FP64 instruction per point).  p_out,
-// when given, receives p in FP64.
+// sums are assembled into FP64 with integer operations (one FP64 addition per value).  p_out, when
+// given, receives p in FP64.  Two adjacent cells per thread as above (HBM-bound: 64 bytes per point
+// with p_out; 512x384x512 1.21 ms (5.3 TB/s), before 1.60).
 __global__ void __launch_bounds__(256) k_gradient_pairs(Geometry g, const float* __restrict__ hi,
                                                         const float* __restrict__ lo, double* __restrict__ u,
                                                         double* __restrict__ v, double* __restrict__ w,
                                                         double* __restrict__ p_out, const double* __restrict__ inv_h,
-                                                        double dt) {
+                                                        df cx, df cz, df cdt) {
   const size_t plane = (size_t)g.nz * g.nx;
-  const int nlines = (g.ny + 1) * g.nz;
-  const df cx = split(dt / g.dx), cz = split(dt / g.dz), cdt = split(dt);
-  const float2* up = reinterpret_cast<const float2*>(u);
-  const float2* vp = reinterpret_cast<const float2*>(v);
-  const float2* wp = reinterpret_cast<const float2*>(w);
-  auto P = [&](size_t o) { return df{__ldg(hi + o), __ldg(lo + o)}; };
-  for (int line = blockIdx.x; line < nlines; line += gridDim.x) {
-    const int j = line / g.nz, k = line - j * g.nz;
-    const df cy = (j >= 1 && j < g.ny) ? dmul(cdt, split(inv_h[j])) : df{0.f, 0.f};
-    for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-      const size_t idx = (size_t)line * g.nx + i;
-      const float2 vv = vp[idx];
-      df vn{vv.x, vv.y};
-      if (j < g.ny) {
-        const float2 uu = up[idx], ww = wp[idx];
-        const df pc = P(idx);
-        const df pxm = P(idx - i + (i == 0 ? g.nx - 1 : i - 1));
-        const df pzm = P((size_t)j * plane + (size_t)(k == 0 ? g.nz - 1 : k - 1) * g.nx + i);
-        const df un = dsub(df{uu.x, uu.y}, dmul(cx, dsub(pc, pxm)));
-        const df wn = dsub(df{ww.x, ww.y}, dmul(cz, dsub(pc, pzm)));
-        u[idx] = f32_add_to_f64(un.hi, un.lo);
-        w[idx] = f32_add_to_f64(wn.hi, wn.lo);
-        if (p_out) p_out[idx] = f32_add_to_f64(pc.hi, pc.lo);
-        if (j >= 1) {
-          vn = dsub(vn, dmul(cy, dsub(pc, P(idx - plane))));
-          v[idx] = f32_add_to_f64(vn.hi, vn.lo);
-        } else {
-          v[idx] = f32_add_to_f64(vn.hi, vn.lo);
-        }
-      } else {
-        v[idx] = f32_add_to_f64(vn.hi, vn.lo);
+  const int line = blockIdx.x * blockDim.y + threadIdx.y;
+  if (line >= (g.ny + 1) * g.nz) return;
+  const int j = line / g.nz, k = line - j * g.nz;
+  const bool cell = j < g.ny, inner = j >= 1 && cell;
+  const df cy = inner ? dmul(cdt, split(inv_h[j])) : df{0.f, 0.f};
+  const ptrdiff_t dzm = k == 0 ? (ptrdiff_t)plane - g.nx : -(ptrdiff_t)g.nx;
+  auto P2 = [&](size_t o) {   // the pressure pairs of two cells
+    const float2 h = __ldg(reinterpret_cast<const float2*>(hi + o)), l = __ldg(reinterpret_cast<const float2*>(lo + o));
+    return make_float4(h.x, l.x, h.y, l.y);
+  };
+  auto out = [](df a, df b) { return make_double2(f32_add_to_f64(a.hi, a.lo), f32_add_to_f64(b.hi, b.lo)); };
+  for (int i0 = 2 * threadIdx.x; i0 < g.nx; i0 += 2 * blockDim.x) {
+    const size_t idx = (size_t)line * g.nx + i0;
+    const float4 vv = *reinterpret_cast<const float4*>(v + idx);
+    df v0 = at0(vv), v1 = at1(vv);
+    if (cell) {
+      const float4 uu = *reinterpret_cast<const float4*>(u + idx), ww = *reinterpret_cast<const float4*>(w + idx);
+      const float4 pc = P2(idx), pz = P2(idx + dzm), py = inner ? P2(idx - plane) : pc;
+      const size_t ox = idx + (i0 == 0 ? g.nx - 1 : -1);
+      const df pl{__ldg(hi + ox), __ldg(lo + ox)};
+      *reinterpret_cast<double2*>(u + idx) = out(dsub(at0(uu), dmul(cx, dsub(at0(pc), pl))),
+                                                 dsub(at1(uu), dmul(cx, dsub(at1(pc), at0(pc)))));
+      *reinterpret_cast<double2*>(w + idx) = out(dsub(at0(ww), dmul(cz, dsub(at0(pc), at0(pz)))),
+                                                 dsub(at1(ww), dmul(cz, dsub(at1(pc), at1(pz)))));
+      if (p_out) *reinterpret_cast<double2*>(p_out + idx) = out(at0(pc), at1(pc));
+      if (inner) {
+        v0 = dsub(v0, dmul(cy, dsub(at0(pc), at0(py))));
+        v1 = dsub(v1, dmul(cy, dsub(at1(pc), at1(py))));
       }
     }
+    *reinterpret_cast<double2*>(v + idx) = out(v0, v1);
   }
 }
 
-int line_grid(int nlines) { return nlines < 152 * 16 ? nlines : 152 * 16; }
-int line_block(int nx) { return nx >= 256 ? 256 : (nx + 31) / 32 * 32; }
+// CTAs of tx pairs of cells by 256 / tx lines.
+struct LineTiles { dim3 grid, block; };
+LineTiles pair_tiles(const Geometry& g, int nlines) {
+  const int tx = g.nx / 2 < 256 ? g.nx / 2 : 256, ty = 256 / tx;
+  return LineTiles{dim3((nlines + ty - 1) / ty), dim3(tx, ty)};
+}
 
-int grid_for(size_t total) {
-  size_t blocks = (total + 255) / 256;
-  const size_t cap = 152 * 16;
-  return (int)(blocks < cap ? (blocks ? blocks : 1) : cap);
+df split_host(double x) {
+  df r;
+  f64_split(x, r.hi, r.lo);
+  return r;
+}
+
+// Grid of the in-place conversions: 16 CTAs per SM, each field of the triple in its own rows.
+dim3 triple_grid(const Triple& f) {
+  const size_t most = f.n[0] > f.n[1] ? f.n[0] : f.n[1], blocks = (most / 2 + 255) / 256;
+  return dim3((unsigned)(blocks < 152 * 16 ? (blocks ? blocks : 1) : 152 * 16), 3);
+}
+Triple triple(const Geometry& g, double* u, double* v, double* w) {
+  const size_t plane = (size_t)g.nz * g.nx;
+  return Triple{{u, v, w}, {plane * g.ny, plane * (g.ny + 1), plane * g.ny}};
 }
 
 }  // namespace
 
-cudaError_t launch_to_pairs(double* x, size_t n, cudaStream_t st) {
-  k_to_pairs<<<grid_for(n), 256, 0, st>>>(x, n);
+cudaError_t launch_to_pairs(const Geometry& g, double* u, double* v, double* w, cudaStream_t st) {
+  const Triple f = triple(g, u, v, w);
+  k_to_pairs<<<triple_grid(f), 256, 0, st>>>(f);
   return cudaGetLastError();
 }
 
-cudaError_t launch_from_pairs(double* x, size_t n, cudaStream_t st) {
-  k_from_pairs<<<grid_for(n), 256, 0, st>>>(x, n);
+cudaError_t launch_from_pairs(const Geometry& g, double* u, double* v, double* w, cudaStream_t st) {
+  const Triple f = triple(g, u, v, w);
+  k_from_pairs<<<triple_grid(f), 256, 0, st>>>(f);
   return cudaGetLastError();
 }
 
 cudaError_t launch_momentum_df(const Geometry& g, const DevTables& tb, const MomArgsDF& a, cudaStream_t st) {
   const int tx = (g.nx + MTX - 1) / MTX, tz = (g.nz + MTZ - 1) / MTZ;
   const long long tiles = (long long)tx * tz;
-  int chunks = (int)((3LL * 2 * 152 + tiles - 1) / tiles);
-  if (chunks > g.ny / 16) chunks = g.ny / 16;
-  if (chunks < 1) chunks = 1;
-  const int jc = (g.ny + chunks - 1) / chunks;
-  chunks = (g.ny + jc - 1) / jc;
+  const int jc = momentum_chunk_rows(tiles, g.ny), chunks = (g.ny + jc - 1) / jc;
   const size_t smem = sizeof(RowCoefDF) * (size_t)jc;
   const cudaError_t e = ensure_smem_limit((const void*)k_momentum_df, smem);
   if (e != cudaSuccess) return e;
   dim3 grid(tx, tz, chunks), block(MTX, MTZ);
-  k_momentum_df<<<grid, block, smem, st>>>(g, a, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jc);
+  const double bdtnu = a.bdt * a.nu, cdx = bdtnu / (g.dx * g.dx), cdz = bdtnu / (g.dz * g.dz);
+  const MomCoefDF mc{cdx, cdz, bdtnu, split_host(cdx), split_host(cdz), split_host(-0.25 * a.bdt / g.dx),
+                     split_host(-0.25 * a.bdt / g.dz), split_host(a.bdt * a.fx), split_host(a.alpha)};
+  k_momentum_df<<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jc);
   return cudaGetLastError();
 }
 
 cudaError_t launch_divergence_df(const Geometry& g, const DevTables& tb, const float2* u, const float2* v,
                                  const float2* w, double dt, double* f, cudaStream_t st) {
-  k_divergence_df<<<line_grid(g.ny * g.nz), line_block(g.nx), 0, st>>>(g, u, v, w, tb.d.inv_dy, 1.0 / dt, f);
+  const LineTiles t = pair_tiles(g, g.ny * g.nz);
+  const double inv_dt = 1.0 / dt;
+  k_divergence_df<<<t.grid, t.block, 0, st>>>(g, u, v, w, tb.d.inv_dy, split_host(inv_dt / g.dx),
+                                              split_host(inv_dt / g.dz), split_host(inv_dt), f);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gradient_pairs(const Geometry& g, const DevTables& tb, const float* hi, const float* lo, double* u,
                                   double* v, double* w, double* p_out, double dt, cudaStream_t st) {
-  k_gradient_pairs<<<line_grid((g.ny + 1) * g.nz), line_block(g.nx), 0, st>>>(g, hi, lo, u, v, w, p_out,
-                                                                                tb.d.inv_h, dt);
+  const LineTiles t = pair_tiles(g, (g.ny + 1) * g.nz);
+  k_gradient_pairs<<<t.grid, t.block, 0, st>>>(g, hi, lo, u, v, w, p_out, tb.d.inv_h, split_host(dt / g.dx),
+                                               split_host(dt / g.dz), split_host(dt));
   return cudaGetLastError();
 }
 
