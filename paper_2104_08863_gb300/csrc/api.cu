@@ -66,6 +66,24 @@ void put_real_table(std::vector<unsigned char>& img, size_t off, const std::vect
   for (size_t i = 0; i < v.size(); ++i) p[i] = (T)v[i];
 }
 
+// cos, sin and tan of 2 pi q / L (0 <= q < L) to within an ulp or so of each: the angle is reduced to
+// an octant by integer arithmetic, (pi/4) (8q mod L) / L, reflected into [0, pi/4] and rotated back.
+struct UnitRoot { double c, s, t; };
+UnitRoot unit_root(long long q, long long L) {
+  const long long oct = 8 * q / L, r = 8 * q - oct * L;
+  const bool odd = oct & 1;
+  const double phi = M_PI / 4.0 * ((double)(odd ? L - r : r) / (double)L);
+  double c = cos(phi), s = odd ? -sin(phi) : sin(phi), t = odd ? -tan(phi) : tan(phi);
+  for (long long k = (oct + 1) / 2; k > 0; --k) {   // by quarter turns: tan(x + pi/2) = -1 / tan(x)
+    const double cc = c;
+    c = -s;
+    s = cc;
+  }
+  if (((oct + 1) / 2) & 1) t = -1.0 / t;
+  if (c == 0.0) c = 0.0;   // no negative zero
+  return UnitRoot{c, s, t};
+}
+
 bool spec_is_fp64(const poisson_plan_s* pl) { return pl->precision == PP_FP64; }
 
 }  // namespace
@@ -230,12 +248,13 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
     const double s = sin(M_PI * k / g.nz);
     pl->lamz[k] = -(4.0 / (g.dz * g.dz)) * s * s;
   }
-  // --- twiddles (FP64 trig, index-reduced angles) ---
+  // --- twiddles ---
   auto twid = [](int L, int n, std::vector<double>& re, std::vector<double>& im) {
     re.resize(n); im.resize(n);
     for (int t = 0; t < n; ++t) {
-      const double ang = -2.0 * M_PI * (double)t / (double)L;
-      re[t] = cos(ang); im[t] = sin(ang);
+      const UnitRoot w = unit_root(t, L);
+      re[t] = w.c;
+      im[t] = -w.s;
     }
   };
   std::vector<double> twm_r, twm_i, twp_r, twp_i, twz_r, twz_i;
@@ -268,9 +287,10 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
     auto cos_tan = [&](int id, int L, int n) {
       std::vector<double> c(n), t(n);
       for (int q = 0; q < n; ++q) {
-        const double ang = 2.0 * M_PI * (double)q / (double)L;
-        c[q] = cos(ang);   // never 0: pi/2 is not a double
-        t[q] = sin(ang) / c[q];
+        const UnitRoot w = unit_root(q, L);
+        // a quarter turn: cos as 2^-54 and tan as +-2^54, whose product is exact
+        c[q] = w.c != 0.0 ? w.c : 0x1p-54;
+        t[q] = w.c != 0.0 ? w.t : w.s * 0x1p54;
       }
       put_cplx_table<double>(img, to[id], c, t);
     };
@@ -812,6 +832,13 @@ poisson_status solve_on_workspace(poisson_plan_s* pl, unsigned char* ws, const D
 }
 }  // namespace pp
 
+// The z lengths that poisson_plan_set_chain takes (its z tiles).
+static bool chain_nz(int nz) {
+  for (int n : {16, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024})
+    if (n == nz) return true;
+  return false;
+}
+
 extern "C" {
 
 poisson_status poisson_solve(poisson_plan_t pl, const void* rhs, void* p, void* stream) {
@@ -1025,7 +1052,7 @@ poisson_status poisson_plan_set_chain(poisson_plan_t pl, int slab_cols, int stre
   const Geometry& g = pl->g;
   const int wz = pp::fft_z_fast_tile<float>(g);
   const bool path_ok = pl->precision != PP_FP64 && !pl->has_tri && pp::scan_tridiag_ok(g.ny, pl->parts) &&
-                       !g.generic_fft && wz > 0;
+                       !g.generic_fft && chain_nz(g.nz);
   if (!path_ok) return PS_EUNSUPPORTED;
   const int step = wz > pp::reg_systems_per_cta(pl->parts) ? wz : pp::reg_systems_per_cta(pl->parts);
   if (slab_cols % step || slab_cols <= pl->low) return PS_EUNSUPPORTED;

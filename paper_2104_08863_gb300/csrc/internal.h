@@ -121,23 +121,20 @@ template <typename T>
 cudaError_t launch_fft_z(const Geometry& g, const DevTables& tb, const FftFactors& fz, int sign, cplx<T>* spec,
                          cudaStream_t st);
 
-// Specialised x-transforms for Nx/2 in {16, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024}
-// (cudaErrorNotSupported otherwise).  Suffix: spectral type, field type (d = double, f = float).
-cudaError_t launch_fwd_x_fast_dd(const Geometry& g, const DevTables& tb, FwdMode mode, const FwdArgs& args,
-                                 cplx<double>* spec, cudaStream_t st);
-cudaError_t launch_fwd_x_fast_ff(const Geometry& g, const DevTables& tb, FwdMode mode, const FwdArgs& args,
-                                 cplx<float>* spec, cudaStream_t st);
-cudaError_t launch_fwd_x_fast_fd(const Geometry& g, const DevTables& tb, FwdMode mode, const FwdArgs& args,
-                                 cplx<float>* spec, cudaStream_t st);
-cudaError_t launch_inv_x_fast_dd(const Geometry& g, const DevTables& tb, InvMode mode, const cplx<double>* spec,
-                                 double* out, double scale, bool accumulate, cudaStream_t st, PairArgs pair);
-cudaError_t launch_inv_x_fast_ff(const Geometry& g, const DevTables& tb, InvMode mode, const cplx<float>* spec,
-                                 float* out, double scale, bool accumulate, cudaStream_t st, PairArgs pair);
-cudaError_t launch_inv_x_fast_fd(const Geometry& g, const DevTables& tb, InvMode mode, const cplx<float>* spec,
-                                 double* out, double scale, bool accumulate, cudaStream_t st, PairArgs pair);
+// Specialised x-transforms (k_fft_x_fast.cuh), cudaErrorNotSupported for other lengths.  Suffix:
+// spectral type, field type (d = double, f = float), group of half-lengths.
+#define PP_X_FAST(SFX, T, TF)                                                                                       \
+  cudaError_t launch_fwd_x_fast_##SFX(const Geometry& g, const DevTables& tb, FwdMode mode, const FwdArgs& args,    \
+                                      cplx<T>* spec, cudaStream_t st);                                              \
+  cudaError_t launch_inv_x_fast_##SFX(const Geometry& g, const DevTables& tb, InvMode mode, const cplx<T>* spec,    \
+                                      TF* out, double scale, bool accumulate, cudaStream_t st, PairArgs pair);
+PP_X_FAST(dd_a, double, double) PP_X_FAST(dd_b, double, double) PP_X_FAST(dd_c, double, double)
+PP_X_FAST(ff_a, float, float) PP_X_FAST(ff_b, float, float) PP_X_FAST(ff_c, float, float)
+PP_X_FAST(fd_a, float, double) PP_X_FAST(fd_b, float, double) PP_X_FAST(fd_c, float, double)
+#undef PP_X_FAST
 
-// Specialised z-transform for Nz in {16, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
-// returns cudaErrorNotSupported for other lengths.  [kx_lo, kx_hi): the kx columns transformed
+// Specialised z-transform for the Nz of the form 2^a 3^b from 16 to 1024 (but 972); returns
+// cudaErrorNotSupported for other lengths.  [kx_lo, kx_hi): the kx columns transformed
 // (kx_hi < 0: all; kx_lo a multiple of fft_z_fast_tile).
 template <typename T>
 cudaError_t launch_fft_z_fast(const Geometry& g, const Tables<T>& tt, int sign, cplx<T>* spec, cudaStream_t st,

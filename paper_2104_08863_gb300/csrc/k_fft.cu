@@ -145,9 +145,12 @@ cudaError_t launch_fwd_x(const Geometry& g, const DevTables& tb, const FftFactor
                          const FwdArgs& args, cplx<T>* spec, cudaStream_t st) {
   if (!g.generic_fft) {
     cudaError_t ef;
-    if constexpr (sizeof(T) == 8) ef = launch_fwd_x_fast_dd(g, tb, mode, args, (cplx<double>*)spec, st);
-    else if constexpr (sizeof(TI) == 4) ef = launch_fwd_x_fast_ff(g, tb, mode, args, (cplx<float>*)spec, st);
-    else ef = launch_fwd_x_fast_fd(g, tb, mode, args, (cplx<float>*)spec, st);
+#define PP_GROUPS(SFX, CALL)                                              \
+  if ((ef = SFX##_a CALL) == cudaErrorNotSupported &&                     \
+      (ef = SFX##_b CALL) == cudaErrorNotSupported) ef = SFX##_c CALL;
+    if constexpr (sizeof(T) == 8) { PP_GROUPS(launch_fwd_x_fast_dd, (g, tb, mode, args, (cplx<double>*)spec, st)) }
+    else if constexpr (sizeof(TI) == 4) { PP_GROUPS(launch_fwd_x_fast_ff, (g, tb, mode, args, (cplx<float>*)spec, st)) }
+    else { PP_GROUPS(launch_fwd_x_fast_fd, (g, tb, mode, args, (cplx<float>*)spec, st)) }
     if (ef != cudaErrorNotSupported) return ef;
   }
   const int nlines = g.ny * g.nz;
@@ -177,12 +180,17 @@ cudaError_t launch_inv_x(const Geometry& g, const DevTables& tb, const FftFactor
                          PairArgs pair) {
   if (!g.generic_fft) {
     cudaError_t ef;
-    if constexpr (sizeof(T) == 8)
-      ef = launch_inv_x_fast_dd(g, tb, mode, (const cplx<double>*)spec, (double*)out, scale, accumulate, st, pair);
-    else if constexpr (sizeof(TO) == 4)
-      ef = launch_inv_x_fast_ff(g, tb, mode, (const cplx<float>*)spec, (float*)out, scale, accumulate, st, pair);
-    else
-      ef = launch_inv_x_fast_fd(g, tb, mode, (const cplx<float>*)spec, (double*)out, scale, accumulate, st, pair);
+    if constexpr (sizeof(T) == 8) {
+      PP_GROUPS(launch_inv_x_fast_dd,
+                (g, tb, mode, (const cplx<double>*)spec, (double*)out, scale, accumulate, st, pair))
+    } else if constexpr (sizeof(TO) == 4) {
+      PP_GROUPS(launch_inv_x_fast_ff,
+                (g, tb, mode, (const cplx<float>*)spec, (float*)out, scale, accumulate, st, pair))
+    } else {
+      PP_GROUPS(launch_inv_x_fast_fd,
+                (g, tb, mode, (const cplx<float>*)spec, (double*)out, scale, accumulate, st, pair))
+    }
+#undef PP_GROUPS
     if (ef != cudaErrorNotSupported) return ef;
   }
   const int nlines = g.ny * g.nz;

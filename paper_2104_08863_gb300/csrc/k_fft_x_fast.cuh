@@ -1,5 +1,6 @@
-// Specialised x-transform kernels (steps (2) and (8) of Sec. 3.2) for the half-lengths
-// M = Nx/2 in {16, 32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024}.
+// Specialised x-transform kernels (steps (2) and (8) of Sec. 3.2) for the half-lengths M = Nx/2 of
+// the form 2^a 3^b from 8 to 1024 (but 864 and 972), instantiated in three groups of translation
+// units (k_fft_x_fast_*.cu).
 //
 // A CTA takes LPB consecutive x-lines, which are one contiguous stretch of the field, packs
 // each real line as M complex values, transforms all lines in place in padded shared memory
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
   if constexpr (sizeof(T) == 8) {
     // FP64: fused twiddles, two bins per item (the input carries the split's factor 1/2)
     fft_lf<T, M, -1, LPB, THREADS, 1, M, false>(buf, tt.lf_m);
-    constexpr int H = M / 2;
+    constexpr int H = (M + 1) / 2;
 #pragma unroll 4
     for (int idx = threadIdx.x; idx < LPB * H; idx += THREADS) {
       const int t = idx / H, kx = idx % H;
@@ -71,10 +72,12 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
       cplx<T>* X = spec + (size_t)line * g.pitch;
       const cplx<T> Zk = buf[padi<T>(t * M + kx)];
       if (kx == 0) {   // the real bins 0 and M, and the middle bin, whose partner is itself
-        const cplx<T> Zh = buf[padi<T>(t * M + H)];
         st_c(X, mk<T>(T(2) * (Zk.x + Zk.y), T(0)));
         st_c(X + M, mk<T>(T(2) * (Zk.x - Zk.y), T(0)));
-        st_c(X + H, mk<T>(T(2) * Zh.x, T(-2) * Zh.y));
+        if constexpr (M % 2 == 0) {
+          const cplx<T> Zh = buf[padi<T>(t * M + H)];
+          st_c(X + H, mk<T>(T(2) * Zh.x, T(-2) * Zh.y));
+        }
       } else {
         cplx<T> Xk, Xm;
         fwd_post_pair(Zk, buf[padi<T>(t * M + M - kx)], ldg_c(tt.lf_post + kx), Xk, Xm);
@@ -97,17 +100,17 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
   }
 }
 
-template <typename T, typename TO, int M, int MODE, bool ACC>
+template <typename T, typename TO, int M, int MODE>
 __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
     k_inv_x_fast(Geometry g, Tables<T> tt, const cplx<T>* __restrict__ spec, TO* __restrict__ out, double scl,
-                 int nlines, const double* __restrict__ dy, double* __restrict__ acc, PairArgs pair) {
+                 int nlines, PairArgs pair) {
   using C = XTile<T, M>;
   constexpr int LPB = C::LPB, THREADS = C::THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw);
   const int line0 = blockIdx.x * LPB;
   if constexpr (sizeof(T) == 8) {   // FP64: bins k and M - k loaded once and packed together
-    constexpr int H = M / 2;
+    constexpr int H = (M + 1) / 2;
     constexpr int PER = (LPB * H + THREADS - 1) / THREADS;
     cplx<T> Xk[PER], Xm[PER];
 #pragma unroll
@@ -129,9 +132,11 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
       const int line = line0 + t;
       if (idx >= LPB * H) continue;
       if (kx == 0) {
-        const cplx<T> Xh = line < nlines ? ld_c(spec + (size_t)line * g.pitch + H) : mk<T>(T(0), T(0));
         buf[padi<T>(t * M)] = mk<T>(Xk[q].x + Xm[q].x, Xk[q].x - Xm[q].x);
-        buf[padi<T>(t * M + H)] = mk<T>(T(2) * Xh.x, T(-2) * Xh.y);
+        if constexpr (M % 2 == 0) {
+          const cplx<T> Xh = line < nlines ? ld_c(spec + (size_t)line * g.pitch + H) : mk<T>(T(0), T(0));
+          buf[padi<T>(t * M + H)] = mk<T>(T(2) * Xh.x, T(-2) * Xh.y);
+        }
       } else {
         cplx<T> Zk, Zm;
         inv_pre_pair(Xk[q], Xm[q], ldg_c(tt.lf_post + kx), Zk, Zm);
@@ -166,7 +171,7 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
     fft_static<T, M, 1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
   }
   const T s = T(scl);
-  if constexpr (!ACC && MODE == INV_FINAL) {
+  if constexpr (MODE == INV_FINAL) {
     // refined pressure: the pair (hi, lo) of every element is loaded before any assembly
     constexpr int PER = (LPB * M + THREADS - 1) / THREADS;
     float2 h[PER], l[PER];
@@ -192,7 +197,7 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
       const size_t off = (size_t)line * g.nx + 2 * n;
       final_store(out + off, h[q], l[q], float(z.x * s), float(z.y * s));
     }
-  } else if constexpr (!ACC) {
+  } else {
 #pragma unroll 4
     for (int idx = threadIdx.x; idx < LPB * M; idx += THREADS) {
       const int t = idx / M, n = idx % M;
@@ -202,39 +207,6 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
       const size_t off = (size_t)line * g.nx + 2 * n;
       inv_store<T, TO, MODE>(out + off, off, z.x * s, z.y * s, pair);
     }
-  } else {
-    // one warp per line: the line's dy-weighted sum is reduced with compensated sums
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NWARPS = THREADS / 32;
-    double wsum = 0.0;
-    for (int t = warp; t < LPB; t += NWARPS) {
-      const int line = line0 + t;
-      if (line >= nlines) break;
-      T hs = T(0), hc = T(0);
-#pragma unroll 8
-      for (int n = lane; n < M; n += 32) {
-        const cplx<T> z = buf[padi<T>(t * M + n)];
-        const T x0 = z.x * s, x1 = z.y * s;
-        const size_t off = (size_t)line * g.nx + 2 * n;
-        inv_store<T, TO, MODE>(out + off, off, x0, x1, pair);
-        acc_add(hs, hc, x0);
-        acc_add(hs, hc, x1);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const T os = __shfl_xor_sync(0xffffffffu, hs, o), oc = __shfl_xor_sync(0xffffffffu, hc, o);
-        T e;
-        if constexpr (sizeof(T) == 4) {
-          two_sum(hs, os, hs, e);
-        } else {
-          hs += os;
-          e = T(0);
-        }
-        hc += oc + e;
-      }
-      if (lane == 0) wsum += dy[line / g.nz] * ((double)hs + (double)hc);
-    }
-    if (lane == 0 && wsum != 0.0) atomicAdd(acc + 1, wsum);
   }
 }
 
@@ -420,11 +392,11 @@ cudaError_t launch_fwd_x_stockham(const Geometry& g, const DevTables& tb, const 
     if ((e = set_smem(k, C::SMEM)) != cudaSuccess) return e;                            \
     k<<<grid, C::THREADS, C::SMEM, st>>>(g, fa, tt, tb, spec, nlines);                  \
   }
-  if constexpr (sizeof(T) == 4 && sizeof(TI) == 8 && M >= 256 && M != 384) {
+  if constexpr (sizeof(T) == 4 && sizeof(TI) == 8 && (M == 256 || M == 512 || M == 768 || M == 1024)) {
     // FP64 right-hand side into the FP32 spectrum: the input is the widest stream of the solve,
     // and keeping the next tile's lines in flight pays for the smaller CTA count (long lines:
-    // tiles of 2-8 lines; Nx/2 = 384 spills and keeps the single-tile kernel; FP32 inputs, half
-    // as wide, measured faster with the single-tile kernel)
+    // tiles of 2-8 lines; Nx/2 = 384 spills and keeps the single-tile kernel, as do the lengths
+    // with more factors of 3; FP32 inputs, half as wide, measured faster with the single-tile kernel)
     if (mode == FWD_PLAIN) {
       using P = XPipe<TI, M>;
       auto k = k_fwd_x_pipe<TI, M>;
@@ -471,22 +443,20 @@ cudaError_t launch_inv_x_stockham(const Geometry& g, const DevTables& tb, const 
   const int nlines = g.ny * g.nz;
   const dim3 grid((nlines + C::LPB - 1) / C::LPB);
   cudaError_t e = cudaSuccess;
-#define PP_INVF(MODEV, ACCV)                                                                     \
+#define PP_INVF(MODEV)                                                                           \
   {                                                                                              \
-    auto k = k_inv_x_fast<T, TO, M, MODEV, ACCV>;                                                \
+    auto k = k_inv_x_fast<T, TO, M, MODEV>;                                                      \
     if ((e = set_smem(k, C::SMEM)) != cudaSuccess) return e;                                     \
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, out, scale, nlines, tb.dy, tb.acc, pair); \
+    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, out, scale, nlines, pair);                 \
   }
+  // FP64 plans only store; the FP64 assembly of a refined solve is its last pass (nothing accumulated)
+  if (accumulate) return cudaErrorNotSupported;
   if constexpr (sizeof(T) == sizeof(TO)) {
-    if (mode == INV_FINAL) return cudaErrorNotSupported;
-    if (mode == INV_ACCUM) {
-      if (accumulate) PP_INVF(INV_ACCUM, true) else PP_INVF(INV_ACCUM, false)
-    } else {
-      if (accumulate) PP_INVF(INV_STORE, true) else PP_INVF(INV_STORE, false)
-    }
+    if (mode != INV_STORE) return cudaErrorNotSupported;
+    PP_INVF(INV_STORE)
   } else {
     if (mode != INV_FINAL) return cudaErrorNotSupported;
-    if (accumulate) PP_INVF(INV_FINAL, true) else PP_INVF(INV_FINAL, false)
+    PP_INVF(INV_FINAL)
   }
 #undef PP_INVF
   return cudaGetLastError();
@@ -503,33 +473,47 @@ cudaError_t launch_inv_x_m(const Geometry& g, const DevTables& tb, const Tables<
   }
 }
 
-#define PP_X_SIZES(F) F(16) F(32) F(48) F(64) F(96) F(128) F(192) F(256) F(384) F(512) F(768) F(1024)
+// The groups of half-lengths, one translation unit each per pair of types.
+#define PP_X_SIZES_A(F) F(8) F(9) F(12) F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64)
+#define PP_X_SIZES_B(F) F(72) F(81) F(96) F(108) F(128) F(144) F(162) F(192) F(216) F(243) F(256)
+#define PP_X_SIZES_C(F) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(1024)
 
-template <typename T, typename TI>
+#define PP_X_CASE_FWD(MV) \
+  case MV: return launch_fwd_x_m<T, TI, MV>(g, tb, tt, mode, args, spec, st);
+#define PP_X_CASE_INV(MV) \
+  case MV: return launch_inv_x_m<T, TO, MV>(g, tb, tt, mode, spec, out, scale, accumulate, st, pair);
+
+// cudaErrorNotSupported when group G (0, 1, 2) does not hold Nx/2.
+template <typename T, typename TI, int G>
 cudaError_t launch_fwd_x_fast_impl(const Geometry& g, const DevTables& tb, const Tables<T>& tt, FwdMode mode,
                                    const FwdArgs& args, cplx<T>* spec, cudaStream_t st) {
   // the per-line residual addresses its neighbour lines by 32-bit offsets
   if (mode == FWD_RESID && (long long)g.nx * g.nz >= (1LL << 31)) return cudaErrorNotSupported;
-  switch (g.M) {
-#define PP_CASE(MV) \
-  case MV: return launch_fwd_x_m<T, TI, MV>(g, tb, tt, mode, args, spec, st);
-    PP_X_SIZES(PP_CASE)
-#undef PP_CASE
-    default: return cudaErrorNotSupported;
+  if constexpr (G == 0) {
+    switch (g.M) { PP_X_SIZES_A(PP_X_CASE_FWD) }
+  } else if constexpr (G == 1) {
+    switch (g.M) { PP_X_SIZES_B(PP_X_CASE_FWD) }
+  } else {
+    switch (g.M) { PP_X_SIZES_C(PP_X_CASE_FWD) }
   }
+  return cudaErrorNotSupported;
 }
 
-template <typename T, typename TO>
+template <typename T, typename TO, int G>
 cudaError_t launch_inv_x_fast_impl(const Geometry& g, const DevTables& tb, const Tables<T>& tt, InvMode mode,
                                    const cplx<T>* spec, TO* out, double scale, bool accumulate, cudaStream_t st,
                                    PairArgs pair) {
-  switch (g.M) {
-#define PP_CASE(MV) \
-  case MV: return launch_inv_x_m<T, TO, MV>(g, tb, tt, mode, spec, out, scale, accumulate, st, pair);
-    PP_X_SIZES(PP_CASE)
-#undef PP_CASE
-    default: return cudaErrorNotSupported;
+  if constexpr (G == 0) {
+    switch (g.M) { PP_X_SIZES_A(PP_X_CASE_INV) }
+  } else if constexpr (G == 1) {
+    switch (g.M) { PP_X_SIZES_B(PP_X_CASE_INV) }
+  } else {
+    switch (g.M) { PP_X_SIZES_C(PP_X_CASE_INV) }
   }
+  return cudaErrorNotSupported;
 }
+
+#undef PP_X_CASE_FWD
+#undef PP_X_CASE_INV
 
 }  // namespace pp

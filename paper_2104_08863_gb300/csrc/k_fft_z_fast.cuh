@@ -6,6 +6,8 @@
 // about 256 threads: several are resident, so that one CTA's loads overlap another's arithmetic,
 // and a small grid still gives every SM one (2.15 ms at 512x384x512, 2.18 with 512 threads).  A launch may
 // cover only the kx columns [kx_lo, kx_hi) (one slab of the spectrum; kx_lo a multiple of W).
+#pragma once
+
 #include "fft_lf.cuh"
 #include "internal.h"
 #include "z_reg.cuh"
@@ -17,7 +19,7 @@ template <typename T, int NZ> struct ZTile {
   static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;             // 64-byte row segments
   static constexpr int W0 = (E * 256) / NZ;
   static constexpr int W = W0 < WMIN ? WMIN : (W0 > 32 ? 32 : W0);
-  static constexpr int T0 = W * NZ / E;
+  static constexpr int T0 = (W * NZ / E + 31) / 32 * 32;
   static constexpr int THREADS = T0 < 64 ? 64 : (T0 > 512 ? 512 : T0);
   static constexpr int SMEM = padded_size<T>(W * NZ) * (int)sizeof(cplx<T>);
   static constexpr int MINB = 512 / THREADS;   // 128 registers; several CTAs overlap memory and math
@@ -87,22 +89,30 @@ static cudaError_t launch_z_reg(const Geometry& g, const Tables<T>& tt, int sign
 template <typename T, int NZ>
 static cudaError_t launch_z(const Geometry& g, const Tables<T>& tt, int sign, cplx<T>* spec, cudaStream_t st,
                             int kx_lo, int kx_hi) {
-  if constexpr (sizeof(T) == 4) return launch_z_reg<T, NZ>(g, tt, sign, spec, st, kx_lo, kx_hi);
-  using C = ZTile<T, NZ>;
-  if (kx_lo % C::W || kx_lo < 0 || kx_hi > g.ncols || kx_hi <= kx_lo) return cudaErrorInvalidValue;
-  const dim3 grid((kx_hi - kx_lo + C::W - 1) / C::W, g.ny);
-  cudaError_t e;
-  if (sign < 0) {
-    auto k = k_fft_z_fast<T, NZ, -1>;
-    if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+  if constexpr (sizeof(T) == 4) {
+    return launch_z_reg<T, NZ>(g, tt, sign, spec, st, kx_lo, kx_hi);
   } else {
-    auto k = k_fft_z_fast<T, NZ, 1>;
-    if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+    using C = ZTile<T, NZ>;
+    if (kx_lo % C::W || kx_lo < 0 || kx_hi > g.ncols || kx_hi <= kx_lo) return cudaErrorInvalidValue;
+    const dim3 grid((kx_hi - kx_lo + C::W - 1) / C::W, g.ny);
+    cudaError_t e;
+    if (sign < 0) {
+      auto k = k_fft_z_fast<T, NZ, -1>;
+      if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
+      k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+    } else {
+      auto k = k_fft_z_fast<T, NZ, 1>;
+      if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
+      k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+    }
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
 }
+
+#define PP_Z_SIZES(F)                                                                                     \
+  F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64) F(72) F(81) F(96) F(108) F(128) F(144) F(162)     \
+  F(192) F(216) F(243) F(256) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(864) \
+  F(1024)
 
 // Returns cudaErrorNotSupported when Nz has no specialisation (the caller then uses the
 // generic kernel).  kx_hi < 0 means all columns.
@@ -113,8 +123,7 @@ cudaError_t launch_fft_z_fast(const Geometry& g, const Tables<T>& tt, int sign, 
   switch (g.nz) {
 #define PP_Z_CASE(NZ) \
     case NZ: return launch_z<T, NZ>(g, tt, sign, spec, st, kx_lo, kx_hi);
-    PP_Z_CASE(16) PP_Z_CASE(32) PP_Z_CASE(48) PP_Z_CASE(64) PP_Z_CASE(96) PP_Z_CASE(128) PP_Z_CASE(192)
-    PP_Z_CASE(256) PP_Z_CASE(384) PP_Z_CASE(512) PP_Z_CASE(768) PP_Z_CASE(1024)
+    PP_Z_SIZES(PP_Z_CASE)
 #undef PP_Z_CASE
     default: return cudaErrorNotSupported;
   }
@@ -126,18 +135,10 @@ int fft_z_fast_tile(const Geometry& g) {
   switch (g.nz) {
 #define PP_ZW_CASE(NZ) \
     case NZ: return sizeof(T) == 4 ? ZReg<T, NZ>::W : ZTile<T, NZ>::W;
-    PP_ZW_CASE(16) PP_ZW_CASE(32) PP_ZW_CASE(48) PP_ZW_CASE(64) PP_ZW_CASE(96) PP_ZW_CASE(128) PP_ZW_CASE(192)
-    PP_ZW_CASE(256) PP_ZW_CASE(384) PP_ZW_CASE(512) PP_ZW_CASE(768) PP_ZW_CASE(1024)
+    PP_Z_SIZES(PP_ZW_CASE)
 #undef PP_ZW_CASE
     default: return 0;
   }
 }
-
-template cudaError_t launch_fft_z_fast<float>(const Geometry&, const Tables<float>&, int, cplx<float>*, cudaStream_t,
-                                              int, int);
-template cudaError_t launch_fft_z_fast<double>(const Geometry&, const Tables<double>&, int, cplx<double>*,
-                                               cudaStream_t, int, int);
-template int fft_z_fast_tile<float>(const Geometry&);
-template int fft_z_fast_tile<double>(const Geometry&);
 
 }  // namespace pp

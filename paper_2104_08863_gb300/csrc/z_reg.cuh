@@ -1,5 +1,5 @@
 // Two-pass register z-transform (FP32): the tile function shared by the standalone kernel
-// (k_fft_z_fast.cu) and the persistent batched kernel (batch_persistent.cu).
+// (k_fft_z_fast.cuh) and the persistent batched kernel (batch_persistent.cu).
 #pragma once
 
 #include "fft_reg.cuh"
