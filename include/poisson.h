@@ -152,6 +152,17 @@ poisson_status poisson_divergence(poisson_plan_t plan, const void* u, const void
 poisson_status projection_step_adjoint(poisson_plan_t plan, void* gu, void* gv, void* gw,
                                        void* stream);
 
+/* The velocity maps of projection_step and projection_step_adjoint into other fields:
+ * (u_out, v_out, w_out) = P (u, v, w), v's wall faces copied, and g_out = P^T g.  The inputs are only
+ * read.  Every output must be another buffer than the inputs and the other outputs (PS_EINVAL);
+ * otherwise as the in-place calls, bit for bit.  PP_FP64 and PP_FP32 plans (PS_EUNSUPPORTED for
+ * PP_FP32_REFINED, whose projection needs its fields as scratch). */
+poisson_status projection_step_to(poisson_plan_t plan, const void* u, const void* v, const void* w,
+                                  void* u_out, void* v_out, void* w_out, double dt, void* stream);
+poisson_status projection_step_adjoint_to(poisson_plan_t plan, const void* gu, const void* gv,
+                                          const void* gw, void* gu_out, void* gv_out, void* gw_out,
+                                          void* stream);
+
 /* End-to-end variant of projection_step on HOST buffers: copies u, v, w to the device
  * staging buffers (caller-owned device memory of the field sizes), runs projection_step,
  * copies u, v, w (and p when p_host != NULL, using p_dev) back and synchronises `stream`.

@@ -386,21 +386,42 @@ def tune_batch(specs, precision=PP_FP32, fp64_low_modes=4, refine_steps=1, devic
     return best, times
 
 
+def _readable(plan: Plan, fields) -> bool:
+    """Whether the out-of-place kernels can read these fields as they are: what the plan's calls take
+    (checked there), at addresses that allow 16-byte accesses."""
+    return plan.precision != PP_FP32_REFINED and all(
+        t.is_cuda and t.dtype == plan.dtype and t.is_contiguous() and tuple(t.shape) == tuple(s)
+        and t.data_ptr() % 16 == 0 for t, s in zip(fields, (plan.cell_shape, plan.v_shape, plan.cell_shape)))
+
+
 class ProjectionFn(torch.autograd.Function):
-    """u = P(u*) (Eqs. 4, 7) with the hand-written adjoint backward P^T (same FFT/PDD kernels)."""
+    """u = P(u*) (Eqs. 4, 7) with the hand-written adjoint backward P^T (same FFT/PDD kernels).
+
+    Both read their arguments and write new tensors.  Arguments that the kernels cannot read in place
+    (another layout or alignment) are copied first, as before the in-place calls of a refined plan."""
 
     @staticmethod
     def forward(ctx, u, v, w, plan: Plan, dt: float):
         ctx.plan = plan
-        uo, vo, wo = u.detach().clone(), v.detach().clone(), w.detach().clone()
+        fields = [t.detach() for t in (u, v, w)]
+        if _readable(plan, fields):
+            out = [torch.empty_like(t) for t in fields]
+            check(_native.lib().projection_step_to(plan._h, *map(_ptr, fields), *map(_ptr, out), float(dt), _stream()),
+                  "projection_step_to")
+            return tuple(out)
+        uo, vo, wo = (t.clone() for t in fields)
         plan.project(uo, vo, wo, dt)
         return uo, vo, wo
 
     @staticmethod
     def backward(ctx, gu, gv, gw):
         plan = ctx.plan
-        gu = gu.detach().clone().contiguous()
-        gv = gv.detach().clone().contiguous()
-        gw = gw.detach().clone().contiguous()
+        fields = [t.detach() for t in (gu, gv, gw)]
+        if _readable(plan, fields):
+            out = [torch.empty_like(t) for t in fields]
+            check(_native.lib().projection_step_adjoint_to(plan._h, *map(_ptr, fields), *map(_ptr, out), _stream()),
+                  "projection_step_adjoint_to")
+            return (*out, None, None)
+        gu, gv, gw = (t.clone().contiguous() for t in fields)
         plan.project_adjoint(gu, gv, gw)
         return gu, gv, gw, None, None

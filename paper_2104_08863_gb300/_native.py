@@ -26,7 +26,8 @@ POISSON_BATCH_PERSISTENT = 0x10
 EXPORTS = (
     "poisson_plan_create", "poisson_workspace_size", "poisson_set_workspace", "poisson_solve",
     "poisson_solve_adjoint", "poisson_solve_static_ws", "poisson_plan_batched", "poisson_solve_batched", "poisson_autotune",
-    "projection_step", "projection_step_adjoint", "projection_step_host", "momentum_predictor",
+    "projection_step", "projection_step_adjoint", "projection_step_to", "projection_step_adjoint_to",
+    "projection_step_host", "momentum_predictor",
     "projection_timestep", "projection_timestep_host", "poisson_divergence", "poisson_plan_set_chain",
     "poisson_fp64_fma_rate", "poisson_device_status",
     "poisson_last_launch_count", "poisson_stage_times", "poisson_plan_destroy", "poisson_status_string",
@@ -74,6 +75,8 @@ def lib() -> ctypes.CDLL:
                                    ctypes.POINTER(ctypes.c_float)]
     L.projection_step.argtypes = [vp, vp, vp, vp, vp, d, vp]
     L.projection_step_adjoint.argtypes = [vp, vp, vp, vp, vp]
+    L.projection_step_to.argtypes = [vp, vp, vp, vp, vp, vp, vp, d, vp]
+    L.projection_step_adjoint_to.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp]
     L.projection_step_host.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, vp, d, vp]
     L.momentum_predictor.argtypes = [vp, vp, vp, vp, vp, vp, vp, d, d, d, vp]
     L.projection_timestep.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, d, d, d, vp]
@@ -91,7 +94,8 @@ def lib() -> ctypes.CDLL:
     L.poisson_status_string.restype = ctypes.c_char_p
     for name in ("poisson_plan_create", "poisson_workspace_size", "poisson_set_workspace", "poisson_solve",
                  "poisson_solve_adjoint", "poisson_solve_static_ws", "poisson_plan_batched", "poisson_solve_batched", "poisson_autotune",
-                 "projection_step", "projection_step_adjoint", "projection_step_host", "momentum_predictor",
+                 "projection_step", "projection_step_adjoint", "projection_step_to", "projection_step_adjoint_to",
+                 "projection_step_host", "momentum_predictor",
                  "projection_timestep", "projection_timestep_host", "poisson_divergence", "poisson_plan_set_chain",
                  "poisson_fp64_fma_rate", "poisson_device_status",
                  "poisson_plan_destroy"):

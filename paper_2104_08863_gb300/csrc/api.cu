@@ -627,28 +627,54 @@ poisson_status solve_impl(Exec& ex, const void* rhs, void* p, bool pair_out = fa
   return PS_OK;
 }
 
-// Eqs. 4 and 7 on u, v, w in place (validated by the caller): divergence fused into the forward
-// x-transform, the solve, the gradient correction.
-poisson_status projection_impl(Exec& ex, void* u, void* v, void* w, void* p_out, double dt) {
+// Eqs. 4 and 7 on u, v, w (validated by the caller) into uo, vo, wo, which may be u, v, w: divergence
+// fused into the forward x-transform, the solve, the gradient correction.
+template <typename T>
+poisson_status projection_fields(Exec& ex, const T* u, const T* v, const T* w, T* uo, T* vo, T* wo, T* p_out,
+                                 double dt) {
   const poisson_plan_s* pl = ex.pl;
   cudaStream_t st = ex.st;
   FwdArgs args = {};
   args.u = u; args.v = v; args.w = w;
   args.in_scale = 1.0 / dt;
-  if (pl->precision == PP_FP64) {
-    double* p = p_out ? (double*)p_out : (double*)(pl->ws + pl->off_pbuf);
-    PP_RET(check_finite_uvw<double>(ex, u, v, w));
-    PP_RET((forward_and_core<double, double>(ex, FWD_DIV, args, GAUGE_ZERO)));
-    PP_RET((inverse_x<double, double>(ex, INV_STORE, p, false)));
-    PP_TRY_N("gradient", launch_gradient<double>(pl->g, ex.dt, p, (double*)u, (double*)v, (double*)w, dt, st));
-  } else {
-    float* p = p_out ? (float*)p_out : (float*)(pl->ws + pl->off_pbuf);
-    PP_RET(check_finite_uvw<float>(ex, u, v, w));
-    PP_RET((forward_and_core<float, float>(ex, FWD_DIV, args, GAUGE_ZERO)));
-    PP_RET((inverse_x<float, float>(ex, INV_STORE, p, false)));
-    PP_TRY_N("gradient", launch_gradient<float>(pl->g, ex.dt, p, (float*)u, (float*)v, (float*)w, dt, st));
-  }
+  T* p = p_out ? p_out : (T*)(pl->ws + pl->off_pbuf);
+  PP_RET(check_finite_uvw<T>(ex, u, v, w));
+  PP_RET((forward_and_core<T, T>(ex, FWD_DIV, args, GAUGE_ZERO)));
+  PP_RET((inverse_x<T, T>(ex, INV_STORE, p, false)));
+  PP_TRY_N("gradient", launch_gradient<T>(pl->g, ex.dt, p, u, v, w, uo, vo, wo, dt, st));
   return PS_OK;
+}
+
+poisson_status projection_impl(Exec& ex, const void* u, const void* v, const void* w, void* uo, void* vo, void* wo,
+                               void* p_out, double dt) {
+  if (ex.pl->precision == PP_FP64)
+    return projection_fields<double>(ex, (const double*)u, (const double*)v, (const double*)w, (double*)uo,
+                                     (double*)vo, (double*)wo, (double*)p_out, dt);
+  return projection_fields<float>(ex, (const float*)u, (const float*)v, (const float*)w, (float*)uo, (float*)vo,
+                                  (float*)wo, (float*)p_out, dt);
+}
+
+// g - D^T S^T G^T g of gu, gv, gw into uo, vo, wo, which may be gu, gv, gw.
+template <typename T>
+poisson_status adjoint_fields(Exec& ex, const T* gu, const T* gv, const T* gw, T* uo, T* vo, T* wo) {
+  const poisson_plan_s* pl = ex.pl;
+  cudaStream_t st = ex.st;
+  FwdArgs args = {};
+  args.u = gu; args.v = gv; args.w = gw;
+  args.in_scale = 1.0;
+  T* q = (T*)(pl->ws + pl->off_pbuf);
+  PP_RET((forward_and_core<T, T>(ex, FWD_GRADT, args, GAUGE_ZERO)));
+  PP_RET((inverse_x<T, T>(ex, INV_STORE, q, false)));
+  PP_TRY_N("adj_epilogue", launch_adjoint_epilogue<T>(pl->g, ex.dt, q, gu, gv, gw, uo, vo, wo, st));
+  return PS_OK;
+}
+
+poisson_status adjoint_impl(Exec& ex, const void* gu, const void* gv, const void* gw, void* uo, void* vo, void* wo) {
+  if (ex.pl->precision == PP_FP64)
+    return adjoint_fields<double>(ex, (const double*)gu, (const double*)gv, (const double*)gw, (double*)uo,
+                                  (double*)vo, (double*)wo);
+  return adjoint_fields<float>(ex, (const float*)gu, (const float*)gv, (const float*)gw, (float*)uo, (float*)vo,
+                               (float*)wo);
 }
 
 // The projection of PP_FP32_REFINED plans (Eqs. 4 and 7) without per-point FP64 arithmetic:
@@ -808,7 +834,7 @@ poisson_status timestep_overlapped(poisson_plan_s* pl, const void* u_h, const vo
           cudaMemcpyAsync((T*)p_h + o, p + o, cells(c) * sizeof(T), cudaMemcpyDeviceToHost, cp) != cudaSuccess)
         return PS_ECUDA;
     }
-    PP_TRY_N("gradient", launch_gradient<T>(g, ex.dt, p, u, v, w, dt, st, rows[c], rows[c + 1]));
+    PP_TRY_N("gradient", launch_gradient<T>(g, ex.dt, p, u, v, w, u, v, w, dt, st, rows[c], rows[c + 1]));
     if (cudaEventRecord(ev_g[c], st) != cudaSuccess || cudaStreamWaitEvent(cp, ev_g[c], 0) != cudaSuccess)
       return PS_ECUDA;
     if (cudaMemcpyAsync((T*)u_h + o, u + o, cells(c) * sizeof(T), cudaMemcpyDeviceToHost, cp) != cudaSuccess ||
@@ -903,7 +929,46 @@ poisson_status projection_step(poisson_plan_t pl, void* u, void* v, void* w, voi
   pl->nev = 0;
   Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
   if (pl->precision == PP_FP32_REFINED) return projection_pairs(ex, u, v, w, p_out, dt);
-  return projection_impl(ex, u, v, w, p_out, dt);
+  return projection_impl(ex, u, v, w, u, v, w, p_out, dt);
+}
+
+// The arguments of the two out-of-place forms: aligned fields, every output another field than every
+// input and every other output.
+static poisson_status check_to_args(const poisson_plan_s* pl, const void* const in[3], void* const out[3]) {
+  if (!pl) return PS_EINVAL;
+  for (int a = 0; a < 3; ++a)
+    if (!in[a] || !out[a]) return PS_EINVAL;
+  if (!pl->children.empty()) return PS_EINVAL;
+  if (!pl->ws) return PS_ENOWORKSPACE;
+  for (int a = 0; a < 3; ++a) {
+    if (!aligned16(in[a]) || !aligned16(out[a])) return PS_EINVAL;
+    for (int b = 0; b < 3; ++b)
+      if (in[b] == out[a] || (b < a && out[b] == out[a])) return PS_EINVAL;
+  }
+  return pl->precision == PP_FP32_REFINED ? PS_EUNSUPPORTED : PS_OK;
+}
+
+poisson_status projection_step_to(poisson_plan_t pl, const void* u, const void* v, const void* w, void* uo, void* vo,
+                                  void* wo, double dt, void* stream) {
+  const void* in[3] = {u, v, w};
+  void* out[3] = {uo, vo, wo};
+  PP_RET(check_to_args(pl, in, out));
+  if (!(dt > 0.0) || !isfinite(dt)) return PS_EINVAL;
+  pl->launches = 0;
+  pl->nev = 0;
+  Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
+  return projection_impl(ex, u, v, w, uo, vo, wo, nullptr, dt);
+}
+
+poisson_status projection_step_adjoint_to(poisson_plan_t pl, const void* gu, const void* gv, const void* gw,
+                                          void* uo, void* vo, void* wo, void* stream) {
+  const void* in[3] = {gu, gv, gw};
+  void* out[3] = {uo, vo, wo};
+  PP_RET(check_to_args(pl, in, out));
+  pl->launches = 0;
+  pl->nev = 0;
+  Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
+  return adjoint_impl(ex, gu, gv, gw, uo, vo, wo);
 }
 
 poisson_status momentum_predictor(poisson_plan_t pl, void* u, void* v, void* w, void* ub, void* vb, void* wb,
@@ -926,7 +991,7 @@ poisson_status projection_timestep(poisson_plan_t pl, void* u, void* v, void* w,
   Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
   if (pl->precision != PP_FP32_REFINED) {
     PP_RET(predictor_impl(ex, u, v, w, ub, vb, wb, dt, nu, fx));
-    return projection_impl(ex, u, v, w, p_out, dt);
+    return projection_impl(ex, u, v, w, u, v, w, p_out, dt);
   }
   // refined: u_star as pairs; f = D(u_star)/dt into ub (FP64); the refined solve into p_out or
   // vb; then the FP64 correction u = u_star - dt G p written over the pairs
@@ -950,24 +1015,7 @@ poisson_status projection_step_adjoint(poisson_plan_t pl, void* gu, void* gv, vo
   pl->launches = 0;
   pl->nev = 0;
   Exec ex{pl, pl->ws, pl->dt, (cudaStream_t)stream, (pl->flags & POISSON_TIMING) != 0};
-  cudaStream_t st = ex.st;
-  FwdArgs args = {};
-  args.u = gu; args.v = gv; args.w = gw;
-  args.in_scale = 1.0;
-  if (pl->precision == PP_FP64) {
-    double* q = (double*)(pl->ws + pl->off_pbuf);
-    PP_RET((forward_and_core<double, double>(ex, FWD_GRADT, args, GAUGE_ZERO)));
-    PP_RET((inverse_x<double, double>(ex, INV_STORE, q, false)));
-    PP_TRY_N("adj_epilogue",
-             launch_adjoint_epilogue<double>(pl->g, ex.dt, q, (double*)gu, (double*)gv, (double*)gw, st));
-  } else {
-    float* q = (float*)(pl->ws + pl->off_pbuf);
-    PP_RET((forward_and_core<float, float>(ex, FWD_GRADT, args, GAUGE_ZERO)));
-    PP_RET((inverse_x<float, float>(ex, INV_STORE, q, false)));
-    PP_TRY_N("adj_epilogue",
-             launch_adjoint_epilogue<float>(pl->g, ex.dt, q, (float*)gu, (float*)gv, (float*)gw, st));
-  }
-  return PS_OK;
+  return adjoint_impl(ex, gu, gv, gw, gu, gv, gw);
 }
 
 poisson_status projection_step_host(poisson_plan_t pl, void* u_h, void* v_h, void* w_h, void* p_h, void* u_d,

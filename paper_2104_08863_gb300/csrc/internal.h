@@ -180,13 +180,15 @@ SideArgs side_args(const DevTables& tb, int low, GaugeMode gauge);
 // Their FP64 pivots tb.low_rb (once per plan; low >= 1).
 cudaError_t launch_low_setup(const Geometry& g, const DevTables& tb, int low, cudaStream_t st);
 
+// (uo, vo, wo) = (u, v, w) - dt G p on the rows [jlo, jhi), in place when they are the same fields;
+// otherwise v's wall faces are copied with the first and the last row.
 template <typename T>
-cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, T* u, T* v, T* w, double dt,
-                            cudaStream_t st, int jlo = 0, int jhi = -1);   // rows [jlo, jhi) (+ the top wall faces)
+cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, const T* u, const T* v, const T* w,
+                            T* uo, T* vo, T* wo, double dt, cudaStream_t st, int jlo = 0, int jhi = -1);
 
 template <typename T>
-cudaError_t launch_adjoint_epilogue(const Geometry& g, const DevTables& tb, const T* q, T* gu, T* gv, T* gw,
-                                    cudaStream_t st);
+cudaError_t launch_adjoint_epilogue(const Geometry& g, const DevTables& tb, const T* q, const T* gu, const T* gv,
+                                    const T* gw, T* uo, T* vo, T* wo, cudaStream_t st);
 
 // out = in * (1/dy_j) or in * dy_j per y-plane j (in == out allowed), and q = dy_j (hi + lo) in FP64.
 template <typename T>

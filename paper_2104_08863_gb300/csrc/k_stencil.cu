@@ -71,40 +71,50 @@ __device__ __forceinline__ PNeigh<T, V> pload(const Geometry& g, const T* __rest
   return n;
 }
 
-// Lines [lbeg, lend) of the ny nz cell lines (line = j nz + k).
+// Lines [lbeg, lend) of the ny nz cell lines (line = j nz + k), or of the (ny + 1) nz face lines when
+// the result goes to other fields than (u, v, w) and v's wall faces are copied.  Each point of in and
+// out belongs to one thread, which reads it before it writes it, so they may be the same fields.
+template <typename T> struct Faces3 { T *u, *v, *w; };
 template <typename T, int V>
-__global__ void __launch_bounds__(STENCIL_THREADS) k_gradient(Geometry g, const T* __restrict__ p, T* __restrict__ u,
-                                                              T* __restrict__ v, T* __restrict__ w,
+__global__ void __launch_bounds__(STENCIL_THREADS) k_gradient(Geometry g, const T* __restrict__ p,
+                                                              Faces3<const T> in, Faces3<T> out,
                                                               const T* __restrict__ inv_h, T dt, T cx, T cz, int lbeg,
                                                               int lend) {
   const int line = lbeg + blockIdx.x * blockDim.y + threadIdx.y;
   if (line >= lend) return;
   const int j = line / g.nz, k = line - j * g.nz;
-  const bool inner = j >= 1;   // v's wall faces are boundary values
+  const bool cell = j < g.ny, inner = cell && j >= 1;   // v's wall faces are boundary values
+  const bool copy = out.v != in.v;
   const T cy = inner ? dt * inv_h[j] : T(0);
   for (int i0 = threadIdx.x * V; i0 < g.nx; i0 += blockDim.x * V) {
     const size_t idx = (size_t)line * g.nx + i0;
-    const PNeigh<T, V> n = pload<T, V>(g, p, j, k, idx, i0, true, inner);
-    Vec<T, V> uu = vload<T, V>(u + idx), ww = vload<T, V>(w + idx), vv;
-    if (inner) vv = vload<T, V>(v + idx);
-#pragma unroll
-    for (int q = 0; q < V; ++q) {
-      uu.x[q] -= cx * (n.c.x[q] - n.xm.x[q]);
-      ww.x[q] -= cz * (n.c.x[q] - n.zm.x[q]);
+    const PNeigh<T, V> n = pload<T, V>(g, p, j, k, idx, i0, cell, inner);
+    Vec<T, V> uu, ww, vv;
+    if (cell) {
+      uu = vload<T, V>(in.u + idx);
+      ww = vload<T, V>(in.w + idx);
     }
-    vstore<T, V>(u + idx, uu);
-    vstore<T, V>(w + idx, ww);
+    if (inner || copy) vv = vload<T, V>(in.v + idx);
+    if (cell) {
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        uu.x[q] -= cx * (n.c.x[q] - n.xm.x[q]);
+        ww.x[q] -= cz * (n.c.x[q] - n.zm.x[q]);
+      }
+      vstore<T, V>(out.u + idx, uu);
+      vstore<T, V>(out.w + idx, ww);
+    }
     if (inner) {
 #pragma unroll
       for (int q = 0; q < V; ++q) vv.x[q] -= cy * (n.c.x[q] - n.ym.x[q]);
-      vstore<T, V>(v + idx, vv);
     }
+    if (inner || copy) vstore<T, V>(out.v + idx, vv);
   }
 }
 
 template <typename T, int V>
-__global__ void __launch_bounds__(STENCIL_THREADS) k_adj_epi(Geometry g, const T* __restrict__ pp_, T* __restrict__ gu,
-                                                             T* __restrict__ gv, T* __restrict__ gw,
+__global__ void __launch_bounds__(STENCIL_THREADS) k_adj_epi(Geometry g, const T* __restrict__ pp_,
+                                                             Faces3<const T> in, Faces3<T> out,
                                                              const double* __restrict__ dy, T ix, T iz) {
   const int line = blockIdx.x * blockDim.y + threadIdx.y;
   if (line >= (g.ny + 1) * g.nz) return;
@@ -114,17 +124,17 @@ __global__ void __launch_bounds__(STENCIL_THREADS) k_adj_epi(Geometry g, const T
   for (int i0 = threadIdx.x * V; i0 < g.nx; i0 += blockDim.x * V) {
     const size_t idx = (size_t)line * g.nx + i0;
     const PNeigh<T, V> n = pload<T, V>(g, pp_, j, k, idx, i0, cell, below);
-    Vec<T, V> vv = vload<T, V>(gv + idx), uu, ww;
+    Vec<T, V> vv = vload<T, V>(in.v + idx), uu, ww;
     if (cell) {
-      uu = vload<T, V>(gu + idx);
-      ww = vload<T, V>(gw + idx);
+      uu = vload<T, V>(in.u + idx);
+      ww = vload<T, V>(in.w + idx);
 #pragma unroll
       for (int q = 0; q < V; ++q) {
         uu.x[q] -= dyj * (n.xm.x[q] - n.c.x[q]) * ix;
         ww.x[q] -= dyj * (n.zm.x[q] - n.c.x[q]) * iz;
       }
-      vstore<T, V>(gu + idx, uu);
-      vstore<T, V>(gw + idx, ww);
+      vstore<T, V>(out.u + idx, uu);
+      vstore<T, V>(out.w + idx, ww);
     }
     // (D_y^T q)_f = q_{f-1}/dy_{f-1} - q_f/dy_f = p'_{f-1} - p'_f  (terms outside 0..ny-1 vanish)
 #pragma unroll
@@ -134,7 +144,7 @@ __global__ void __launch_bounds__(STENCIL_THREADS) k_adj_epi(Geometry g, const T
       if (cell) t -= n.c.x[q];
       vv.x[q] -= t;
     }
-    vstore<T, V>(gv + idx, vv);
+    vstore<T, V>(out.v + idx, vv);
   }
 }
 
@@ -233,31 +243,35 @@ static LineTiles line_tiles(const Geometry& g, int V, int nlines) {
 template <typename T> static bool wide_vectors(const Geometry& g) { return g.nx % (16 / (int)sizeof(T)) == 0; }
 
 template <typename T>
-cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, T* u, T* v, T* w, double dt,
-                            cudaStream_t st, int jlo, int jhi) {
+cudaError_t launch_gradient(const Geometry& g, const DevTables& tb, const T* p, const T* u, const T* v, const T* w,
+                            T* uo, T* vo, T* wo, double dt, cudaStream_t st, int jlo, int jhi) {
   if (jhi < 0) jhi = g.ny;
   if (jlo < 0 || jhi > g.ny || jhi <= jlo) return cudaErrorInvalidValue;
-  const int lbeg = jlo * g.nz, lend = jhi * g.nz;
+  const int lbeg = jlo * g.nz, lend = (jhi == g.ny && vo != v ? g.ny + 1 : jhi) * g.nz;
   constexpr int VW = 16 / (int)sizeof(T);
   const int V = wide_vectors<T>(g) ? VW : 2;
   const LineTiles t = line_tiles(g, V, lend - lbeg);
   // dt/dx and dt/dz once on the host: two FP64 divisions per thread took as long as its traffic
   const T d = T(dt), cx = T(d / g.dx), cz = T(d / g.dz);
   const T* ih = inv_h_table<T>(tb);
-  if (V == VW) k_gradient<T, VW><<<t.grid, t.block, 0, st>>>(g, p, u, v, w, ih, d, cx, cz, lbeg, lend);
-  else k_gradient<T, 2><<<t.grid, t.block, 0, st>>>(g, p, u, v, w, ih, d, cx, cz, lbeg, lend);
+  const Faces3<const T> in{u, v, w};
+  const Faces3<T> out{uo, vo, wo};
+  if (V == VW) k_gradient<T, VW><<<t.grid, t.block, 0, st>>>(g, p, in, out, ih, d, cx, cz, lbeg, lend);
+  else k_gradient<T, 2><<<t.grid, t.block, 0, st>>>(g, p, in, out, ih, d, cx, cz, lbeg, lend);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_adjoint_epilogue(const Geometry& g, const DevTables& tb, const T* q, T* gu, T* gv, T* gw,
-                                    cudaStream_t st) {
+cudaError_t launch_adjoint_epilogue(const Geometry& g, const DevTables& tb, const T* q, const T* gu, const T* gv,
+                                    const T* gw, T* uo, T* vo, T* wo, cudaStream_t st) {
   constexpr int VW = 16 / (int)sizeof(T);
   const int V = wide_vectors<T>(g) ? VW : 2;
   const LineTiles t = line_tiles(g, V, (g.ny + 1) * g.nz);
   const T ix = T(g.inv_dx), iz = T(g.inv_dz);
-  if (V == VW) k_adj_epi<T, VW><<<t.grid, t.block, 0, st>>>(g, q, gu, gv, gw, tb.dy, ix, iz);
-  else k_adj_epi<T, 2><<<t.grid, t.block, 0, st>>>(g, q, gu, gv, gw, tb.dy, ix, iz);
+  const Faces3<const T> in{gu, gv, gw};
+  const Faces3<T> out{uo, vo, wo};
+  if (V == VW) k_adj_epi<T, VW><<<t.grid, t.block, 0, st>>>(g, q, in, out, tb.dy, ix, iz);
+  else k_adj_epi<T, 2><<<t.grid, t.block, 0, st>>>(g, q, in, out, tb.dy, ix, iz);
   return cudaGetLastError();
 }
 
@@ -295,14 +309,14 @@ cudaError_t launch_check_finite(const T* x, size_t n, int* status, cudaStream_t 
   return cudaGetLastError();
 }
 
-template cudaError_t launch_gradient<double>(const Geometry&, const DevTables&, const double*, double*, double*,
-                                             double*, double, cudaStream_t, int, int);
-template cudaError_t launch_gradient<float>(const Geometry&, const DevTables&, const float*, float*, float*, float*,
-                                            double, cudaStream_t, int, int);
-template cudaError_t launch_adjoint_epilogue<double>(const Geometry&, const DevTables&, const double*, double*,
-                                                     double*, double*, cudaStream_t);
-template cudaError_t launch_adjoint_epilogue<float>(const Geometry&, const DevTables&, const float*, float*, float*,
-                                                    float*, cudaStream_t);
+#define PP_FACES_INST(T)                                                                                          \
+  template cudaError_t launch_gradient<T>(const Geometry&, const DevTables&, const T*, const T*, const T*,        \
+                                          const T*, T*, T*, T*, double, cudaStream_t, int, int);                  \
+  template cudaError_t launch_adjoint_epilogue<T>(const Geometry&, const DevTables&, const T*, const T*, const T*, \
+                                                  const T*, T*, T*, T*, cudaStream_t);
+PP_FACES_INST(double)
+PP_FACES_INST(float)
+#undef PP_FACES_INST
 template cudaError_t launch_scale_planes<double>(const Geometry&, const DevTables&, const double*, double*, bool,
                                                  cudaStream_t);
 template cudaError_t launch_scale_planes<float>(const Geometry&, const DevTables&, const float*, float*, bool,
