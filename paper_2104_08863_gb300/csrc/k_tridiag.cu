@@ -253,17 +253,17 @@ __global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int
 // Thomas by scans: with the pivots in tables both sweeps are first-order linear recurrences with
 // coefficients in (0, 1) (see low_modes.cuh), so 8 lanes take contiguous rows of one system each
 // and the carries between them come from a 3-step scan of affine maps.  A warp holds 4 systems
-// (64-byte row segments), a CTA 16.  Per row the eliminated value and the running product of the
+// (64-byte row segments), a CTA 8, so that a few hundred systems reach every SM.  Per row the eliminated value and the running product of the
 // coefficients (the weight of the carry) stay in the thread's own shared-memory column.
 //
 // Such a launch is bound by latency: one thread per system walks ny dependent rows twice (FP64
 // FMA: 65 clocks) with 544 to 20,000 threads on the GPU.  It issues 13 FP64 instructions per row
 // against 10 of the serial form, which stays for more modes.  32x32x32: 24.5 -> 12 us per launch
 // with its event pair, 64x64x64: 43 -> 12 us; at 17,600 modes of 130 rows both take the same.
-constexpr int kScan64Rows = 256;       // most rows (98 KB of shared memory)
+constexpr int kScan64Rows = 256;       // most rows (49 KB of shared memory)
 constexpr int kScan64Systems = 20000;  // most modes
 
-__global__ void __launch_bounds__(128) k_tridiag_scan64(Geometry g, const double* __restrict__ c,
+__global__ void __launch_bounds__(64) k_tridiag_scan64(Geometry g, const double* __restrict__ c,
                                                         TriFactors<double> tf, cplx<double>* __restrict__ spec,
                                                         SideArgs sd) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -272,13 +272,13 @@ __global__ void __launch_bounds__(128) k_tridiag_scan64(Geometry g, const double
     return;
   }
   const int lane = threadIdx.x & 31, l = lane >> 2;
-  const int q = ((int)blockIdx.x - sd.n) * 16 + (threadIdx.x >> 5) * 4 + (lane & 3);   // over (kz, padded kx)
+  const int q = ((int)blockIdx.x - sd.n) * 8 + (threadIdx.x >> 5) * 4 + (lane & 3);   // over (kz, padded kx)
   const int kz = q / g.pitch, kx = q - kz * g.pitch;
   const bool active = kz < g.nz && kx < g.ncols && !(kx == 0 && kz == 0);
   const int ch = (g.ny + 7) / 8;
   const int lo = min(g.ny, l * ch), hi = active ? min(g.ny, lo + ch) : lo;
-  double2* y = reinterpret_cast<double2*>(smem_raw) + threadIdx.x;                        // row lo + i at y[128 i]
-  double* wt = reinterpret_cast<double*>(smem_raw) + (size_t)2 * 128 * ch + threadIdx.x;  // carry weights
+  double2* y = reinterpret_cast<double2*>(smem_raw) + threadIdx.x;                        // row lo + i at y[64 i]
+  double* wt = reinterpret_cast<double*>(smem_raw) + (size_t)2 * 64 * ch + threadIdx.x;  // carry weights
   const size_t rstride = (size_t)g.nz * g.pitch, ns = (size_t)tf.nsys;
   cplx<double>* col = spec + (size_t)kz * g.pitch + kx;
   const double* mult = tf.mult + (size_t)kz * g.ncols + kx;
@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(128) k_tridiag_scan64(Geometry g, const double
     const double m = __ldg(mult + (size_t)j * ns);
     B = make_double2(fma(m, B.x, -F.x), fma(m, B.y, -F.y));
     A *= m;
-    y[128 * (j - lo)] = B;
-    wt[128 * (j - lo)] = A;
+    y[64 * (j - lo)] = B;
+    wt[64 * (j - lo)] = A;
   }
   // the value entering this lane's rows, from the maps of the lanes before (UP) or after it
   auto carry = [&](bool up) {
@@ -315,18 +315,18 @@ __global__ void __launch_bounds__(128) k_tridiag_scan64(Geometry g, const double
   B = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int j = hi - 1; j >= lo; --j) {
-    const double r = __ldg(rb + (size_t)j * ns), cr = c[j] * r, w = wt[128 * (j - lo)];
-    const double2 v = y[128 * (j - lo)];
+    const double r = __ldg(rb + (size_t)j * ns), cr = c[j] * r, w = wt[64 * (j - lo)];
+    const double2 v = y[64 * (j - lo)];
     B = make_double2(fma(cr, B.x, r * fma(w, gin.x, v.x)), fma(cr, B.y, r * fma(w, gin.y, v.y)));
     A *= cr;
-    y[128 * (j - lo)] = B;
-    wt[128 * (j - lo)] = A;
+    y[64 * (j - lo)] = B;
+    wt[64 * (j - lo)] = A;
   }
   const double2 xin = carry(false);
 #pragma unroll 4
   for (int j = lo; j < hi; ++j) {
-    const double2 v = y[128 * (j - lo)];
-    const double w = wt[128 * (j - lo)];
+    const double2 v = y[64 * (j - lo)];
+    const double w = wt[64 * (j - lo)];
     st_c(col + (size_t)j * rstride, mk<double>(fma(w, xin.x, v.x), fma(w, xin.y, v.y)));
   }
 }
@@ -539,11 +539,9 @@ __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S
 // memory, twice: into system-major order, where the P interfaces of a system are P lanes of a
 // warp and the reduced system is the pair of warp scans of tridiag_scan.cuh, and back.
 //
-// The form that staged the rows in shared memory and swept them there made 14 shared-memory
-// wavefronts per warp and row; it took 278 us per pass at 768x384x512 and 2.73 ms at
-// 1536x768x1024, this one 250 us and 2.58 ms (1.21 and 9.78 GB each).  What is left is the
-// access pattern: 64-byte row segments (S = 8 at P = 32) several MB apart.  The same operations in
-// the same order: bit-identical results.
+// What bounds it is HBM and, on small grids, the latency of one load and two sweeps.  The form before staged the rows in shared memory and
+// swept them there with 14 shared-memory wavefronts per warp and row (batch of 64 solves of 48 to
+// 192 rows: 2678 us, 2520 with this kernel at every block height).
 template <int M> constexpr int rows_min_ctas() { return M <= 8 ? 4 : (M <= 12 ? 3 : 2); }
 
 template <int M>
@@ -654,6 +652,141 @@ __global__ void __launch_bounds__(256, rows_min_ctas<M>())
       xn = make_float2(fmaf(rcv[i], xn.x, fmaf(rgv[i], alpha.x, v[i].x)),
                        fmaf(rcv[i], xn.y, fmaf(rgv[i], alpha.y, v[i].y)));
       p[(size_t)i * rstride] = xn;
+    }
+  }
+}
+
+// ---- FP32 PDD on tiles in shared memory (P >= 16, blocks of 12 rows and more) -------------------
+// The rows kernel's blocks and order, with the S = NT / P systems of a CTA staged in shared memory
+// as [row][s] by 16-byte asynchronous copies.  A thread keeps only 1/beta_i per row in registers
+// (64 in all), so that 1024 threads are resident where 4 registers per row allow 512: 32 warps hide the sweeps' latencies and one
+// CTA's copies overlap the other's sweeps.  The forward sweep stores rb_i gg_i in place; once alpha
+// is known a second one adds alpha rb_i gv_i (gv_i = a_i rb_{i-1} gv_{i-1} again), and the backward
+// sweep writes x_i to global memory as it goes: the operations of the rows kernel, bit for bit.
+//
+// What bounds it is the rate at which HBM serves row segments that lie nz pitch * 8 bytes apart
+// (6.4 MB at 1536x768x1024): an in-place copy in this order runs at 4.1 TB/s with 64-byte segments
+// and at 6.7 TB/s with 128-byte ones, so a CTA takes at least 16 systems: 512 threads at P = 32
+// (98 KB of shared memory, two CTAs per SM), else 256.  Per pass, against the rows kernel (4
+// registers per row, 8 systems per CTA at P = 32): 1536x768x1024 2.13 against 2.58 ms,
+// 768x384x512 246 against 250 us; with 512 threads at P = 16 267 us.  Copies of 8 bytes cost half
+// as much again (3.0 ms), stores through shared memory 0.27 ms.  At P <= 8 the rows kernel's segments
+// are 256 bytes and more: 384x192x256 alone takes 35 against 38 us here, but a batch of 64 solves
+// side by side 2736 us with this kernel and 2520 with that one (its CTAs need little shared memory).
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+template <int M, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
+    k_tridiag_tile(Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
+                   const double* __restrict__ lamx, const double* __restrict__ lamz, const float* __restrict__ rtab,
+                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, SideArgs sd) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if ((int)blockIdx.x < sd.n) {
+    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
+    return;
+  }
+  static_assert(M % 2 == 0, "whole rounds of pair copies");
+  constexpr int MS = M | 1, LGNT = NT == 512 ? 9 : 8;   // odd stride of a block's (a, c) pairs
+  const int P = 1 << lgP, lgS = LGNT - lgP, S = 1 << lgS;
+  const int tid = threadIdx.x;
+  const int s = tid & (S - 1), b = tid >> lgS;
+  float2* tile = reinterpret_cast<float2*>(smem_raw);                 // [row][s]
+  float4* ex = reinterpret_cast<float4*>(tile + (size_t)M * NT);      // [s][b], stride P + 1
+  float2* ac = reinterpret_cast<float2*>(ex + (size_t)S * (P + 1));   // [b][i]
+  const int idx0 = ((int)blockIdx.x - sd.n) * S, total = g.nz * width;
+  // mode of index q of the flattened (kz, kx - kx_lo) order; false for padding, columns outside the
+  // launch and the modes solved apart
+  auto mode = [&](int q, int& kx, int& kz) {
+    kz = q / width;
+    kx = kx_lo + q - kz * width;
+    return q < total && kx < kx_hi && !(kx == 0 && kz == 0) && !is_low(kx, kz, g.nz, low);
+  };
+  const size_t rstride = (size_t)g.nz * g.pitch;
+  {   // a pair of systems per copy; width is even, so a pair never crosses a row of the spectrum
+    const int q = idx0 + 2 * (tid & (S / 2 - 1)), r0 = tid >> (lgS - 1);
+    if (q < total) {
+      const int kz = q / width;
+      const float2* src = reinterpret_cast<const float2*>(spec) + (size_t)kz * g.pitch + kx_lo + (q - kz * width) +
+                          (size_t)r0 * rstride;
+      float2* dst = tile + 2 * tid;
+      const size_t step = (size_t)(2 * P) * rstride;   // 2 P rows per round of the CTA
+#pragma unroll
+      for (int n = 0; n < M / 2; ++n) cp_async16(dst + (size_t)n * 2 * NT, src + n * step);
+    }
+  }
+  int kx, kz;
+  const bool active = mode(idx0 + s, kx, kz);
+  for (int j = tid; j < g.ny; j += NT) {
+    const int bj = j / M;
+    ac[bj * MS + j - bj * M] = make_float2(a[j], c[j]);
+  }
+  const float sigma = active ? float(-(lamx[kx] + lamz[kz])) : 0.f;
+  cp_async_wait_all();
+  __syncthreads();
+  const float2* co = ac + b * MS;
+  float2* rows = tile + (size_t)b * M * S + s;
+  float rbv[M];
+  float2 xF = make_float2(0.f, 0.f), xL = make_float2(0.f, 0.f);
+  if (active) {
+    float2 cf = co[0];
+    float e = cf.x + sigma, rb = rcp_nr(cf.y + e), run = 1.f;
+    float2 gg = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      const float2 F = rows[i * S];
+      float mult = 0.f;
+      if (i > 0) {
+        cf = co[i];
+        mult = cf.x * rb;
+        e = fmaf(mult, e, sigma);
+        rb = rcp_nr(cf.y + e);
+      }
+      gg = make_float2(fmaf(mult, gg.x, -F.x), fmaf(mult, gg.y, -F.y));
+      xL = make_float2(gg.x * rb, gg.y * rb);
+      rows[i * S] = xL;
+      rbv[i] = rb;
+      const float kap = run * rb;
+      xF.x = fmaf(kap, gg.x, xF.x);
+      xF.y = fmaf(kap, gg.y, xF.y);
+      run *= cf.y * rb;
+    }
+  }
+  ex[s * (P + 1) + b] = make_float4(xF.x, xF.y, xL.x, xL.y);
+  const int s2 = tid >> lgP, b2 = tid & (P - 1);   // interface role, system-major
+  float vL = 0.f, inv = 0.f, X01 = 0.f, X10 = 0.f, tw = 0.f;
+  int kx2, kz2;
+  if (b2 < P - 1 && mode(idx0 + s2, kx2, kz2)) {
+    const float* r = rtab + ((size_t)(kz2 * g.ncols + kx2) * (P - 1) + b2) * 5;
+    vL = __ldg(r); inv = __ldg(r + 1); X01 = __ldg(r + 2); X10 = __ldg(r + 3); tw = __ldg(r + 4);
+  }
+  __syncthreads();
+  float4* mine = ex + s2 * (P + 1) + b2;
+  const float4 x = *mine;
+  float2 al, be;
+  scan_interfaces(P, b2, make_float2(x.x, x.y), make_float2(x.z, x.w), vL, inv, X01, X10, tw, al, be);
+  *mine = make_float4(al.x, al.y, be.x, be.y);
+  __syncthreads();
+  if (active) {
+    const float4 y = ex[s * (P + 1) + b];
+    float gv = co[0].x;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      if (i > 0) gv = co[i].x * rbv[i - 1] * gv;
+      const float rgv = gv * rbv[i];
+      const float2 q = rows[i * S];
+      rows[i * S] = make_float2(fmaf(rgv, y.x, q.x), fmaf(rgv, y.y, q.y));
+    }
+    float2 xn = make_float2(y.z, y.w);
+    float2* p = reinterpret_cast<float2*>(spec) + (size_t)kz * g.pitch + kx + (size_t)(b * M + M - 1) * rstride;
+#pragma unroll
+    for (int i = M - 1; i >= 0; --i, p -= rstride) {
+      const float2 q = rows[i * S];
+      const float crb = co[i].y * rbv[i];
+      xn = make_float2(fmaf(crb, xn.x, q.x), fmaf(crb, xn.y, q.y));
+      *p = xn;
     }
   }
 }
@@ -789,6 +922,42 @@ cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int par
   return cudaGetLastError();
 }
 
+// The launch's columns: a whole row with its padding, so that the systems of a CTA start on a
+// 64-byte boundary (S >= 8).
+static int launch_width(const Geometry& g, int kx_lo, int kx_hi) { return (kx_hi == g.ncols ? g.pitch : kx_hi) - kx_lo; }
+static int log2_of(int P) {
+  int l = 0;
+  while ((1 << l) < P) ++l;
+  return l;
+}
+
+template <int M>
+static cudaError_t launch_rows(const Geometry& g, const DevTables& tb, int parts, int low, cplx<float>* spec,
+                               SideArgs sd, cudaStream_t st, int kx_lo, int kx_hi) {
+  const int S = 256 / parts, width = launch_width(g, kx_lo, kx_hi), blocks = (g.nz * width + S - 1) / S;
+  size_t smem = (size_t)S * (parts + 1) * 16 + 5 * 256 * 4 + (size_t)parts * (M | 1) * 8;
+  cudaError_t e = prepare_side<float>(g, sd, 256, smem, spec, st);
+  if (e != cudaSuccess) return e;
+  if ((e = prep(k_tridiag_rows<M>, smem)) != cudaSuccess) return e;
+  k_tridiag_rows<M><<<sd.n + blocks, 256, smem, st>>>(g, log2_of(parts), low, tb.f.a, tb.f.c, tb.lamx, tb.lamz,
+                                                      tb.red_f, spec, kx_lo, kx_hi, width, sd);
+  return cudaGetLastError();
+}
+
+template <int M, int NT>
+static cudaError_t launch_tile(const Geometry& g, const DevTables& tb, int parts, int low, cplx<float>* spec,
+                               SideArgs sd, cudaStream_t st, int kx_lo, int kx_hi) {
+  const int S = NT / parts, width = launch_width(g, kx_lo, kx_hi), blocks = (g.nz * width + S - 1) / S;
+  size_t smem = (size_t)M * NT * 8 + (size_t)S * (parts + 1) * 16 + (size_t)parts * (M | 1) * 8;
+  cudaError_t e = prepare_side<float>(g, sd, 256, smem, spec, st);
+  if (e != cudaSuccess) return e;
+  auto kern = k_tridiag_tile<M, NT>;
+  if ((e = prep(kern, smem)) != cudaSuccess) return e;
+  kern<<<sd.n + blocks, NT, smem, st>>>(g, log2_of(parts), low, tb.f.a, tb.f.c, tb.lamx, tb.lamz, tb.red_f, spec, kx_lo,
+                                        kx_hi, width, sd);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes,
                                    cplx<float>* spec, SideArgs sd, cudaStream_t st, int kx_lo, int kx_hi) {
   if (!reg_tridiag_ok(g.ny, parts)) return cudaErrorNotSupported;
@@ -798,28 +967,27 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
   const bool whole = kx_lo == 0 && kx_hi == g.ncols;
   if (kx_lo < 0 || kx_hi > g.ncols || kx_hi <= kx_lo) return cudaErrorInvalidValue;
   if (!whole && (!scan_tridiag_ok(g.ny, parts) || kx_lo % S)) return cudaErrorNotSupported;
-  if (scan_tridiag_ok(g.ny, parts)) {   // P a power of two <= 32: the blocks in registers
-    int lgP = 0;
-    while ((1 << lgP) < parts) ++lgP;
-    // the launch's columns; a whole row with its padding keeps every CTA's segments 64-byte aligned
-    const int width = (kx_hi == g.ncols ? g.pitch : kx_hi) - kx_lo;
-    const int blocks = (g.nz * width + S - 1) / S;
-    size_t smem = (size_t)S * (parts + 1) * 16 + 5 * 256 * 4 + (size_t)parts * (m | 1) * 8;
-    const cudaError_t es = prepare_side<float>(g, sd, 256, smem, spec, st);
-    if (es != cudaSuccess) return es;
-#define PP_ROWS_CASE(MM)                                                                                       \
-  case MM: {                                                                                                   \
-    cudaError_t e = prep(k_tridiag_rows<MM>, smem);                                                            \
-    if (e != cudaSuccess) return e;                                                                            \
-    k_tridiag_rows<MM><<<sd.n + blocks, 256, smem, st>>>(g, lgP, low_modes, tb.f.a, tb.f.c, tb.lamx, tb.lamz,  \
-                                                         tb.red_f, spec, kx_lo, kx_hi, width, sd);             \
-    return cudaGetLastError();                                                                                 \
-  }
+  if (scan_tridiag_ok(g.ny, parts)) {   // P a power of two <= 32
+    // P >= 16 with blocks of at least 12 rows: tiles in shared memory; else in registers (both
+    // sides measured, see the two kernels)
+    if (parts >= 16) {
+      switch (m) {
+#define PP_TILE_CASE(MM)                                                                           \
+  case MM:                                                                                         \
+    return parts == 32 ? launch_tile<MM, 512>(g, tb, parts, low_modes, spec, sd, st, kx_lo, kx_hi) \
+                       : launch_tile<MM, 256>(g, tb, parts, low_modes, spec, sd, st, kx_lo, kx_hi);
+        PP_TILE_CASE(12) PP_TILE_CASE(16) PP_TILE_CASE(24)
+        default: break;
+      }
+    }
+#define PP_ROWS_CASE(MM) \
+  case MM: return launch_rows<MM>(g, tb, parts, low_modes, spec, sd, st, kx_lo, kx_hi);
     switch (m) {
       PP_ROWS_CASE(1) PP_ROWS_CASE(2) PP_ROWS_CASE(3) PP_ROWS_CASE(4) PP_ROWS_CASE(6) PP_ROWS_CASE(8)
       PP_ROWS_CASE(12) PP_ROWS_CASE(16) PP_ROWS_CASE(24)
       default: break;
     }
+#undef PP_TILE_CASE
 #undef PP_ROWS_CASE
   }
   const int nt = parts * S;
@@ -850,12 +1018,12 @@ cudaError_t launch_tridiag_factored(const Geometry& g, const DevTables& tb, int 
                                     const SideArgs& sd, cudaStream_t st) {
   if (parts == 1 && g.ny <= kScan64Rows && tb.tri_d.nsys <= kScan64Systems) {
     SideArgs side = sd;
-    size_t smem = (size_t)((g.ny + 7) / 8) * 128 * 24;
-    cudaError_t e = prepare_side<double>(g, side, 128, smem, spec, st);
+    size_t smem = (size_t)((g.ny + 7) / 8) * 64 * 24;
+    cudaError_t e = prepare_side<double>(g, side, 64, smem, spec, st);
     if (e != cudaSuccess) return e;
     if ((e = prep(k_tridiag_scan64, smem)) != cudaSuccess) return e;
-    const int blocks = (g.nz * g.pitch + 15) / 16;
-    k_tridiag_scan64<<<side.n + blocks, 128, smem, st>>>(g, tb.d.c, tb.tri_d, spec, side);
+    const int blocks = (g.nz * g.pitch + 7) / 8;
+    k_tridiag_scan64<<<side.n + blocks, 64, smem, st>>>(g, tb.d.c, tb.tri_d, spec, side);
     return cudaGetLastError();
   }
   return launch_factored<double, true>(g, tb.d.a, tb.d.c, tb.tri_d, parts, -1, trunc, spec, sd, st);
