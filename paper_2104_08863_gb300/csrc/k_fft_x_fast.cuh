@@ -1,14 +1,17 @@
 // Specialised x-transform kernels (steps (2) and (8) of Sec. 3.2) for the half-lengths M = Nx/2 of
 // the form 2^a 3^b from 8 to 1024 (but 864 and 972), instantiated in three groups of translation
-// units (k_fft_x_fast_*.cu).
+// units (k_fft_x_fast_*.cu).  Other lengths take the runtime-radix kernels (k_fft.cu), which cost
+// more at every length that both have: forward and z of an FP32 162x90x108 solve 17.5 and 19.5 us
+// there, 11.5 and 7.5 us here; forward, z and inverse of an FP64 216x130x162 solve 199, 157, 195 us
+// there, 163, 147, 148 us here.
 //
 // A CTA takes LPB consecutive x-lines, which are one contiguous stretch of the field, packs
 // each real line as M complex values, transforms all lines in place in padded shared memory
 // with the compile-time Stockham engine, and unpacks the Nx/2+1 spectral bins (forward) or
 // writes the Nx real values (inverse).  LPB and the thread count give each thread 8 staged complex
-// values per stage.  FP64 CTAs have 64 threads where a line allows it: the FP64 pipe bounds them at
-// any size, and at 64x64x64 the 256 CTAs fill the SMs that 64 of 256 threads did not (divergence and
-// x 26 -> 18 us, inverse 18 -> 12).
+// values per stage.  FP64 CTAs have 64 threads where a line allows it (32 up to M = 16): the FP64
+// pipe bounds them at any size, and at 64x64x64 the 256 CTAs fill the SMs that 64 of 256 threads
+// did not (divergence and x 26 -> 18 us, inverse 18 -> 12).
 #pragma once
 
 #include <map>
@@ -26,10 +29,11 @@ namespace pp {
 template <typename T, int M> struct XTile {
   static constexpr int E = 8;
   static constexpr int MAXR = 8;
-  static constexpr int LPB0 = (E * (sizeof(T) == 4 ? 256 : 64)) / M;
+  static constexpr int TMIN = sizeof(T) == 4 ? 64 : 32;
+  static constexpr int LPB0 = (E * (sizeof(T) == 4 ? 256 : (M <= 16 ? 32 : 64))) / M;
   static constexpr int LPB = LPB0 < 1 ? 1 : (LPB0 > 64 ? 64 : LPB0);
   static constexpr int T0 = ((LPB * M / E) + 31) / 32 * 32;
-  static constexpr int THREADS = T0 < 64 ? 64 : (T0 > 512 ? 512 : T0);
+  static constexpr int THREADS = T0 < TMIN ? TMIN : (T0 > 512 ? 512 : T0);
   static constexpr int SMEM = padded_size<T>(LPB * M) * (int)sizeof(cplx<T>);
   static constexpr int MINB = sizeof(T) == 4 ? 4 : 512 / THREADS;
 };

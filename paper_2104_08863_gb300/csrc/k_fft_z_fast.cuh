@@ -3,9 +3,10 @@
 // coalesced row segments of W complex values, transformed in place in (padded) shared memory
 // by the compile-time Stockham engine (FP64: its form with fused twiddles), and stored back.  W and
 // the thread count are chosen so that each thread stages 8 complex values per stage and a CTA has
-// about 256 threads: several are resident, so that one CTA's loads overlap another's arithmetic,
-// and a small grid still gives every SM one (2.15 ms at 512x384x512, 2.18 with 512 threads).  A launch may
-// cover only the kx columns [kx_lo, kx_hi) (one slab of the spectrum; kx_lo a multiple of W).
+// about 64 threads (columns of 64 bytes at least): the FP64 pipe bounds the pass at any size, and a
+// small or ragged grid fills the SMs better (216x130x162 157 -> 123 us with 139 at 256 threads,
+// 64x64x64 14 -> 12 us; 512x384x512 2.15 ms, 2.18 at 512 threads).  A launch may cover only the kx
+// columns [kx_lo, kx_hi) (one slab of the spectrum; kx_lo a multiple of W).
 #pragma once
 
 #include "fft_lf.cuh"
@@ -17,7 +18,7 @@ namespace pp {
 template <typename T, int NZ> struct ZTile {
   static constexpr int E = sizeof(T) == 4 ? 16 : 8;               // complex values per thread
   static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;             // 64-byte row segments
-  static constexpr int W0 = (E * 256) / NZ;
+  static constexpr int W0 = (E * 64) / NZ;
   static constexpr int W = W0 < WMIN ? WMIN : (W0 > 32 ? 32 : W0);
   static constexpr int T0 = (W * NZ / E + 31) / 32 * 32;
   static constexpr int THREADS = T0 < 64 ? 64 : (T0 > 512 ? 512 : T0);
