@@ -89,18 +89,10 @@ __global__ void __launch_bounds__(XTile<T, M>::THREADS, XTile<T, M>::MINB)
         st_c(X + M - kx, Xm);
       }
     }
-    return;
-  }
-  fft_static<T, M, -1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
-  constexpr int M1 = M + 1;
-#pragma unroll 4
-  for (int idx = threadIdx.x; idx < LPB * M1; idx += THREADS) {
-    const int t = idx / M1, kx = idx % M1;
-    const int line = line0 + t;
-    if (line >= nlines) continue;
-    const cplx<T> Zk = buf[padi<T>(t * M + (kx == M ? 0 : kx))];
-    const cplx<T> Zc = conj(buf[padi<T>(t * M + (kx == 0 ? 0 : M - kx))]);
-    st_c(spec + (size_t)line * g.pitch + kx, fwd_post(Zk, Zc, ldg_c(tt.tw_post + kx)));
+  } else {
+    fft_static<T, M, -1, LPB, THREADS, 1, M, false, C::MAXR>(buf, tt.tw_m);
+    store_spectra<M, LPB, THREADS>([&](int t, int k) { return buf[padi<T>(t * M + k)]; }, tt.tw_post, spec, g.pitch, line0,
+                                   nlines);
   }
 }
 
@@ -275,15 +267,8 @@ __global__ void __launch_bounds__(XPipe<TI, M>::THREADS, XPipe<TI, M>::MINB)
       if (b + (int)gridDim.x < ntiles) issue(b + gridDim.x);
     };
     fft_static_from<float, M, -1, LPB, THREADS, 1, M, false, XTile<float, M>::MAXR>(buf, tt.tw_m, load, refill);
-    constexpr int M1 = M + 1;
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < LPB * M1; idx += THREADS) {
-      const int t = idx / M1, kx = idx % M1;
-      if (t >= nl) continue;
-      const cplx<float> Zk = buf[padi<float>(t * M + (kx == M ? 0 : kx))];
-      const cplx<float> Zc = conj(buf[padi<float>(t * M + (kx == 0 ? 0 : M - kx))]);
-      st_c(spec + (size_t)(line0 + t) * g.pitch + kx, fwd_post(Zk, Zc, ldg_c(tt.tw_post + kx)));
-    }
+    store_spectra<M, LPB, THREADS>([&](int t, int k) { return buf[padi<float>(t * M + k)]; }, tt.tw_post, spec, g.pitch,
+                                   line0, line0 + nl);
   }
 }
 

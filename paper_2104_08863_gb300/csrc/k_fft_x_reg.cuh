@@ -7,8 +7,8 @@
 // the mode: a plain load, the divergence of Eq. 7, the adjoint's G^T g), takes their
 // N2-point DFT, multiplies output k2 by W_M^{n1 k2} and writes it to shared memory at
 // [t][k2][n1]; pass 2 thread (t, k2) takes the N1-point DFT of row k2 (output k1 is Z[k2 + N2 k1]).
-// Forward: the Z are written back in natural order and the Nx/2+1 spectral bins unpacked from
-// Z_k and Z_{M-k} (fwd_post) and stored.  Inverse: pass 1 packs X_k and X_{M-k} (inv_pre) on the
+// Forward: the Z are written back in natural order and the Nx/2+1 spectral bins unpacked in pairs
+// from Z_k and Z_{M-k} (store_spectra).  Inverse: pass 1 packs X_k and X_{M-k} (inv_pre) on the
 // way in, pass 2 writes (or adds) the real values straight from registers, with the line's
 // dy-weighted sum when asked.  Against the Stockham kernels this makes
 // one (inverse) or two (forward) shared-memory round trips instead of one per stage plus two, and
@@ -86,19 +86,9 @@ __device__ __forceinline__ void fwd_x_reg_tile(const Geometry& g, const FwdArgs&
     });
   }
   __syncthreads();
-  constexpr int M1 = M + 1;
-  if (live) {
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < LPB * M1; idx += THREADS) {
-      const int t = idx / M1, kx = idx - t * M1;
-      const int line = line0 + t;
-      if (line >= nlines) continue;
-      const cplx<float>* nat = buf + t * LS;
-      const cplx<float> Zk = nat[kx == M ? 0 : kx];
-      const cplx<float> Zc = conj(nat[kx == 0 ? 0 : M - kx]);
-      st_c(spec + (size_t)line * g.pitch + kx, fwd_post(Zk, Zc, ldg_c(tt.tw_post + kx)));
-    }
-  }
+  if (live)
+    store_spectra<M, LPB, THREADS>([&](int tl, int k) { return buf[tl * LS + k]; }, tt.tw_post, spec, g.pitch, line0,
+                                   nlines);
 }
 
 // Three CTAs per SM (85 registers), as for the inverse below.
@@ -184,19 +174,9 @@ __device__ __forceinline__ void fwd_x_reg_resid_tile(const Geometry& g, const Fw
     });
   }
   __syncthreads();
-  constexpr int M1 = M + 1;
-  if (live) {
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < LPB * M1; idx += THREADS) {
-      const int tl = idx / M1, kx = idx - tl * M1;
-      const int line = line0 + tl;
-      if (line >= nlines) continue;
-      const cplx<float>* nat = buf + tl * LS;
-      const cplx<float> Zk = nat[kx == M ? 0 : kx];
-      const cplx<float> Zc = conj(nat[kx == 0 ? 0 : M - kx]);
-      st_c(spec + (size_t)line * g.pitch + kx, fwd_post(Zk, Zc, ldg_c(tt.tw_post + kx)));
-    }
-  }
+  if (live)
+    store_spectra<M, LPB, THREADS>([&](int tl, int k) { return buf[tl * LS + k]; }, tt.tw_post, spec, g.pitch, line0,
+                                   nlines);
 }
 
 // RIN: a later correction (the stored first residual in place of f - <f>, see resid_line).

@@ -195,6 +195,45 @@ __device__ __forceinline__ cplx<T> fwd_post(cplx<T> Zk, cplx<T> ZmConj, cplx<T> 
   return scale(s - mul_i(cmul(W, d), 1), T(0.5));
 }
 
+// Bins k and M-k (0 < k < M/2) of a real line at once: with s, d as above and t = W d / 2,
+// X_k = s/2 - i t and X_{M-k} = conj(s/2 + i t).  14 operations for both, where fwd_post takes 14 for
+// each, and each Z is read once: the unpacking was a third of the FP32 forward transform's instructions
+// (768x384x512 forward x 308 -> 236 us, 6.7 TB/s would be 179; residual pass of 1536x768x1024 7.31 ->
+// 6.92 ms, its FP64-input pass 3.69 -> 3.28 ms).
+template <typename T>
+__device__ __forceinline__ void fwd_post2(cplx<T> Zk, cplx<T> Zm, cplx<T> W, cplx<T>& Xk, cplx<T>& Xm) {
+  const cplx<T> s = mk<T>(Zk.x + Zm.x, Zk.y - Zm.y), d = mk<T>(Zk.x - Zm.x, Zk.y + Zm.y);
+  const cplx<T> t = cmul(scale(W, T(0.5)), d);
+  Xk = mk<T>(fma(T(0.5), s.x, t.y), fma(T(0.5), s.y, -t.x));
+  Xm = mk<T>(fma(T(0.5), s.x, -t.y), fma(T(-0.5), s.y, -t.x));
+}
+
+// The half spectra X (rows of `pitch`) of the LPB lines line0.. below nlines from their half-length
+// transforms Z(t, k): two bins per item, and bins 0, M and (M even) M/2, whose partner is itself,
+// with the first item of a line.
+template <int M, int LPB, int THREADS, typename Z>
+__device__ __forceinline__ void store_spectra(Z z, const cplx<float>* __restrict__ tw_post, cplx<float>* __restrict__ spec,
+                                              int pitch, int line0, int nlines) {
+  constexpr int H = (M + 1) / 2;
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < LPB * H; idx += THREADS) {
+    const int t = idx / H, k = idx - t * H;
+    if (line0 + t >= nlines) continue;
+    cplx<float>* X = spec + (size_t)(line0 + t) * pitch;
+    const cplx<float> Zk = z(t, k);
+    if (k == 0) {
+      st_c(X, mk<float>(Zk.x + Zk.y, 0.f));
+      st_c(X + M, mk<float>(Zk.x - Zk.y, 0.f));
+      if constexpr (M % 2 == 0) st_c(X + M / 2, conj(z(t, M / 2)));
+    } else {
+      cplx<float> Xk, Xm;
+      fwd_post2(Zk, z(t, M - k), ldg_c(tw_post + k), Xk, Xm);
+      st_c(X + k, Xk);
+      st_c(X + M - k, Xm);
+    }
+  }
+}
+
 // Pack bins k and M-k of a Hermitian half spectrum for the half-length inverse transform
 // (k = 0 uses the real parts of bins 0 and M only).
 template <typename T>
