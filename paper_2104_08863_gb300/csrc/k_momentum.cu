@@ -23,8 +23,8 @@
 // FP32 is bound by HBM (24 / 36 bytes per point) once the instructions are few enough: one point
 // per thread issued 221 instructions per point, most of them addresses, at 20 warps per SM
 // (269 / 372 us for the two stages of 384x192x256); now 113 / 131 us (4.0 / 5.2 TB/s).  FP64 is
-// bound by its issue rate of two instructions per clock and SM (62 / 65 per point, before 67 / 70):
-// 512x384x512 11.4 / 11.9 ms, before 12.6 / 12.5.
+// bound by its issue rate of two instructions per clock and SM (about 59 / 62 per point, before 67 / 70):
+// 512x384x512 11.0 / 11.5 ms, before 12.6 / 12.5.
 #include "internal.h"
 
 namespace pp {
@@ -85,7 +85,12 @@ __device__ __forceinline__ MVec<T, V> vldv(const T* p) { return *reinterpret_cas
 template <typename T, int V>
 __device__ __forceinline__ void vst(T* p, const MVec<T, V>& r) { *reinterpret_cast<MVec<T, V>*>(p) = r; }
 
-template <typename T, int V, bool BASE>
+// SHARE: the u-w and v-w fluxes through z-face k + 1 are those that the thread at k + 1 computes
+// anyway, taken from it through shared memory (two buffers, one barrier per row) instead of computed
+// again; the last line of a tile computes them.  Only the FP64 kernel does (7 of its 62 instructions
+// per point go, 4 in two stay as differences): 512x384x512 11.44 / 11.94 -> 10.97 / 11.53 ms; FP32 is
+// not bound by its arithmetic.
+template <typename T, int V, bool BASE, bool SHARE>
 __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs<T> a, MomCoef mc,
                                                             const double* __restrict__ inv_dy,
                                                             const double* __restrict__ inv_h,
@@ -94,6 +99,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
   using Vt = MVec<T, V>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RowCoef<T>* rc = reinterpret_cast<RowCoef<T>*>(smem_raw);
+  __shared__ MVec<T, V> edge[SHARE ? 2 : 1][SHARE ? 2 * MOM_THREADS : 1];   // [buffer][u-w, v-w][thread]
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int j0 = jlo + blockIdx.z * jc;
   const int j1 = min(jhi, j0 + jc);
@@ -118,9 +124,16 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
     rc[r] = c;
   }
   __syncthreads();
-  const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
-  const int k = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i0 >= nx || k >= nz) return;
+  int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
+  int k = blockIdx.y * blockDim.y + threadIdx.y;
+  const bool live = i0 < nx && k < nz;
+  if (!live) {
+    if constexpr (!SHARE) return;
+    i0 = 0;   // keeps the barriers' company on a point of its own, storing nothing
+    k = 0;
+  }
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const bool shared_zp = SHARE && threadIdx.y + 1 < blockDim.y && k + 1 < nz && live;
   const T cDx = T(mc.cdx), cDz = T(mc.cdz), cAx = T(mc.cax), cAz = T(mc.caz);
   const T fterm = T(mc.fterm), alpha = T(a.alpha);
   const ptrdiff_t plane = (ptrdiff_t)nz * nx;
@@ -158,7 +171,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
 #pragma unroll
     for (int q = 0; q < V; ++q) e_vw[q] = (v_zm.x[q] + v_c.x[q]) * (w_m.x[q] + w_c.x[q]);
   } else {   // bottom wall face of v: boundary value
-    vst<T, V>(a.ov + o, BASE ? vldv<T, V>(a.bv + o) : v_c);
+    if (live) vst<T, V>(a.ov + o, BASE ? vldv<T, V>(a.bv + o) : v_c);
   }
   for (int j = j0; j < j1; ++j, o += plane) {
     const RowCoef<T> c = rc[j - j0];
@@ -176,7 +189,9 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
     const Vt u_zm = vldg<T, V>(su + o + dzm), u_zp = vldg<T, V>(su + o + dzp);
     const Vt w_zm = vldg<T, V>(sw + o + dzm), w_zp = vldg<T, V>(sw + o + dzp), v_zp = vldg<T, V>(sv + o + dzp);
     const T u_xm = __ldg(su + o + dxm), uzm_xp = __ldg(su + o + dzm + dxp);
-    const T w_xm = __ldg(sw + o + dxm), w_xp = __ldg(sw + o + dxp), wzp_xm = __ldg(sw + o + dzp + dxm);
+    const T w_xm = __ldg(sw + o + dxm), w_xp = __ldg(sw + o + dxp);
+    T wzp_xm = T(0);
+    if (!shared_zp) wzp_xm = __ldg(sw + o + dzp + dxm);
     Vt bu, bw, bv;
     if constexpr (BASE) {
       bu = vldv<T, V>(a.bu + o);
@@ -195,6 +210,39 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
       e_uv_n[V] = T(0);
     }
     uv_flux(w_xm, w_c, w_xp, u_zm, uzm_xp, u_c, u_xp, e_uw);   // (w_xm + w_c) (u_zm + u_c)
+    T fz_u[V], fz_v[V];   // flux differences across the cell in z: u-w for u, v-w for v
+    if constexpr (SHARE) {
+      Vt* e = edge[(j - j0) & 1];
+      Vt su_, sv_;
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        su_.x[q] = e_uw[q];
+        sv_.x[q] = e_vw[q];
+      }
+      e[tid] = su_;
+      e[MOM_THREADS + tid] = sv_;
+      __syncthreads();
+      if (shared_zp) {
+        const Vt nu_ = e[tid + blockDim.x], nv_ = e[MOM_THREADS + tid + blockDim.x];
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+          fz_u[q] = nu_.x[q] - e_uw[q];
+          fz_v[q] = nv_.x[q] - e_vw[q];
+        }
+      }
+    }
+    if (!shared_zp) {
+      Vt wmz = wm_zp;   // w(j-1, k+1): rolled, or (few lines) loaded again
+      if constexpr (SHARE) {
+        if (j > j0) wmz = vldg<T, V>(sw + o - plane + dzp);
+      }
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        const T wzpxm = q ? w_zp.x[q - 1] : wzp_xm;
+        fz_u[q] = (wzpxm + w_zp.x[q]) * (u_c.x[q] + u_zp.x[q]) - e_uw[q];
+        fz_v[q] = (v_c.x[q] + v_zp.x[q]) * (wmz.x[q] + w_zp.x[q]) - e_vw[q];
+      }
+    }
     Vt ru, rw, rv;
 #pragma unroll
     for (int q = 0; q < V; ++q) {
@@ -202,7 +250,6 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
       const T uxm = q ? u_c.x[q - 1] : u_xm, uxp = q + 1 < V ? u_c.x[q + 1] : u_xp;
       const T wxm = q ? w_c.x[q - 1] : w_xm, wxp = q + 1 < V ? w_c.x[q + 1] : w_xp;
       const T vxm = q ? v_c.x[q - 1] : v_xm, vxp = q + 1 < V ? v_c.x[q + 1] : v_xp;
-      const T wzpxm = q ? w_zp.x[q - 1] : wzp_xm;
       {   // u
         T acc = fterm;
         if constexpr (BASE) acc = alpha * bu.x[q] + acc;
@@ -211,7 +258,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
         acc = cDx * sx + acc;
         acc = cAx * ((uxp - uxm) * (sx + T(2) * uc)) + acc;
         acc = cDz * (u_zp.x[q] + u_zm.x[q]) + acc;
-        acc = cAz * ((wzpxm + w_zp.x[q]) * (uc + u_zp.x[q]) - e_uw[q]) + acc;
+        acc = cAz * fz_u[q] + acc;
         acc = c.cay * (e_uv_n[q] - e_uv[q]) + acc;
         acc = c.ca * u_m.x[q] + acc;
         ru.x[q] = c.cc * u_n.x[q] + acc;
@@ -236,19 +283,21 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
         acc = cDx * (vxp + vxm) + acc;
         acc = cAx * (e_uv[q + 1] - e_uv[q]) + acc;
         acc = cDz * (v_zp.x[q] + v_zm.x[q]) + acc;
-        acc = cAz * ((vv + v_zp.x[q]) * (wm_zp.x[q] + w_zp.x[q]) - e_vw[q]) + acc;
+        acc = cAz * fz_v[q] + acc;
         acc = c.va * v_m.x[q] + acc;
         rv.x[q] = c.vc * v_n.x[q] + acc;
       }
     }
-    vst<T, V>(a.ou + o, ru);
-    vst<T, V>(a.ow + o, rw);
-    if (j >= 1) vst<T, V>(a.ov + o, rv);   // interior faces
+    if (live) {
+      vst<T, V>(a.ou + o, ru);
+      vst<T, V>(a.ow + o, rw);
+      if (j >= 1) vst<T, V>(a.ov + o, rv);   // interior faces
+    }
     // roll
     u_m = u_c; u_c = u_n; u_xp = un_xp;
     w_m = w_c; w_c = w_n;
     v_m = v_c; v_c = v_n; v_xm = vn_xm; v_xp = vn_xp; v_zm = vn_zm;
-    wm_zp = w_zp;
+    if constexpr (!SHARE) wm_zp = w_zp;
 #pragma unroll
     for (int q = 0; q < V; ++q) {
       e_uv[q] = e_uv_n[q];
@@ -256,7 +305,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
     }
     e_uv[V] = e_uv_n[V];
   }
-  if (j1 == ny) vst<T, V>(a.ov + o, BASE ? vldv<T, V>(a.bv + o) : v_c);   // top wall face of v: boundary value
+  if (live && j1 == ny) vst<T, V>(a.ov + o, BASE ? vldv<T, V>(a.bv + o) : v_c);   // top wall face of v: boundary value
 }
 
 template <typename T, int V>
@@ -270,12 +319,13 @@ cudaError_t launch_momentum_v(const Geometry& g, const DevTables& tb, const MomA
   const int jc = momentum_chunk_rows((long long)gx * gz, rows);
   const size_t smem = sizeof(RowCoef<T>) * (size_t)jc;
   const dim3 grid(gx, gz, (rows + jc - 1) / jc), block(tx, tz);
+  constexpr bool SH = sizeof(T) == 8;
   const bool base = a.bu != nullptr;
-  const void* kern = base ? (const void*)k_momentum<T, V, true> : (const void*)k_momentum<T, V, false>;
+  const void* kern = base ? (const void*)k_momentum<T, V, true, SH> : (const void*)k_momentum<T, V, false, SH>;
   const cudaError_t e = ensure_smem_limit(kern, smem);
   if (e != cudaSuccess) return e;
-  if (base) k_momentum<T, V, true><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
-  else k_momentum<T, V, false><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
+  if (base) k_momentum<T, V, true, SH><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
+  else k_momentum<T, V, false, SH><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
   return cudaGetLastError();
 }
 
