@@ -17,10 +17,14 @@ namespace pp {
 // global loads are all issued before any arithmetic.  The k2 blocks of shared memory are padded so
 // that their byte stride is 64 mod 128: the pass-2 reads of a warp (four k2 blocks of W columns)
 // then fall on alternating bank halves.
+// Nz = 512 is split 16 x 32: CTAs of 128 threads with 32 values each in pass 1 and two rounds of 16 in
+// pass 2, four of them per SM where 32 x 16 has two of 256; the same loads are in flight, but the
+// phases of four CTAs overlap better (768x384x512: 215 us per pass, 241 before; a copy in the same
+// order takes 179).  At Nz = 1024 both factors are 32 and shared memory leaves room for three.
 template <typename T, int NZ> struct ZReg {
-  static constexpr int N1 = split_n1(NZ), N2 = NZ / N1;
+  static constexpr int N1 = NZ == 512 ? 16 : split_n1(NZ), N2 = NZ / N1;
   static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;   // 64-byte row segments
-  static constexpr int W0 = 256 / N1;
+  static constexpr int W0 = (NZ == 512 ? 128 : 256) / N1;
   static constexpr int W1 = W0 >= 32 ? 32 : (W0 >= 16 ? 16 : 8);   // a power of two: aligned row segments
   static constexpr int W = W1 < WMIN ? WMIN : W1;
   static constexpr int THREADS = W * N1;
@@ -67,26 +71,27 @@ __device__ __forceinline__ void z_reg_tile(const Geometry& g, const Tables<T>& t
     });
   }
   __syncthreads();
-  if (live && q < N2) {
-    const int k2 = q;
-    cplx<T> u[N1];
+  if (live) {
+    for (int k2 = q; k2 < N2; k2 += N1) {   // one round, or two when N2 > N1
+      cplx<T> u[N1];
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) u[n1] = buf[k2 * B + n1 * W + c];
-    reg_dft<T, N1, SIGN>(u);
-    if (cok) {
-      cplx<T>* dst = plane + (size_t)k2 * g.pitch + c;
-      const size_t step = (size_t)N2 * g.pitch;
-      static_for<0, N1>([&](auto sc) {
-        constexpr int s = decltype(sc)::value;
-        constexpr int k1 = reg_freq(N1, s);
-        st_c(dst + k1 * step, u[s]);
-      });
+      for (int n1 = 0; n1 < N1; ++n1) u[n1] = buf[k2 * B + n1 * W + c];
+      reg_dft<T, N1, SIGN>(u);
+      if (cok) {
+        cplx<T>* dst = plane + (size_t)k2 * g.pitch + c;
+        const size_t step = (size_t)N2 * g.pitch;
+        static_for<0, N1>([&](auto sc) {
+          constexpr int s = decltype(sc)::value;
+          constexpr int k1 = reg_freq(N1, s);
+          st_c(dst + k1 * step, u[s]);
+        });
+      }
     }
   }
 }
 
 template <typename T, int NZ, int SIGN>
-__global__ void __launch_bounds__(ZReg<T, NZ>::THREADS, 2) k_fft_z_reg(Geometry g, Tables<T> tt,
+__global__ void __launch_bounds__(ZReg<T, NZ>::THREADS, 512 / ZReg<T, NZ>::THREADS) k_fft_z_reg(Geometry g, Tables<T> tt,
                                                                       cplx<T>* __restrict__ spec, int kx_lo,
                                                                       int kx_hi) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
