@@ -101,6 +101,14 @@ cudaError_t ensure_smem_limit(const void* kernel, size_t bytes) {
   return e;
 }
 
+cudaError_t launch_plan_setup(const poisson_plan_s* pl, const DevTables& dt, unsigned char* ws, cudaStream_t st) {
+  if (!pl->has_tri)
+    return launch_reduced_setup(pl->g, dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, pl->low, (float*)(ws + pl->off_red),
+                                st);
+  const cudaError_t e = launch_low_setup(pl->g, dt, pl->low, st);
+  return e != cudaSuccess ? e : launch_tridiag_setup(pl->g, dt, pl->parts, st);
+}
+
 DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base) {
   DevTables dt;
   unsigned char* tb = base + pl->off_tables;
@@ -381,12 +389,7 @@ poisson_status poisson_set_workspace(poisson_plan_t pl, void* ws, size_t bytes, 
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return PS_ECUDA;
   pl->ws = base;
   pl->dt = pp::bind_tables(pl, base);
-  if (pp::launch_low_setup(pl->g, pl->dt, pl->low, st) != cudaSuccess) return PS_ECUDA;
-  if (!pl->has_tri && pl->parts > 1 &&
-      launch_reduced_setup(pl->g, pl->dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, (float*)(base + pl->off_red),
-                           st) != cudaSuccess)
-    return PS_ECUDA;
-  if (pl->has_tri && launch_tridiag_setup(pl->g, pl->dt, pl->parts, st) != cudaSuccess) return PS_ECUDA;
+  if (pp::launch_plan_setup(pl, pl->dt, base, st) != cudaSuccess) return PS_ECUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) return PS_ECUDA;
   return PS_OK;
 }

@@ -168,7 +168,8 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
 __host__ __device__ inline bool scan_tridiag_ok(int ny, int P) { return reg_tridiag_ok(ny, P) && P <= 32 && (P & (P - 1)) == 0; }
 // Bytes of the reduced-system table of the register kernel, and its FP64 set-up (once per plan).
 size_t reduced_table_bytes(const Geometry& g, int parts);
-cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int parts, bool trunc, float* tab,
+// The low modes' pivots (launch_low_setup) are built by the same launch.
+cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int parts, bool trunc, int low, float* tab,
                                  cudaStream_t st);
 
 // Gauge modes of the (0, 0) solve: plain zero weighted mean; GAUGE_STORE_MEAN also stores the
@@ -298,6 +299,8 @@ struct poisson_plan_s {
 namespace pp {
 // Table pointers of a plan inside a workspace that starts at `base`.
 DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base);
+// The per-mode tables of a plan (PDD factors or reduced systems, low modes' pivots) on a workspace.
+cudaError_t launch_plan_setup(const poisson_plan_s* pl, const DevTables& dt, unsigned char* ws, cudaStream_t st);
 // poisson_solve's pipeline on an explicit workspace (no timing events).
 poisson_status solve_on_workspace(poisson_plan_s* pl, unsigned char* ws, const DevTables& dt, const void* rhs,
                                   void* p, cudaStream_t st);

@@ -90,14 +90,14 @@ __global__ void __launch_bounds__(256) k_tridiag_setup(Geometry g, int P, int m,
 }
 
 template <typename T, bool FULL>
-__global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int m, int S, int low, int trunc,
+__global__ void __launch_bounds__(256) k_tridiag_factored(const __grid_constant__ Geometry g, int P, int m, int S, int low, int trunc,
                                                           const T* __restrict__ a, const T* __restrict__ c,
                                                           TriFactors<T> tf, cplx<T>* __restrict__ spec,
-                                                          SideArgs sd) {
+                                                          const __grid_constant__ SideArgs sd) {
   constexpr int CH = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if ((int)blockIdx.x < sd.n) {
-    low_system<T>(g, sd, spec, blockIdx.x, smem_raw);
+    low_system<T>(g, sd, spec, blockIdx.x);
     return;
   }
   T* sm = reinterpret_cast<T*>(smem_raw);
@@ -263,12 +263,12 @@ __global__ void __launch_bounds__(256) k_tridiag_factored(Geometry g, int P, int
 constexpr int kScan64Rows = 256;       // most rows (49 KB of shared memory)
 constexpr int kScan64Systems = 20000;  // most modes
 
-__global__ void __launch_bounds__(64) k_tridiag_scan64(Geometry g, const double* __restrict__ c,
+__global__ void __launch_bounds__(64) k_tridiag_scan64(const __grid_constant__ Geometry g, const double* __restrict__ c,
                                                         TriFactors<double> tf, cplx<double>* __restrict__ spec,
-                                                        SideArgs sd) {
+                                                        const __grid_constant__ SideArgs sd) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if ((int)blockIdx.x < sd.n) {
-    low_system<double>(g, sd, spec, blockIdx.x, smem_raw);
+    low_system<double>(g, sd, spec, blockIdx.x);
     return;
   }
   const int lane = threadIdx.x & 31, l = lane >> 2;
@@ -373,11 +373,47 @@ __device__ void block_spikes64(const double* a, const double* c, double sigma, i
   wL = c[r0 + m - 1] * rbp;
 }
 
-__global__ void __launch_bounds__(128) k_reduced_setup(Geometry g, int P, int m, int trunc, const double* __restrict__ a,
+// Pivots of the modes solved apart, one thread per system of the list (low_system's order):
+// rb[sys ny + j] = 1 / beta_j by the margin recurrence, in FP64.
+struct LowSetup { int n, low; double* rb; };
+__device__ void low_pivots(const Geometry& g, const LowSetup& ls, int sys, const double* __restrict__ a,
+                           const double* __restrict__ c, const double* __restrict__ lamx,
+                           const double* __restrict__ lamz) {
+  if (sys < 1 || sys >= ls.n) return;
+  const int kx = sys % (ls.low + 1), q = sys / (ls.low + 1);
+  const int kz = q <= ls.low ? q : g.nz - (q - ls.low);
+  const double sigma = -(lamx[kx] + lamz[kz]);
+  double e = 0.0, r = 0.0;
+  for (int j = 0; j < g.ny; ++j) {
+    e = j > 0 ? sigma + a[j] * e * r : sigma;
+    r = 1.0 / (c[j] + e);
+    ls.rb[(size_t)sys * g.ny + j] = r;
+  }
+}
+constexpr int kSetupThreads = 128;
+static LowSetup low_setup(const DevTables& tb, int low) {
+  return LowSetup{low < 1 ? 0 : (low + 1) * (2 * low + 1), low, tb.low_rb};   // low = 0: the (0, 0) mode only
+}
+static int low_blocks(const LowSetup& ls) { return (ls.n + kSetupThreads - 1) / kSetupThreads; }
+
+__global__ void __launch_bounds__(kSetupThreads) k_low_setup(Geometry g, LowSetup ls, const double* __restrict__ a,
+                                                            const double* __restrict__ c,
+                                                            const double* __restrict__ lamx,
+                                                            const double* __restrict__ lamz) {
+  low_pivots(g, ls, blockIdx.x * blockDim.x + threadIdx.x, a, c, lamx, lamz);
+}
+
+// With the low modes' pivots by its first CTAs: both are chains of FP64 divisions, side by side.
+__global__ void __launch_bounds__(kSetupThreads) k_reduced_setup(Geometry g, LowSetup ls, int nlow, int P, int m, int trunc,
+                                                      const double* __restrict__ a,
                                                       const double* __restrict__ c, const double* __restrict__ lamx,
                                                       const double* __restrict__ lamz, float* __restrict__ tab) {
+  if ((int)blockIdx.x < nlow) {
+    low_pivots(g, ls, blockIdx.x * blockDim.x + threadIdx.x, a, c, lamx, lamz);
+    return;
+  }
   const int nsys = g.nz * g.ncols;
-  const int sys = blockIdx.x * blockDim.x + threadIdx.x;
+  const int sys = ((int)blockIdx.x - nlow) * blockDim.x + threadIdx.x;
   if (sys >= nsys) return;
   int kx, kz;
   sys_to_mode(sys, g.ncols, kx, kz);
@@ -405,15 +441,16 @@ __global__ void __launch_bounds__(128) k_reduced_setup(Geometry g, int P, int m,
 }
 
 template <int M>
-__global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S, int low, const float* __restrict__ a,
-                                                        const float* __restrict__ c, const double* __restrict__ lamx,
-                                                        const double* __restrict__ lamz, const float* __restrict__ rtab,
-                                                        cplx<float>* __restrict__ spec, SideArgs sd) {
+__global__ void __launch_bounds__(256, 2)
+    k_tridiag_reg(const __grid_constant__ Geometry g, int P, int S, int low, const float* __restrict__ a,
+                  const float* __restrict__ c, const double* __restrict__ lamx, const double* __restrict__ lamz,
+                  const float* __restrict__ rtab, cplx<float>* __restrict__ spec,
+                  const __grid_constant__ SideArgs sd) {
   // shared: the interface arrays (6 x NT floats), the CTA's slice of the reduced-system table
   // (5 (P-1) S floats, [i][k][s]), then the blocks' rows [row][thread]
   extern __shared__ __align__(16) float red_s[];
   if ((int)blockIdx.x < sd.n) {
-    low_system<float>(g, sd, spec, blockIdx.x, reinterpret_cast<unsigned char*>(red_s));
+    low_system<float>(g, sd, spec, blockIdx.x);
     return;
   }
   enum { R_XFR, R_XFI, R_XLR, R_XLI, R_ZR, R_ZI };
@@ -539,19 +576,19 @@ __global__ void __launch_bounds__(256, 2) k_tridiag_reg(Geometry g, int P, int S
 // memory, twice: into system-major order, where the P interfaces of a system are P lanes of a
 // warp and the reduced system is the pair of warp scans of tridiag_scan.cuh, and back.
 //
-// What bounds it is HBM and, on small grids, the latency of one load and two sweeps.  The form before staged the rows in shared memory and
-// swept them there with 14 shared-memory wavefronts per warp and row (batch of 64 solves of 48 to
+// What bounds it is HBM and, on small grids, the latency of one load and two sweeps.  The form
+// before staged the rows in shared memory and swept them there with 14 shared-memory wavefronts per warp and row (batch of 64 solves of 48 to
 // 192 rows: 2678 us, 2520 with this kernel at every block height).
 template <int M> constexpr int rows_min_ctas() { return M <= 8 ? 4 : (M <= 12 ? 3 : 2); }
 
 template <int M>
 __global__ void __launch_bounds__(256, rows_min_ctas<M>())
-    k_tridiag_rows(Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
+    k_tridiag_rows(const __grid_constant__ Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
                    const double* __restrict__ lamx, const double* __restrict__ lamz, const float* __restrict__ rtab,
-                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, SideArgs sd) {
+                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, const __grid_constant__ SideArgs sd) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if ((int)blockIdx.x < sd.n) {
-    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
+    low_system<float>(g, sd, spec, blockIdx.x);
     return;
   }
   constexpr int MS = M | 1;   // odd stride of a block's (a, c) pairs
@@ -680,12 +717,12 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 
 template <int M, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT)
-    k_tridiag_tile(Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
+    k_tridiag_tile(const __grid_constant__ Geometry g, int lgP, int low, const float* __restrict__ a, const float* __restrict__ c,
                    const double* __restrict__ lamx, const double* __restrict__ lamz, const float* __restrict__ rtab,
-                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, SideArgs sd) {
+                   cplx<float>* __restrict__ spec, int kx_lo, int kx_hi, int width, const __grid_constant__ SideArgs sd) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if ((int)blockIdx.x < sd.n) {
-    low_system<float>(g, sd, spec, blockIdx.x, smem_raw);
+    low_system<float>(g, sd, spec, blockIdx.x);
     return;
   }
   static_assert(M % 2 == 0, "whole rounds of pair copies");
@@ -791,24 +828,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
   }
 }
 
-// Pivots of the modes solved apart, one thread per system of the list (low_system's order):
-// rb[sys ny + j] = 1 / beta_j by the margin recurrence, in FP64.
-__global__ void __launch_bounds__(32) k_low_setup(Geometry g, int n, int low, const double* __restrict__ a,
-                                                  const double* __restrict__ c, const double* __restrict__ lamx,
-                                                  const double* __restrict__ lamz, double* __restrict__ rb) {
-  const int sys = blockIdx.x * blockDim.x + threadIdx.x;
-  if (sys < 1 || sys >= n) return;
-  const int kx = sys % (low + 1), q = sys / (low + 1);
-  const int kz = q <= low ? q : g.nz - (q - low);
-  const double sigma = -(lamx[kx] + lamz[kz]);
-  double e = 0.0, r = 0.0;
-  for (int j = 0; j < g.ny; ++j) {
-    e = j > 0 ? sigma + a[j] * e * r : sigma;
-    r = 1.0 / (c[j] + e);
-    rb[(size_t)sys * g.ny + j] = r;
-  }
-}
-
 // ------------------------------------------------------------------------------ launchers
 template <typename K>
 static cudaError_t prep(K kernel, size_t smem) {
@@ -821,16 +840,20 @@ static cudaError_t prep(K kernel, size_t smem) {
 static constexpr size_t kSideFusedBytes = 48 * 1024;
 
 template <typename TD>
-__global__ void __launch_bounds__(128) k_tridiag_side(Geometry g, SideArgs sd, cplx<TD>* __restrict__ spec) {
+__global__ void __launch_bounds__(128) k_tridiag_side(const __grid_constant__ Geometry g, const __grid_constant__ SideArgs sd, cplx<TD>* __restrict__ spec) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  low_system<TD>(g, sd, spec, blockIdx.x, smem_raw);
+  low_system<TD>(g, sd, spec, blockIdx.x);
 }
 
-// Groups of sd for CTAs of `threads` threads: a warp per system up to 256 rows, else 128 threads.
+// Groups of sd for CTAs of `threads` threads: a warp per system up to 256 rows, else 128 threads; at
+// most two systems to a CTA, since the groups of a CTA share the two FP64 instructions per clock of
+// their SM (162x90x108 solve 39.2 -> 37.2 us, 192x96x192 pass 18 -> 16 us with eight; the batch of 64 solves
+// does not see the difference).
 static void side_groups(const Geometry& g, SideArgs& sd, int threads) {
   const int whole = threads & ~31;
   sd.threads = g.ny <= 256 ? 32 : (whole < 128 ? whole : 128);
   sd.per = whole / sd.threads;
+  if (sd.per > kLowMaxGroups) sd.per = kLowMaxGroups;
   while (sd.per > 1 && (size_t)16 * g.ny * sd.per > kSideFusedBytes) --sd.per;
   sd.n = (sd.nsys + sd.per - 1) / sd.per;
 }
@@ -873,9 +896,9 @@ SideArgs side_args(const DevTables& tb, int low, GaugeMode gauge) {
 }
 
 cudaError_t launch_low_setup(const Geometry& g, const DevTables& tb, int low, cudaStream_t st) {
-  if (low < 1) return cudaSuccess;   // low = 0: the (0, 0) mode only
-  const int n = (low + 1) * (2 * low + 1);
-  k_low_setup<<<(n + 31) / 32, 32, 0, st>>>(g, n, low, tb.d.a, tb.d.c, tb.lamx, tb.lamz, tb.low_rb);
+  const LowSetup ls = low_setup(tb, low);
+  if (ls.n == 0) return cudaSuccess;
+  k_low_setup<<<low_blocks(ls), kSetupThreads, 0, st>>>(g, ls, tb.d.a, tb.d.c, tb.lamx, tb.lamz);
   return cudaGetLastError();
 }
 
@@ -913,12 +936,14 @@ size_t reduced_table_bytes(const Geometry& g, int parts) {
   return parts > 1 ? (size_t)5 * (parts - 1) * g.nz * g.ncols * sizeof(float) : 0;
 }
 
-cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int parts, bool trunc, float* tab,
+cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int parts, bool trunc, int low, float* tab,
                                  cudaStream_t st) {
-  if (parts <= 1) return cudaSuccess;
+  if (parts <= 1) return launch_low_setup(g, tb, low, st);
   const int nsys = g.nz * g.ncols;
-  k_reduced_setup<<<(nsys + 127) / 128, 128, 0, st>>>(g, parts, g.ny / parts, trunc ? 1 : 0, tb.d.a, tb.d.c, tb.lamx,
-                                                       tb.lamz, tab);
+  const LowSetup ls = low_setup(tb, low);
+  const int nlow = low_blocks(ls);
+  k_reduced_setup<<<nlow + (nsys + kSetupThreads - 1) / kSetupThreads, kSetupThreads, 0, st>>>(
+      g, ls, nlow, parts, g.ny / parts, trunc ? 1 : 0, tb.d.a, tb.d.c, tb.lamx, tb.lamz, tab);
   return cudaGetLastError();
 }
 
