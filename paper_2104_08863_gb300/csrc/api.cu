@@ -42,11 +42,20 @@ bool factor(int L, FftFactors& f) {
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Automatic PDD partition.  FP64 (factored kernel, FP64-issue bound): the most blocks with at
-// least 48 rows each.  FP32 (register kernel): blocks of the largest supported height <= 24.
+// least 48 rows each.  FP32 (register kernels): the fewest blocks of one of the tiled heights <= 24,
+// unless those are more than 32 and a partition into at most 32 blocks of any height <= 24 exists:
+// 253 rows are then 11 blocks of 23 and not 253 of one row, whose reduced system is a serial chain of
+// 252 interfaces on 8-byte row segments (an FP32 solve and its adjoint at 1536x253x27: 1585 us, now
+// 124).
 int auto_parts(int ny, int precision) {
   if (precision != PP_FP64) {
-    for (int P = 1; P <= 256; ++P)
-      if (ny % P == 0 && ny / P <= 24 && pp::reg_tridiag_ok(ny, P)) return P;
+    int tiled = 0;
+    for (int P = 1; P <= 256 && !tiled; ++P)
+      if (ny % P == 0 && ny / P <= 24 && pp::reg_tridiag_ok(ny, P)) tiled = P;
+    if (tiled > 32)
+      for (int P = 1; P <= 32; ++P)
+        if (pp::reg_kernel_ok(ny, P)) return P;
+    if (tiled) return tiled;
   }
   int best = 1;
   for (int P = 2; P <= 32; ++P)
@@ -213,6 +222,7 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   pl->tridiag = d->tridiag;
   pl->flags = d->flags;
   if (!factor(g.M, pl->fm) || !factor(g.nz, pl->fz) || g.M < 2) { delete pl; return PS_EUNSUPPORTED; }
+  const bool auto_part = d->tridiag != PT_THOMAS && d->pdd_parts <= 0;
   int P = 1;
   if (d->tridiag == PT_THOMAS) P = 1;
   else if (d->pdd_parts > 0) P = d->pdd_parts;
@@ -353,7 +363,8 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
     const size_t nsys = (size_t)g.nz * g.ncols;
     pl->off_tri = off;
     // FP32 plans whose blocks fit in registers build their factors on the fly (no tables)
-    pl->has_tri = d->precision == PP_FP64 || !pp::reg_tridiag_ok(ny, P);
+    const bool any_height = auto_part && pp::reg_kernel_ok(ny, P);   // chosen by auto_parts
+    pl->has_tri = d->precision == PP_FP64 || !(pp::reg_tridiag_ok(ny, P) || any_height);
     if (d->precision == PP_FP64) off = align_up(off + 8 * nsys * (4 * (size_t)ny + 4 * (size_t)P), 256);
     else if (pl->has_tri) off = align_up(off + 4 * nsys * (2 * (size_t)ny + 4 * (size_t)P), 256);
     pl->off_red = off;

@@ -159,6 +159,9 @@ __host__ __device__ inline bool reg_tridiag_ok(int ny, int P) {
   const int m = ny / P;
   return m == 1 || m == 2 || m == 3 || m == 4 || m == 6 || m == 8 || m == 12 || m == 16 || m == 24;
 }
+// What the register kernel itself takes: the automatic partition of row counts that the heights above
+// would cut into more than 32 blocks uses any height up to 24 (auto_parts).
+__host__ __device__ inline bool reg_kernel_ok(int ny, int P) { return P >= 1 && P <= 256 && ny % P == 0 && ny / P <= 24; }
 __host__ __device__ inline int reg_systems_per_cta(int P) { return P >= 256 ? 1 : 256 / P; }
 // [kx_lo, kx_hi): the kx columns solved (kx_hi < 0: all); a partial range is supported by the
 // warp-scan variant only (P a power of two <= 32), with kx_lo a multiple of
@@ -260,7 +263,7 @@ struct poisson_plan_s {
   // workspace layout (byte offsets)
   size_t off_spec, off_pbuf, off_pbuf2, off_r1, off_low, off_tables, off_status, off_acc, off_tri, off_red,
       ws_bytes;
-  bool has_tri;   // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans with m = ny/P outside the register kernel's set)
+  bool has_tri;   // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans whose caller names blocks of a height that is not tiled, or above 24 rows)
   size_t tab_offsets[32];
   unsigned char* ws;
   pp::DevTables dt;

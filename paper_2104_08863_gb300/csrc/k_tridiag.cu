@@ -440,8 +440,10 @@ __global__ void __launch_bounds__(kSetupThreads) k_reduced_setup(Geometry g, Low
   }
 }
 
+// More CTAs to an SM at small heights, whose many interfaces make the reduced system a long chain
+// (1536x536x486, 67 blocks of 8: solve 6155 us with 3 CTAs, 6077 with 4).
 template <int M>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, M <= 8 ? 4 : (M <= 12 ? 3 : 2))
     k_tridiag_reg(const __grid_constant__ Geometry g, int P, int S, int low, const float* __restrict__ a,
                   const float* __restrict__ c, const double* __restrict__ lamx, const double* __restrict__ lamz,
                   const float* __restrict__ rtab, cplx<float>* __restrict__ spec,
@@ -985,7 +987,7 @@ static cudaError_t launch_tile(const Geometry& g, const DevTables& tb, int parts
 
 cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int parts, int low_modes,
                                    cplx<float>* spec, SideArgs sd, cudaStream_t st, int kx_lo, int kx_hi) {
-  if (!reg_tridiag_ok(g.ny, parts)) return cudaErrorNotSupported;
+  if (!reg_kernel_ok(g.ny, parts)) return cudaErrorNotSupported;
   const int m = g.ny / parts;
   const int S = reg_systems_per_cta(parts);
   if (kx_hi < 0) kx_hi = g.ncols;
@@ -1031,8 +1033,10 @@ cudaError_t launch_tridiag_reg_f32(const Geometry& g, const DevTables& tb, int p
     break;                                                                                                      \
   }
   switch (m) {
-    PP_REG_CASE(1) PP_REG_CASE(2) PP_REG_CASE(3) PP_REG_CASE(4) PP_REG_CASE(6) PP_REG_CASE(8)
-    PP_REG_CASE(12) PP_REG_CASE(16) PP_REG_CASE(24)
+    PP_REG_CASE(1) PP_REG_CASE(2) PP_REG_CASE(3) PP_REG_CASE(4) PP_REG_CASE(5) PP_REG_CASE(6)
+    PP_REG_CASE(7) PP_REG_CASE(8) PP_REG_CASE(9) PP_REG_CASE(10) PP_REG_CASE(11) PP_REG_CASE(12)
+    PP_REG_CASE(13) PP_REG_CASE(14) PP_REG_CASE(15) PP_REG_CASE(16) PP_REG_CASE(17) PP_REG_CASE(18)
+    PP_REG_CASE(19) PP_REG_CASE(20) PP_REG_CASE(21) PP_REG_CASE(22) PP_REG_CASE(23) PP_REG_CASE(24)
     default: return cudaErrorNotSupported;
   }
 #undef PP_REG_CASE
