@@ -2,10 +2,10 @@
 //
 // A batched plan holds one sub-plan per instance and carves their workspaces out of one caller
 // allocation.  poisson_solve_batched captures, once, a CUDA graph and replays it while the
-// pointers stay the same.  The graph holds either one branch per instance, forked from the
-// caller's stream and holding that instance's kernel sequence (the same pipeline as
-// poisson_solve), so that small instances run concurrently and the host pays one graph launch
-// per batch instead of ~7 launches per instance; or (POISSON_BATCH_PERSISTENT, every instance
+// pointers stay the same.  The graph holds either branches forked from the caller's stream, each with
+// the kernel sequences of one instance or of several in turn (the same pipeline as poisson_solve; see
+// branch_chains), so that instances run concurrently and the host pays one graph launch
+// per batch instead of ~6 launches per instance; or (POISSON_BATCH_PERSISTENT, every instance
 // supported) one persistent kernel over a device work list (batch_persistent.cu).
 //
 // poisson_autotune picks, per grid, the PDD partition count and the FFT tiling (compile-time
@@ -33,6 +33,42 @@ void drop_graph(poisson_plan_s* pl) {
 }  // namespace
 
 namespace pp {
+
+// The instances of each branch of the graph, in order.  A solve writes and reads its half spectrum
+// five times over.  With a branch to each instance all spectra are in flight at once, and once they
+// do not fit in the L2 (129 MB) every pass goes to memory; the FP32 forms, which memory bounds, then
+// take only as many branches as keep about 48 MB of spectra in flight (3 at least, so that one solve's
+// kernel fills the SMs that another's last wave leaves).  64 FP32 solves of 1.0 GB of spectra: 64
+// branches 2294 us, 8 2056, 4 1951, 3 1935, 2 2011, 1 2607; 41 of 0.39 GB: 41 branches 918, 10 793,
+// 4 752, 3 786; 19 refined of 0.26 GB: 1755, 10 1725, 4 1597, 2 1726.  Below that line more branches
+// win (64 solves of 0.1 MB: 144 us, 4 branches 263; 12 of 106 MB in all: 224, 3 branches 252), and
+// FP64, bound by its issue rate, does not see a difference (23 of 0.9 GB: 12063, 3 branches 12078).
+static std::vector<std::vector<int>> branch_chains(const poisson_plan_s* pl) {
+  const int n = (int)pl->children.size();
+  std::vector<size_t> bytes(n);
+  std::vector<int> order(n);
+  size_t total = 0;
+  bool fp64 = false;
+  for (int i = 0; i < n; ++i) {
+    const poisson_plan_s* c = pl->children[i];
+    fp64 = fp64 || c->precision == PP_FP64;
+    bytes[i] = (size_t)c->g.pitch * c->g.nz * c->g.ny * (c->precision == PP_FP64 ? 16 : 8);
+    total += bytes[i];
+    order[i] = i;
+  }
+  size_t nb = n;
+  if (!fp64 && total > ((size_t)128 << 20)) nb = std::min(nb, std::max<size_t>(3, ((size_t)48 << 20) * n / total));
+  // longest first onto the shortest branch; an instance's launches cost about as much as 4 MB
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return bytes[x] > bytes[y]; });
+  std::vector<std::vector<int>> chains(nb);
+  std::vector<size_t> load(nb, 0);
+  for (int i : order) {
+    const size_t b = std::min_element(load.begin(), load.end()) - load.begin();
+    chains[b].push_back(i);
+    load[b] += bytes[i] + ((size_t)4 << 20);
+  }
+  return chains;
+}
 
 // Instance table and work list of the persistent launch, built once per workspace.  Items are
 // ordered pass by pass; within a pass the instances go largest first.
@@ -242,7 +278,9 @@ poisson_status poisson_solve_batched(poisson_plan_t pl, const void* const* rhs, 
   }
   if (!same) {
     drop_graph(pl);
-    while ((int)pl->forks.size() < n + 1) {   // n branches + the capture stream
+    const std::vector<std::vector<int>> chains = pp::branch_chains(pl);
+    const int nb = (int)chains.size();
+    while ((int)pl->forks.size() < nb + 1) {   // the branches + the capture stream
       cudaStream_t s;
       cudaEvent_t e;
       if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return PS_ECUDA;
@@ -250,7 +288,7 @@ poisson_status poisson_solve_batched(poisson_plan_t pl, const void* const* rhs, 
       pl->forks.push_back(s);
       pl->fork_ev.push_back(e);
     }
-    if (pl->fork_ev.size() < (size_t)n + 1) {
+    if (pl->fork_ev.size() < (size_t)nb + 1) {
       cudaEvent_t e;
       if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return PS_ECUDA;
       pl->fork_ev.push_back(e);
@@ -265,19 +303,22 @@ poisson_status poisson_solve_batched(poisson_plan_t pl, const void* const* rhs, 
     }
     // Capture on a library stream (the caller's may be the legacy default stream, which cannot
     // be captured); the graph is then launched on the caller's stream.
-    cudaEvent_t e0 = pl->fork_ev[n];
-    cudaStream_t cap = pl->forks[n];
+    cudaEvent_t e0 = pl->fork_ev[nb];
+    cudaStream_t cap = pl->forks[nb];
     if (cudaStreamSynchronize(st) != cudaSuccess) return PS_ECUDA;
     if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return PS_ECUDA;
     poisson_status s = PS_OK;
     if (cudaEventRecord(e0, cap) != cudaSuccess) s = PS_ECUDA;
-    for (int i = 0; s == PS_OK && i < n; ++i) {
-      poisson_plan_s* c = pl->children[i];
-      cudaStream_t fs = pl->forks[i];
+    for (int b = 0; s == PS_OK && b < nb; ++b) {
+      cudaStream_t fs = pl->forks[b];
       if (cudaStreamWaitEvent(fs, e0, 0) != cudaSuccess) { s = PS_ECUDA; break; }
-      s = pp::solve_on_workspace(c, c->ws, c->dt, rhs[i], p[i], fs);
+      for (int i : chains[b]) {
+        poisson_plan_s* c = pl->children[i];
+        s = pp::solve_on_workspace(c, c->ws, c->dt, rhs[i], p[i], fs);
+        if (s != PS_OK) break;
+      }
       if (s != PS_OK) break;
-      if (cudaEventRecord(pl->fork_ev[i], fs) != cudaSuccess || cudaStreamWaitEvent(cap, pl->fork_ev[i], 0) != cudaSuccess)
+      if (cudaEventRecord(pl->fork_ev[b], fs) != cudaSuccess || cudaStreamWaitEvent(cap, pl->fork_ev[b], 0) != cudaSuccess)
         s = PS_ECUDA;
     }
     cudaGraph_t graph = nullptr;
