@@ -57,7 +57,7 @@ static std::vector<std::vector<int>> branch_chains(const poisson_plan_s* pl) {
     order[i] = i;
   }
   size_t nb = n;
-  if (!fp64 && total > ((size_t)128 << 20)) nb = std::min(nb, std::max<size_t>(3, ((size_t)48 << 20) * n / total));
+  if (!fp64 && !fits_l2(total)) nb = std::min(nb, std::max<size_t>(3, ((size_t)48 << 20) * n / total));
   // longest first onto the shortest branch; an instance's launches cost about as much as 4 MB
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return bytes[x] > bytes[y]; });
   std::vector<std::vector<int>> chains(nb);

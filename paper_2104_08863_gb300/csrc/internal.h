@@ -10,6 +10,9 @@
 
 namespace pp {
 
+// Whether data of this size stays in the L2 (129 MB) between the pass that writes it and the next.
+inline bool fits_l2(size_t bytes) { return bytes < ((size_t)128 << 20); }
+
 // Device-side table pointers for one arithmetic type T.
 template <typename T> struct Tables {
   const cplx<T>* tw_m;     // e^{-2 pi i t / M}, t < M   (half-length complex FFT in x)

@@ -334,11 +334,14 @@ cudaError_t launch_inv_x_reg(const Geometry& g, const DevTables& tb, InvMode mod
   const int nlines = g.ny * g.nz;
   const dim3 grid((nlines + C::LPB - 1) / C::LPB);
   cudaError_t e = cudaSuccess;
+  // A spectrum that the L2 holds is taken from its last line to the first, beginning with what the
+  // inverse z-transform wrote last (384x192x256, 76 MB: 38.8 -> 35.0 us).
+  const bool rev = fits_l2((size_t)nlines * g.pitch * sizeof(cplx<float>));
 #define PP_INVR(MODEV, ACCV)                                                                       \
   {                                                                                                \
     auto k = k_inv_x_reg<TO, M, MODEV, ACCV>;                                                      \
     if ((e = set_smem(k, C::SMEM)) != cudaSuccess) return e;                                       \
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tb.f, spec, out, scale, nlines, tb.dy, tb.acc, pair); \
+    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tb.f, spec, out, scale, nlines, tb.dy, tb.acc, pair, rev); \
   }
   if (mode == INV_ACCUM) {
     if (accumulate) PP_INVR(INV_ACCUM, true) else PP_INVR(INV_ACCUM, false)

@@ -288,15 +288,21 @@ __device__ __forceinline__ void inv_x_reg_tile(const Geometry& g, const Tables<f
   }
 }
 
+// Lines up to 2 kInvRevMaxM points can be taken from the last to the first (rev).  Beyond, a tile
+// number that is not the block's costs a register more than there is (768x384x512: 261 -> 271 us).
+constexpr int kInvRevMaxM = 256;
+
 // Three CTAs per SM (85 registers): the inverse's pass 2 streams its results straight from
 // registers, and the extra resident warps hide that more than the spills it causes cost (1.9 vs
 // 2.1 ms per pass at 1536x768x1024; the forward and the z-transform measured the other way).
 template <typename TO, int M, int MODE, bool ACC>
 __global__ void __launch_bounds__(XReg<M>::THREADS, 3)
     k_inv_x_reg(Geometry g, Tables<float> tt, const cplx<float>* __restrict__ spec, TO* __restrict__ out, double scl,
-                int nlines, const double* __restrict__ dy, double* __restrict__ acc, PairArgs pair) {
+                int nlines, const double* __restrict__ dy, double* __restrict__ acc, PairArgs pair, bool rev) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  inv_x_reg_tile<TO, M, MODE, ACC>(g, tt, spec, out, scl, nlines, dy, acc, pair, blockIdx.x, smem_raw);
+  int tile = blockIdx.x;
+  if constexpr (M <= kInvRevMaxM) tile = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  inv_x_reg_tile<TO, M, MODE, ACC>(g, tt, spec, out, scl, nlines, dy, acc, pair, tile, smem_raw);
 }
 
 }  // namespace pp

@@ -74,15 +74,18 @@ static cudaError_t launch_z_reg(const Geometry& g, const Tables<T>& tt, int sign
   using C = ZReg<T, NZ>;
   if (kx_lo % C::W || kx_lo < 0 || kx_hi > g.ncols || kx_hi <= kx_lo) return cudaErrorInvalidValue;
   const dim3 grid((kx_hi - kx_lo + C::W - 1) / C::W, g.ny);
+  // The forward transform of a spectrum that the L2 holds goes from the last plane to the first: it
+  // begins with what the forward x-transform wrote last (384x192x256, 76 MB: 28.5 -> 26.5 us).
+  const bool rev = sign < 0 && fits_l2((size_t)g.ny * g.nz * g.pitch * sizeof(cplx<T>));
   cudaError_t e;
   if (sign < 0) {
     auto k = k_fft_z_reg<T, NZ, -1>;
     if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi, rev);
   } else {
     auto k = k_fft_z_reg<T, NZ, 1>;
     if ((e = set_smem_once(k, C::SMEM)) != cudaSuccess) return e;
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi);
+    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tt, spec, kx_lo, kx_hi, false);
   }
   return cudaGetLastError();
 }

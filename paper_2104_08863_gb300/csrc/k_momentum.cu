@@ -101,7 +101,9 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
   RowCoef<T>* rc = reinterpret_cast<RowCoef<T>*>(smem_raw);
   __shared__ MVec<T, V> edge[SHARE ? 2 : 1][SHARE ? 2 * MOM_THREADS : 1];   // [buffer][u-w, v-w][thread]
   const int nx = g.nx, ny = g.ny, nz = g.nz;
-  const int j0 = jlo + blockIdx.z * jc;
+  // the second stage begins with the rows that the first wrote last, while they are in the L2 (512x384x512
+  // FP64: 11.55 -> 11.46 ms)
+  const int j0 = jlo + (BASE ? gridDim.z - 1 - blockIdx.z : blockIdx.z) * jc;
   const int j1 = min(jhi, j0 + jc);
   for (int r = threadIdx.y * blockDim.x + threadIdx.x; r < j1 - j0; r += blockDim.x * blockDim.y) {
     const int j = j0 + r;

@@ -93,9 +93,10 @@ __device__ __forceinline__ void z_reg_tile(const Geometry& g, const Tables<T>& t
 template <typename T, int NZ, int SIGN>
 __global__ void __launch_bounds__(ZReg<T, NZ>::THREADS, 512 / ZReg<T, NZ>::THREADS) k_fft_z_reg(Geometry g, Tables<T> tt,
                                                                       cplx<T>* __restrict__ spec, int kx_lo,
-                                                                      int kx_hi) {
+                                                                      int kx_hi, bool rev) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  z_reg_tile<T, NZ, SIGN>(g, tt, spec, kx_lo, kx_hi, blockIdx.x, blockIdx.y, smem_raw);
+  z_reg_tile<T, NZ, SIGN>(g, tt, spec, kx_lo, kx_hi, blockIdx.x, rev ? gridDim.y - 1 - blockIdx.y : blockIdx.y,
+                          smem_raw);
 }
 
 }  // namespace pp
