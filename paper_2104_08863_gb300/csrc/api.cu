@@ -98,10 +98,11 @@ bool spec_is_fp64(const poisson_plan_s* pl) { return pl->precision == PP_FP64; }
 }  // namespace
 
 namespace pp {
-cudaError_t ensure_smem_limit(const void* kernel, size_t bytes) {
+cudaError_t ensure_smem_limit(const void* kernel, size_t bytes, size_t static_bytes) {
   static std::mutex mu;
   static std::unordered_map<const void*, size_t> granted;
-  if (bytes <= 47 * 1024) return cudaSuccess;   // 48 KB less room for a kernel's static shared memory
+  // 48 KB, static shared memory included (1 KB of it for kernels that do not state theirs)
+  if (bytes + static_bytes <= 47 * 1024) return cudaSuccess;
   std::lock_guard<std::mutex> lock(mu);
   auto it = granted.find(kernel);
   if (it != granted.end() && it->second >= bytes) return cudaSuccess;

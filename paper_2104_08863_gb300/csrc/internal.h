@@ -80,7 +80,7 @@ struct LaunchCount {
 
 // Raise a kernel's dynamic shared-memory limit to at least `bytes`, once per kernel (a registry
 // keyed by the kernel's address), so that the attribute call does not recur inside stream capture.
-cudaError_t ensure_smem_limit(const void* kernel, size_t bytes);
+cudaError_t ensure_smem_limit(const void* kernel, size_t bytes, size_t static_bytes = 0);
 
 // --- launchers (return cudaGetLastError() after the launch) --------------------------
 enum FwdMode { FWD_PLAIN = 0, FWD_DIV = 1, FWD_RESID = 2, FWD_GRADT = 3 };

@@ -31,12 +31,12 @@ namespace pp {
 
 // Rows per chunk: the split of the rows that minimises (CTAs on the busiest SM) x (rows + the
 // chunk's own start, worth about one row), so that small grids fill the SMs and large ones do not
-// repeat the start; at least 4 rows.  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks
+// repeat the start; at least 4 rows, at most 1024 (64 KB of coefficients).  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks
 // had at least 16 rows and filled 64 SMs.)
 int momentum_chunk_rows(long long tiles, int rows) {
   int best = rows;
   double cost = -1.0;
-  for (int chunks = 1; chunks <= (rows + 3) / 4; ++chunks) {
+  for (int chunks = (rows + 1023) / 1024; chunks <= (rows + 3) / 4; ++chunks) {
     const int jc = (rows + chunks - 1) / chunks;
     const long long ctas = tiles * ((rows + jc - 1) / jc);
     const double t = (double)((ctas + 151) / 152) * (jc + 1.0);
@@ -324,7 +324,7 @@ cudaError_t launch_momentum_v(const Geometry& g, const DevTables& tb, const MomA
   constexpr bool SH = sizeof(T) == 8;
   const bool base = a.bu != nullptr;
   const void* kern = base ? (const void*)k_momentum<T, V, true, SH> : (const void*)k_momentum<T, V, false, SH>;
-  const cudaError_t e = ensure_smem_limit(kern, smem);
+  const cudaError_t e = ensure_smem_limit(kern, smem, SH ? sizeof(MVec<T, V>) * 4 * MOM_THREADS : 0);
   if (e != cudaSuccess) return e;
   if (base) k_momentum<T, V, true, SH><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
   else k_momentum<T, V, false, SH><<<grid, block, smem, st>>>(g, a, mc, tb.d.inv_dy, tb.d.inv_h, tb.d.a, tb.d.c, jlo, jhi, jc);
