@@ -266,7 +266,9 @@ struct poisson_plan_s {
   // workspace layout (byte offsets)
   size_t off_spec, off_pbuf, off_pbuf2, off_r1, off_low, off_tables, off_status, off_acc, off_tri, off_red,
       ws_bytes;
-  bool has_tri;   // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans whose caller names blocks of a height that is not tiled, or above 24 rows)
+  // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans with blocks above 24 rows, or of a
+  // height outside reg_tridiag_ok that the caller named)
+  bool has_tri;
   size_t tab_offsets[32];
   unsigned char* ws;
   pp::DevTables dt;

@@ -253,8 +253,9 @@ __global__ void __launch_bounds__(256) k_tridiag_factored(const __grid_constant_
 // Thomas by scans: with the pivots in tables both sweeps are first-order linear recurrences with
 // coefficients in (0, 1) (see low_modes.cuh), so 8 lanes take contiguous rows of one system each
 // and the carries between them come from a 3-step scan of affine maps.  A warp holds 4 systems
-// (64-byte row segments), a CTA 8, so that a few hundred systems reach every SM.  Per row the eliminated value and the running product of the
-// coefficients (the weight of the carry) stay in the thread's own shared-memory column.
+// (64-byte row segments), a CTA 8, so that a few hundred systems reach every SM.  Per row the
+// eliminated value and the running product of the coefficients (the weight of the carry) stay in the
+// thread's own shared-memory column.
 //
 // Such a launch is bound by latency: one thread per system walks ny dependent rows twice (FP64
 // FMA: 65 clocks) with 544 to 20,000 threads on the GPU.  It issues 13 FP64 instructions per row
@@ -579,8 +580,9 @@ __global__ void __launch_bounds__(256, M <= 8 ? 4 : (M <= 12 ? 3 : 2))
 // warp and the reduced system is the pair of warp scans of tridiag_scan.cuh, and back.
 //
 // What bounds it is HBM and, on small grids, the latency of one load and two sweeps.  The form
-// before staged the rows in shared memory and swept them there with 14 shared-memory wavefronts per warp and row (batch of 64 solves of 48 to
-// 192 rows: 2678 us, 2520 with this kernel at every block height).
+// before staged the rows in shared memory and swept them there with 14 shared-memory wavefronts per
+// warp and row (batch of 64 solves of 48 to 192 rows, a branch of the graph to each: 2678 us, 2520 with
+// this kernel at every block height).
 template <int M> constexpr int rows_min_ctas() { return M <= 8 ? 4 : (M <= 12 ? 3 : 2); }
 
 template <int M>
@@ -698,8 +700,8 @@ __global__ void __launch_bounds__(256, rows_min_ctas<M>())
 // ---- FP32 PDD on tiles in shared memory (P >= 16, blocks of 12 rows and more) -------------------
 // The rows kernel's blocks and order, with the S = NT / P systems of a CTA staged in shared memory
 // as [row][s] by 16-byte asynchronous copies.  A thread keeps only 1/beta_i per row in registers
-// (64 in all), so that 1024 threads are resident where 4 registers per row allow 512: 32 warps hide the sweeps' latencies and one
-// CTA's copies overlap the other's sweeps.  The forward sweep stores rb_i gg_i in place; once alpha
+// (64 in all), so that 1024 threads are resident where 4 registers per row allow 512: 32 warps hide
+// the sweeps' latencies and one CTA's copies overlap the other's sweeps.  The forward sweep stores rb_i gg_i in place; once alpha
 // is known a second one adds alpha rb_i gv_i (gv_i = a_i rb_{i-1} gv_{i-1} again), and the backward
 // sweep writes x_i to global memory as it goes: the operations of the rows kernel, bit for bit.
 //
@@ -842,7 +844,9 @@ static cudaError_t prep(K kernel, size_t smem) {
 static constexpr size_t kSideFusedBytes = 48 * 1024;
 
 template <typename TD>
-__global__ void __launch_bounds__(128) k_tridiag_side(const __grid_constant__ Geometry g, const __grid_constant__ SideArgs sd, cplx<TD>* __restrict__ spec) {
+__global__ void __launch_bounds__(128) k_tridiag_side(const __grid_constant__ Geometry g,
+                                                      const __grid_constant__ SideArgs sd,
+                                                      cplx<TD>* __restrict__ spec) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   low_system<TD>(g, sd, spec, blockIdx.x);
 }
