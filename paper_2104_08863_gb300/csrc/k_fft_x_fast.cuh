@@ -341,7 +341,7 @@ cudaError_t launch_inv_x_reg(const Geometry& g, const DevTables& tb, InvMode mod
   {                                                                                                \
     auto k = k_inv_x_reg<TO, M, MODEV, ACCV>;                                                      \
     if ((e = set_smem(k, C::SMEM)) != cudaSuccess) return e;                                       \
-    k<<<grid, C::THREADS, C::SMEM, st>>>(g, tb.f, spec, out, scale, nlines, tb.dy, tb.acc, pair, rev); \
+    k<<<grid, C::LAUNCH, C::SMEM, st>>>(g, tb.f, spec, out, scale, nlines, tb.dy, tb.acc, pair, rev);  \
   }
   if (mode == INV_ACCUM) {
     if (accumulate) PP_INVR(INV_ACCUM, true) else PP_INVR(INV_ACCUM, false)

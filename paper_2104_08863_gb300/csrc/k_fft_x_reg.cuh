@@ -26,6 +26,7 @@ template <int M> struct XReg {
   static constexpr int LPB0 = 256 / N1;
   static constexpr int LPB = LPB0 < 1 ? 1 : (LPB0 > 32 ? 32 : LPB0);
   static constexpr int THREADS = LPB * N1;
+  static constexpr int LAUNCH = (THREADS + 31) / 32 * 32;   // THREADS in whole warps
   static constexpr int B = N1 % 2 == 0 ? N1 + 1 : N1;
   static constexpr int LS = N2 * B > M ? N2 * B : M;   // per-line stride (>= M for the natural order)
   static constexpr int SMEM = LPB * LS * (int)sizeof(cplx<float>);
@@ -190,7 +191,8 @@ __global__ void __launch_bounds__(XReg<M>::THREADS, 3)
 
 // Inverse x-transform of the FP32 half spectrum into an FP32 field with the epilogue MODE
 // (INV_STORE, INV_ACCUM); ACC also adds the dy-weighted sum of the result to acc[1], formed in
-// double-float arithmetic on the FP32 units (one FP64 atomic per warp).
+// double-float arithmetic on the FP32 units (one FP64 atomic per warp).  The warp sums are shuffles of all
+// 32 lanes, so a launch with ACC has whole warps; the threads past C::THREADS add nothing.
 template <typename TO, int M, int MODE, bool ACC>
 __device__ __forceinline__ void inv_x_reg_tile(const Geometry& g, const Tables<float>& tt,
                                                const cplx<float>* __restrict__ spec, TO* __restrict__ out,
@@ -296,7 +298,7 @@ constexpr int kInvRevMaxM = 256;
 // registers, and the extra resident warps hide that more than the spills it causes cost (1.9 vs
 // 2.1 ms per pass at 1536x768x1024; the forward and the z-transform measured the other way).
 template <typename TO, int M, int MODE, bool ACC>
-__global__ void __launch_bounds__(XReg<M>::THREADS, 3)
+__global__ void __launch_bounds__(XReg<M>::LAUNCH, 3)
     k_inv_x_reg(Geometry g, Tables<float> tt, const cplx<float>* __restrict__ spec, TO* __restrict__ out, double scl,
                 int nlines, const double* __restrict__ dy, double* __restrict__ acc, PairArgs pair, bool rev) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
