@@ -10,9 +10,11 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <map>
 #include <mutex>
 #include <new>
-#include <unordered_map>
+#include <tuple>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -100,15 +102,37 @@ bool spec_is_fp64(const poisson_plan_s* pl) { return pl->precision == PP_FP64; }
 namespace pp {
 cudaError_t ensure_smem_limit(const void* kernel, size_t bytes, size_t static_bytes) {
   static std::mutex mu;
-  static std::unordered_map<const void*, size_t> granted;
+  static std::map<std::pair<int, const void*>, size_t> granted;   // (device, kernel): the limit is the device's
   // 48 KB, static shared memory included (1 KB of it for kernels that do not state theirs)
   if (bytes + static_bytes <= 47 * 1024) return cudaSuccess;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
-  auto it = granted.find(kernel);
-  if (it != granted.end() && it->second >= bytes) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) granted[kernel] = bytes;
+  size_t& have = granted[{dev, kernel}];
+  if (have >= bytes) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) have = bytes;
   return e;
+}
+
+cudaError_t resident_grid(const void* kernel, int threads, int smem, int& grid) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int>, int> cache;   // (device, kernel, shared memory)
+  cudaError_t e = ensure_smem_limit(kernel, (size_t)smem);
+  int dev = 0, sms = 0, per = 0;
+  if (e != cudaSuccess || (e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  int& known = cache[{dev, kernel, smem}];
+  if (!known) {
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, (size_t)smem)) != cudaSuccess)
+      return e;
+    if (per < 1) return cudaErrorInvalidConfiguration;
+    known = sms * per;
+  }
+  grid = known;
+  return cudaSuccess;
 }
 
 cudaError_t launch_plan_setup(const poisson_plan_s* pl, const DevTables& dt, unsigned char* ws, cudaStream_t st) {

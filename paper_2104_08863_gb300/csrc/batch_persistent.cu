@@ -317,19 +317,9 @@ int batch_zcols(const poisson_plan_s* c) {
 
 cudaError_t launch_batch_persistent(const BatchInst* inst, const BatchItem* items, int nitems, BatchCtl* ctl,
                                     size_t ctl_bytes, int* status, int selftest, cudaStream_t st) {
-  cudaError_t e = ensure_smem_limit((const void*)k_batch_persistent, (size_t)kBatchSmem);
+  int grid = 0;
+  cudaError_t e = resident_grid((const void*)k_batch_persistent, kBatchThreads, kBatchSmem, grid);
   if (e != cudaSuccess) return e;
-  static int grid = 0;
-  if (!grid) {
-    int dev = 0, sms = 0, per = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_persistent, kBatchThreads,
-                                                           (size_t)kBatchSmem)) != cudaSuccess)
-      return e;
-    if (per < 1) return cudaErrorInvalidConfiguration;
-    grid = sms * per;
-  }
   if ((e = cudaMemsetAsync(ctl, 0, ctl_bytes, st)) != cudaSuccess) return e;
   k_batch_persistent<<<grid, kBatchThreads, kBatchSmem, st>>>(inst, items, nitems, ctl, status, selftest);
   return cudaGetLastError();

@@ -78,9 +78,12 @@ struct LaunchCount {
   int n = 0;
 };
 
-// Raise a kernel's dynamic shared-memory limit to at least `bytes`, once per kernel (a registry
-// keyed by the kernel's address), so that the attribute call does not recur inside stream capture.
+// Raise a kernel's dynamic shared-memory limit on the current device to at least `bytes`, once per
+// device and kernel, so that the attribute call does not recur inside stream capture.
 cudaError_t ensure_smem_limit(const void* kernel, size_t bytes, size_t static_bytes = 0);
+// CTAs of a kernel that the current device holds at once (queried once per device, kernel and size); its
+// shared-memory limit is raised too.
+cudaError_t resident_grid(const void* kernel, int threads, int smem, int& grid);
 
 // --- launchers (return cudaGetLastError() after the launch) --------------------------
 enum FwdMode { FWD_PLAIN = 0, FWD_DIV = 1, FWD_RESID = 2, FWD_GRADT = 3 };

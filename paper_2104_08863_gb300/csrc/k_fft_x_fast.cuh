@@ -14,10 +14,6 @@
 // did not (divergence and x 26 -> 18 us, inverse 18 -> 12).
 #pragma once
 
-#include <map>
-#include <mutex>
-#include <utility>
-
 #include "bulk_copy.cuh"
 #include "fft_lf.cuh"
 #include "fft_static.cuh"
@@ -272,28 +268,6 @@ __global__ void __launch_bounds__(XPipe<TI, M>::THREADS, XPipe<TI, M>::MINB)
   }
 }
 
-// Resident CTAs of a kernel on the whole GPU (queried once per kernel and shared-memory size).
-template <typename K>
-inline cudaError_t resident_grid(K kernel, int threads, int smem, int& grid) {
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, int> cache;
-  cudaError_t e = ensure_smem_limit((const void*)kernel, (size_t)smem);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lock(mu);
-  auto key = std::make_pair((const void*)kernel, smem);
-  auto it = cache.find(key);
-  if (it != cache.end()) { grid = it->second; return cudaSuccess; }
-  int dev = 0, sms = 0, per = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, (size_t)smem)) != cudaSuccess)
-    return e;
-  if (per < 1) return cudaErrorInvalidConfiguration;
-  grid = sms * per;
-  cache[key] = grid;
-  return cudaSuccess;
-}
-
 template <typename K>
 inline cudaError_t set_smem(K kernel, int smem) {
   return ensure_smem_limit((const void*)kernel, (size_t)smem);
@@ -393,7 +367,7 @@ cudaError_t launch_fwd_x_stockham(const Geometry& g, const DevTables& tb, const 
       using P = XPipe<TI, M>;
       auto k = k_fwd_x_pipe<TI, M>;
       int rg = 0;
-      if ((e = resident_grid(k, P::THREADS, P::SMEM, rg)) != cudaSuccess) return e;
+      if ((e = resident_grid((const void*)k, P::THREADS, P::SMEM, rg)) != cudaSuccess) return e;
       const int ntiles = (nlines + P::LPB - 1) / P::LPB;
       k<<<rg < ntiles ? rg : ntiles, P::THREADS, P::SMEM, st>>>(g, args, tt, spec, 0, nlines, tb.status);
       return cudaGetLastError();

@@ -62,7 +62,7 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int bytes) {
   granted[{device, f}] = (size_t)bytes;
   return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) {
   ++occupancy_queries;
   *n = 2;
   return cudaSuccess;

@@ -29,7 +29,7 @@ def native(tmp_path_factory):
         b.build(force=True)
     out = str(tmp_path_factory.mktemp("recorded") / "libpoisson_recorded.so")
     inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(b._nvcc()))), "include")
-    subprocess.run([cxx, "-shared", "-fPIC", "-std=c++17", "-I" + inc, "-o", out, "-Wl,-Bsymbolic",
+    subprocess.run([cxx, "-shared", "-fPIC", "-std=c++17", "-I" + inc, "-o", out, "-Wl,-Bsymbolic,-z,defs",
                     os.path.join(HERE, "host", "fake_cudart.cpp"), *objs], check=True)
     L = ctypes.CDLL(out)
     L.fake_name.restype = ctypes.c_char_p
@@ -77,3 +77,22 @@ def test_gauge_sum_runs_in_whole_warps(native, half, generic):
     assert len(inv) == 3
     assert all(t % 32 == 0 for _, t, _ in inv[:2]), inv   # the last pass adds nothing up
     native[1].poisson_plan_destroy(h)
+
+
+def test_limits_and_grids_are_set_up_on_each_device(native):
+    """A kernel's shared-memory limit and the number of its CTAs that are resident belong to a device: the
+    second device's first call raises its own limits (a launch above 48 KB fails without) and asks for
+    its own grid size."""
+    L = native[1]
+    h, size = _plan(native, 1536, 96, 64, 2, tridiag=2, pdd_parts=4)   # piped x-transform, PDD blocks of 24 rows
+    queries = []
+    try:
+        for dev in (0, 1):
+            L.fake_set_device(dev)
+            kernels = _solve(native, h, size)
+            queries.append(L.fake_occupancy_queries())
+            assert any(smem > 48 << 10 for _, _, smem in kernels)
+    finally:
+        L.fake_set_device(0)
+        L.poisson_plan_destroy(h)
+    assert queries[0] == queries[1] == 1
