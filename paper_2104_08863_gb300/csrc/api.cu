@@ -147,9 +147,12 @@ DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base) {
   DevTables dt;
   unsigned char* tb = base + pl->off_tables;
   const size_t* to = pl->tab_offsets;
-  dt.d.tw_m = (const cplx<double>*)(tb + to[0]);
-  dt.d.tw_post = (const cplx<double>*)(tb + to[1]);
-  dt.d.tw_z = (const cplx<double>*)(tb + to[2]);
+  // the forms of the FP64 unit roots that the plan's image holds (poisson_plan_create)
+  const bool lf_x = spec_is_fp64(pl) && x_specialised(pl->g), lf_z = spec_is_fp64(pl) && z_specialised(pl->g);
+  auto roots = [&](bool held, int id) { return held ? (const cplx<double>*)(tb + to[id]) : nullptr; };
+  dt.d.tw_m = roots(!lf_x, 0);
+  dt.d.tw_post = roots(!lf_x, 1);
+  dt.d.tw_z = roots(!lf_z, 2);
   dt.d.a = (const double*)(tb + to[3]);
   dt.d.c = (const double*)(tb + to[4]);
   dt.f.tw_m = (const cplx<float>*)(tb + to[5]);
@@ -167,9 +170,9 @@ DevTables bind_tables(const poisson_plan_s* pl, unsigned char* base) {
   dt.f.inv_h = (const float*)(tb + to[17]);
   dt.f.a_lo = (const float*)(tb + to[18]);
   dt.f.c_lo = (const float*)(tb + to[19]);
-  dt.d.lf_m = (const cplx<double>*)(tb + to[20]);
-  dt.d.lf_post = (const cplx<double>*)(tb + to[21]);
-  dt.d.lf_z = (const cplx<double>*)(tb + to[22]);
+  dt.d.lf_m = roots(lf_x, 20);
+  dt.d.lf_post = roots(lf_x, 21);
+  dt.d.lf_z = roots(lf_z, 22);
   dt.f.lf_m = dt.f.lf_post = dt.f.lf_z = nullptr;
   dt.d.a_lo = nullptr;
   dt.d.c_lo = nullptr;
@@ -309,7 +312,10 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   size_t off = 0;
   size_t* to = pl->tab_offsets;
   auto slot = [&](int id, size_t bytes) { to[id] = off; off = align_up(off + bytes, 256); };
-  slot(0, 16 * (size_t)g.M);  slot(1, 16 * (size_t)(g.M + 1)); slot(2, 16 * (size_t)g.nz);
+  // FP64 plans on specialised lengths hold (cos, tan) tables in the place of the unit roots, so that a plan
+  // needs no more workspace than the unit roots alone would (poisson_solve_static_ws has 8 MB)
+  const bool lf_x = spec_is_fp64(pl) && x_specialised(g), lf_z = spec_is_fp64(pl) && z_specialised(g);
+  slot(0, lf_x ? 0 : 16 * (size_t)g.M); slot(1, lf_x ? 0 : 16 * (size_t)(g.M + 1)); slot(2, lf_z ? 0 : 16 * (size_t)g.nz);
   slot(3, 8 * (size_t)ny);    slot(4, 8 * (size_t)ny);
   slot(5, 8 * (size_t)g.M);   slot(6, 8 * (size_t)(g.M + 1)); slot(7, 8 * (size_t)g.nz);
   slot(8, 4 * (size_t)ny);    slot(9, 4 * (size_t)ny);
@@ -318,29 +324,29 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   slot(14, 8 * (size_t)ny);   slot(15, 8 * (size_t)(ny + 1));
   slot(16, 4 * (size_t)ny);   slot(17, 4 * (size_t)(ny + 1));
   slot(18, 4 * (size_t)ny);   slot(19, 4 * (size_t)ny);
-  const bool lf = spec_is_fp64(pl);   // (cos, tan) tables of the FP64 transforms
-  slot(20, lf ? 16 * (size_t)g.M : 0); slot(21, lf ? 16 * (size_t)(g.M / 2 + 1) : 0); slot(22, lf ? 16 * (size_t)g.nz : 0);
+  slot(20, lf_x ? 16 * (size_t)g.M : 0); slot(21, lf_x ? 16 * (size_t)(g.M / 2 + 1) : 0); slot(22, lf_z ? 16 * (size_t)g.nz : 0);
   const size_t tab_bytes = off;
   pl->host_tables.assign(tab_bytes, 0);
   auto& img = pl->host_tables;
-  put_cplx_table<double>(img, to[0], twm_r, twm_i);
-  put_cplx_table<double>(img, to[1], twp_r, twp_i);
-  put_cplx_table<double>(img, to[2], twz_r, twz_i);
-  if (lf) {
-    auto cos_tan = [&](int id, int L, int n) {
-      std::vector<double> c(n), t(n);
-      for (int q = 0; q < n; ++q) {
-        const UnitRoot w = unit_root(q, L);
-        // a quarter turn: cos as 2^-54 and tan as +-2^54, whose product is exact
-        c[q] = w.c != 0.0 ? w.c : 0x1p-54;
-        t[q] = w.c != 0.0 ? w.t : w.s * 0x1p54;
-      }
-      put_cplx_table<double>(img, to[id], c, t);
-    };
+  auto cos_tan = [&](int id, int L, int n) {
+    std::vector<double> c(n), t(n);
+    for (int q = 0; q < n; ++q) {
+      const UnitRoot w = unit_root(q, L);
+      // a quarter turn: cos as 2^-54 and tan as +-2^54, whose product is exact
+      c[q] = w.c != 0.0 ? w.c : 0x1p-54;
+      t[q] = w.c != 0.0 ? w.t : w.s * 0x1p54;
+    }
+    put_cplx_table<double>(img, to[id], c, t);
+  };
+  if (lf_x) {
     cos_tan(20, g.M, g.M);
     cos_tan(21, g.nx, g.M / 2 + 1);
-    cos_tan(22, g.nz, g.nz);
+  } else {
+    put_cplx_table<double>(img, to[0], twm_r, twm_i);
+    put_cplx_table<double>(img, to[1], twp_r, twp_i);
   }
+  if (lf_z) cos_tan(22, g.nz, g.nz);
+  else put_cplx_table<double>(img, to[2], twz_r, twz_i);
   put_real_table<double>(img, to[3], pl->a);
   put_real_table<double>(img, to[4], pl->c);
   put_cplx_table<float>(img, to[5], twm_r, twm_i);

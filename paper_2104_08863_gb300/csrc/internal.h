@@ -18,7 +18,8 @@ template <typename T> struct Tables {
   const cplx<T>* tw_m;     // e^{-2 pi i t / M}, t < M   (half-length complex FFT in x)
   const cplx<T>* tw_post;  // e^{-2 pi i k / Nx}, k <= M (real-to-complex packing)
   const cplx<T>* tw_z;     // e^{-2 pi i t / Nz}, t < Nz
-  // FP64 only (fft_lf.cuh): (cos, tan) of 2 pi t / M (t < M), 2 pi k / Nx (k <= M/2), 2 pi t / Nz
+  // FP64 only (fft_lf.cuh): (cos, tan) of 2 pi t / M (t < M), 2 pi k / Nx (k <= M/2), 2 pi t / Nz.
+  // An FP64 plan holds one form for x and one for z, that of the kernels which its lengths take (null: the other).
   const cplx<T>* lf_m;
   const cplx<T>* lf_post;
   const cplx<T>* lf_z;
@@ -73,6 +74,26 @@ struct Geometry {
   int generic_fft;   // 1: use the runtime-generic FFT kernels (POISSON_GENERIC_FFT)
   int selftest_wait; // 1: the bulk-copy-staged x-transform skips its first copy (POISSON_SELFTEST_WAIT)
 };
+
+// The half-lengths Nx/2 of the specialised x-transforms (k_fft_x_fast.cuh), in groups of one translation
+// unit each per pair of types, and the lengths Nz of the specialised z-transforms (k_fft_z_fast.cuh).
+#define PP_X_SIZES_A(F) F(8) F(9) F(12) F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64)
+#define PP_X_SIZES_B(F) F(72) F(81) F(96) F(108) F(128) F(144) F(162) F(192) F(216) F(243) F(256)
+#define PP_X_SIZES_C(F) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(1024)
+#define PP_Z_SIZES(F)                                                                                      \
+  F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64) F(72) F(81) F(96) F(108) F(128) F(144) F(162)      \
+  F(192) F(216) F(243) F(256) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(864) \
+  F(1024)
+#define PP_IS(N) || n == N
+inline bool x_specialised(const Geometry& g) {
+  const int n = g.M;
+  return !g.generic_fft && (false PP_X_SIZES_A(PP_IS) PP_X_SIZES_B(PP_IS) PP_X_SIZES_C(PP_IS));
+}
+inline bool z_specialised(const Geometry& g) {
+  const int n = g.nz;
+  return !g.generic_fft && (false PP_Z_SIZES(PP_IS));
+}
+#undef PP_IS
 
 struct LaunchCount {
   int n = 0;

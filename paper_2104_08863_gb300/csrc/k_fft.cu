@@ -153,6 +153,7 @@ cudaError_t launch_fwd_x(const Geometry& g, const DevTables& tb, const FftFactor
     else { PP_GROUPS(launch_fwd_x_fast_fd, (g, tb, mode, args, (cplx<float>*)spec, st)) }
     if (ef != cudaErrorNotSupported) return ef;
   }
+  if (!tabs<T>(tb).tw_m) return cudaErrorInvalidValue;   // the plan has the specialised form's tables
   const int nlines = g.ny * g.nz;
   const int lpb = lines_per_cta(fm.L);
   const size_t smem = 2 * (size_t)lpb * fm.L * sizeof(cplx<T>);
@@ -193,6 +194,7 @@ cudaError_t launch_inv_x(const Geometry& g, const DevTables& tb, const FftFactor
 #undef PP_GROUPS
     if (ef != cudaErrorNotSupported) return ef;
   }
+  if (!tabs<T>(tb).tw_m) return cudaErrorInvalidValue;
   const int nlines = g.ny * g.nz;
   const int lpb = lines_per_cta(fm.L);
   const size_t smem = 2 * (size_t)lpb * fm.L * sizeof(cplx<T>);
@@ -226,6 +228,7 @@ cudaError_t launch_fft_z(const Geometry& g, const DevTables& tb, const FftFactor
     const cudaError_t ef = launch_fft_z_fast<T>(g, tabs<T>(tb), sign, spec, st);
     if (ef != cudaErrorNotSupported) return ef;
   }
+  if (!tabs<T>(tb).tw_z) return cudaErrorInvalidValue;
   int W = (int)(64 / sizeof(cplx<T>));           // 64-byte row segments
   while (W * fz.L < 2048 && W < 32) W *= 2;       // small Nz: widen the tile
   if (W > g.ncols) W = g.ncols;

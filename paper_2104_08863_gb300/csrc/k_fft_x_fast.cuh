@@ -439,11 +439,6 @@ cudaError_t launch_inv_x_m(const Geometry& g, const DevTables& tb, const Tables<
   }
 }
 
-// The groups of half-lengths, one translation unit each per pair of types.
-#define PP_X_SIZES_A(F) F(8) F(9) F(12) F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64)
-#define PP_X_SIZES_B(F) F(72) F(81) F(96) F(108) F(128) F(144) F(162) F(192) F(216) F(243) F(256)
-#define PP_X_SIZES_C(F) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(1024)
-
 #define PP_X_CASE_FWD(MV) \
   case MV: return launch_fwd_x_m<T, TI, MV>(g, tb, tt, mode, args, spec, st);
 #define PP_X_CASE_INV(MV) \

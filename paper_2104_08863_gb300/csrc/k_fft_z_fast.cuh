@@ -113,11 +113,6 @@ static cudaError_t launch_z(const Geometry& g, const Tables<T>& tt, int sign, cp
   }
 }
 
-#define PP_Z_SIZES(F)                                                                                     \
-  F(16) F(18) F(24) F(27) F(32) F(36) F(48) F(54) F(64) F(72) F(81) F(96) F(108) F(128) F(144) F(162)     \
-  F(192) F(216) F(243) F(256) F(288) F(324) F(384) F(432) F(486) F(512) F(576) F(648) F(729) F(768) F(864) \
-  F(1024)
-
 // Returns cudaErrorNotSupported when Nz has no specialisation (the caller then uses the
 // generic kernel).  kx_hi < 0 means all columns.
 template <typename T>

@@ -96,3 +96,16 @@ def test_limits_and_grids_are_set_up_on_each_device(native):
         L.fake_set_device(0)
         L.poisson_plan_destroy(h)
     assert queries[0] == queries[1] == 1
+
+
+@pytest.mark.parametrize("flags", [0, 4])
+@pytest.mark.parametrize("nx,ny,nz", [(24, 100, 96), (108, 5, 432), (128, 55, 36), (128, 18, 108), (972, 33, 8)])
+def test_fp64_grids_that_just_fit_the_static_workspace(native, nx, ny, nz, flags):
+    """FP64 plans hold one form of the unit roots per direction: with the unit roots alone these grids leave
+    256 to 8,192 bytes of the library's 8 MB workspace, and the (cos, tan) form takes no more."""
+    L = native[1]
+    h, size = _plan(native, nx, ny, nz, 0, flags=flags)
+    assert size <= 8 << 20
+    L.poisson_solve_static_ws.argtypes = [ctypes.c_void_p] * 4
+    assert L.poisson_solve_static_ws(h, PTR, PTR << 1, None) == 0
+    L.poisson_plan_destroy(h)
