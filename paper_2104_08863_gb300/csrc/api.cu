@@ -250,7 +250,6 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
   pl->tridiag = d->tridiag;
   pl->flags = d->flags;
   if (!factor(g.M, pl->fm) || !factor(g.nz, pl->fz) || g.M < 2) { delete pl; return PS_EUNSUPPORTED; }
-  const bool auto_part = d->tridiag != PT_THOMAS && d->pdd_parts <= 0;
   int P = 1;
   if (d->tridiag == PT_THOMAS) P = 1;
   else if (d->pdd_parts > 0) P = d->pdd_parts;
@@ -394,7 +393,8 @@ poisson_status poisson_plan_create(const poisson_desc* d, poisson_plan_t* out) {
     const size_t nsys = (size_t)g.nz * g.ncols;
     pl->off_tri = off;
     // FP32 plans whose blocks fit in registers build their factors on the fly (no tables)
-    const bool any_height = auto_part && pp::reg_kernel_ok(ny, P);   // chosen by auto_parts
+    // by (ny, P) alone, so that the automatic partition is the same plan when a caller or the autotuner names it
+    const bool any_height = P == auto_parts(ny, d->precision) && pp::reg_kernel_ok(ny, P);
     pl->has_tri = d->precision == PP_FP64 || !(pp::reg_tridiag_ok(ny, P) || any_height);
     if (d->precision == PP_FP64) off = align_up(off + 8 * nsys * (4 * (size_t)ny + 4 * (size_t)P), 256);
     else if (pl->has_tri) off = align_up(off + 4 * nsys * (2 * (size_t)ny + 4 * (size_t)P), 256);

@@ -291,7 +291,7 @@ struct poisson_plan_s {
   size_t off_spec, off_pbuf, off_pbuf2, off_r1, off_low, off_tables, off_status, off_acc, off_tri, off_red,
       ws_bytes;
   // per-mode PDD factor tables in the workspace (FP64 plans; FP32 plans with blocks above 24 rows, or of a
-  // height outside reg_tridiag_ok that the caller named)
+  // height outside reg_tridiag_ok other than the automatic partition's)
   bool has_tri;
   size_t tab_offsets[32];
   unsigned char* ws;

@@ -109,3 +109,20 @@ def test_fp64_grids_that_just_fit_the_static_workspace(native, nx, ny, nz, flags
     L.poisson_solve_static_ws.argtypes = [ctypes.c_void_p] * 4
     assert L.poisson_solve_static_ws(h, PTR, PTR << 1, None) == 0
     L.poisson_plan_destroy(h)
+
+
+@pytest.mark.parametrize("tridiag", [2, 3])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("ny", [24, 37, 96, 130, 221, 247, 253, 289, 377])
+def test_naming_the_automatic_partition_gives_the_automatic_plan(native, ny, precision, tridiag):
+    """poisson_autotune names its candidates, and so does a caller who keeps a partition: the partition that
+    0 stands for gives the same kernels and the same workspace when it is named."""
+    def kernels(parts):
+        h, size = _plan(native, 36, ny, 16, precision, tridiag=tridiag, pdd_parts=parts)
+        out = _solve(native, h, size)
+        native[1].poisson_plan_destroy(h)
+        return size, out
+    auto = kernels(0)
+    same = [p for p in range(1, 257) if ny % p == 0 and (p <= 32 or (precision and ny // p in (1, 2, 3, 4, 6, 8)))
+            and kernels(p) == auto]
+    assert len(same) >= 1
