@@ -388,17 +388,20 @@ def tune_batch(specs, precision=PP_FP32, fp64_low_modes=4, refine_steps=1, devic
 
 def _readable(plan: Plan, fields) -> bool:
     """Whether the out-of-place kernels can read these fields as they are: what the plan's calls take
-    (checked there), at addresses that allow 16-byte accesses."""
+    (checked there), at addresses that allow 16-byte accesses, their memory holding their values (it does
+    not for a lazily negated view or a zero tensor without storage)."""
     return plan.precision != PP_FP32_REFINED and all(
         t.is_cuda and t.dtype == plan.dtype and t.is_contiguous() and tuple(t.shape) == tuple(s)
-        and t.data_ptr() % 16 == 0 for t, s in zip(fields, (plan.cell_shape, plan.v_shape, plan.cell_shape)))
+        and not t.is_neg() and not t._is_zerotensor() and t.data_ptr() % 16 == 0
+        for t, s in zip(fields, (plan.cell_shape, plan.v_shape, plan.cell_shape)))
 
 
 class ProjectionFn(torch.autograd.Function):
     """u = P(u*) (Eqs. 4, 7) with the hand-written adjoint backward P^T (same FFT/PDD kernels).
 
     Both read their arguments and write new tensors.  Arguments that the kernels cannot read in place
-    (another layout or alignment) are copied first, as before the in-place calls of a refined plan."""
+    (another alignment, slices of larger tensors) are copied first, as before the in-place calls of a
+    refined plan.  A velocity whose copy keeps a permuted layout is refused, as Plan.project refuses it."""
 
     @staticmethod
     def forward(ctx, u, v, w, plan: Plan, dt: float):

@@ -29,11 +29,13 @@ def _fields(plan, seed, how):
             b = torch.zeros((s[0], 2 * s[1], s[2]), device="cuda:0", dtype=plan.dtype)
             b[:, ::2] = t
             t = b[:, ::2]
+        elif how == "negated":      # contiguous, the memory holding -t
+            t = torch._neg_view(-t)
         out.append(t)
     return out
 
 
-@pytest.mark.parametrize("how", ["plain", "misaligned", "strided"])
+@pytest.mark.parametrize("how", ["plain", "misaligned", "strided", "negated"])
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("nx,ny,nz", [(8, 2, 2), (18, 5, 6), (36, 7, 9), (256, 3, 4)])
 def test_projection_fn_equals_in_place_calls(nx, ny, nz, precision, how):
@@ -54,6 +56,29 @@ def test_projection_fn_equals_in_place_calls(nx, ny, nz, precision, how):
         assert torch.equal(a, b)
     for a, b in zip(x, keep):
         assert torch.equal(a.detach(), b)
+
+
+def test_permuted_fields():
+    """A dense permuted velocity is refused (its copy keeps the layout), a gradient of that layout is not."""
+    P, plan = _plan(16, 4, 6, 0)
+    turn = lambda t: t.permute(2, 0, 1).contiguous().permute(1, 2, 0)
+    x, g = _fields(plan, 6, "plain"), _fields(plan, 7, "plain")
+    with pytest.raises(ValueError):
+        P.ProjectionFn.apply(*map(turn, x), plan, 0.1)
+    leaves = [t.requires_grad_(True) for t in x]
+    out = P.ProjectionFn.apply(*leaves, plan, 0.1)
+    want = torch.autograd.grad(out, leaves, grad_outputs=g, retain_graph=True)
+    for a, b in zip(torch.autograd.grad(out, leaves, grad_outputs=list(map(turn, g))), want):
+        assert torch.equal(a, b)
+
+
+def test_zero_tensor_gradient():
+    P, plan = _plan(16, 4, 6, 0)
+    leaves = [t.requires_grad_(True) for t in _fields(plan, 8, "plain")]
+    out = P.ProjectionFn.apply(*leaves, plan, 0.1)
+    zeros = [torch._efficientzerotensor(tuple(t.shape), device=t.device, dtype=t.dtype) for t in out]
+    for a in torch.autograd.grad(out, leaves, grad_outputs=zeros):
+        assert not a.any()
 
 
 def test_refused_arguments():
