@@ -48,7 +48,8 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // unless those are more than 32 and a partition into at most 32 blocks of any height <= 24 exists:
 // 253 rows are then 11 blocks of 23 and not 253 of one row, whose reduced system is a serial chain of
 // 252 interfaces on 8-byte row segments (an FP32 solve and its adjoint at 1536x253x27: 1585 us, now
-// 124).
+// 124).  Row counts above 256 that no tiled height cuts into at most 256 blocks (26 of those to 768 have a
+// partition of another height: 289, 323, 361, ...) keep the factor tables of the rule for FP64.
 int auto_parts(int ny, int precision) {
   if (precision != PP_FP64) {
     int tiled = 0;

@@ -12,7 +12,7 @@ import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-ROWS = {5: 155, 7: 203, 9: 261, 10: 290, 11: 319, 13: 377, 14: 406, 15: 435, 17: 221, 18: 522, 19: 247, 20: 260,
+ROWS = {5: 155, 7: 203, 9: 261, 10: 290, 11: 121, 13: 143, 14: 406, 15: 435, 17: 221, 18: 522, 19: 247, 20: 260,
         21: 231, 22: 242, 23: 253}
 
 
