@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
   const bool live = i0 < nx && k < nz;
   if (!live) {
     if constexpr (!SHARE) return;
-    i0 = 0;   // keeps the barriers' company on a point of its own, storing nothing
+    i0 = 0;   // takes part in the barriers with the source values of line 0, loading no base, storing nothing
     k = 0;
   }
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
@@ -194,8 +194,8 @@ __global__ void __launch_bounds__(MOM_THREADS, 2) k_momentum(Geometry g, MomArgs
     const T w_xm = __ldg(sw + o + dxm), w_xp = __ldg(sw + o + dxp);
     T wzp_xm = T(0);
     if (!shared_zp) wzp_xm = __ldg(sw + o + dzp + dxm);
-    Vt bu, bw, bv;
-    if constexpr (BASE) {
+    Vt bu{}, bw{}, bv{};
+    if (BASE && live) {   // (0, 0) has a thread of its own, which writes its result over the base in place
       bu = vldv<T, V>(a.bu + o);
       bw = vldv<T, V>(a.bw + o);
       bv = vldv<T, V>(a.bv + o);
