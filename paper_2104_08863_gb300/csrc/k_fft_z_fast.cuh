@@ -15,9 +15,10 @@
 
 namespace pp {
 
-template <typename T, int NZ> struct ZTile {
-  static constexpr int E = sizeof(T) == 4 ? 16 : 8;               // complex values per thread
-  static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;             // 64-byte row segments
+template <typename T, int NZ> struct ZTile {   // FP64 (FP32 takes the register kernel, z_reg.cuh)
+  static_assert(sizeof(T) == 8, "FP64");
+  static constexpr int E = 8;      // complex values per thread
+  static constexpr int WMIN = 4;   // 64-byte row segments
   static constexpr int W0 = (E * 64) / NZ;
   static constexpr int W = W0 < WMIN ? WMIN : (W0 > 32 ? 32 : W0);
   static constexpr int T0 = (W * NZ / E + 31) / 32 * 32;
@@ -133,7 +134,9 @@ template <typename T>
 int fft_z_fast_tile(const Geometry& g) {
   switch (g.nz) {
 #define PP_ZW_CASE(NZ) \
-    case NZ: return sizeof(T) == 4 ? ZReg<T, NZ>::W : ZTile<T, NZ>::W;
+    case NZ:                                               \
+      if constexpr (sizeof(T) == 4) return ZReg<T, NZ>::W; \
+      else return ZTile<T, NZ>::W;
     PP_Z_SIZES(PP_ZW_CASE)
 #undef PP_ZW_CASE
     default: return 0;

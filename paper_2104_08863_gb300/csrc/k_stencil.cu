@@ -219,13 +219,7 @@ static int stream_grid(size_t total) {
   return (int)(blocks < cap ? (blocks ? blocks : 1) : cap);
 }
 
-// Line-wise launch of the face stencils: one CTA per x-line at a time (grid-stride over the
-// (ny+1) nz lines), threads over x, so no per-element 64-bit index division.
-static int line_grid(const Geometry& g) {
-  const int nlines = (g.ny + 1) * g.nz;
-  const int cap = 152 * 16;
-  return nlines < cap ? nlines : cap;
-}
+// Threads over x of the line-wise divergence (one CTA per x-line at a time, grid-stride over the lines).
 static int line_block(const Geometry& g) { return g.nx >= 256 ? 256 : (g.nx + 31) / 32 * 32; }
 
 template <typename T> static const T* inv_h_table(const DevTables& tb);
