@@ -69,8 +69,8 @@ typedef enum {
 #define POISSON_GENERIC_FFT  0x4u   /* flag: use the runtime-generic FFT kernels instead of the
                                        compile-time specialised ones (a tiling the autotuner tries) */
 #define POISSON_BATCH_PERSISTENT 0x10u /* batched plans (flag of descs[0]): run the whole batch as ONE
-                                       persistent kernel over a device work queue instead of one
-                                       graph branch per instance (see poisson_solve_batched)      */
+                                       persistent kernel over a device work queue instead of a
+                                       graph of kernel branches (see poisson_solve_batched)       */
 #define POISSON_SELFTEST_WAIT 0x8u  /* diagnostics flag: the x-transform that stages its FP64
                                        input by bulk copies (FP32 plans, Nx/2 >= 256) skips its
                                        first copy, so its bounded wait runs out (~2 s): the call
@@ -241,8 +241,10 @@ poisson_status poisson_plan_batched(const poisson_desc* descs, int count, poisso
 
 /* Solve every instance i of a batched plan: rhs[i] -> p[i] (host arrays of `count` device
  * pointers, laid out and typed as for poisson_solve).  All instances run in ONE CUDA graph
- * launch on `stream`.  By default each instance's kernel sequence is a branch of the graph, so
- * kernels of different instances run concurrently.  With POISSON_BATCH_PERSISTENT (descs[0].flags)
+ * launch on `stream`.  By default the graph has branches with the kernel sequences of one instance
+ * or of several in turn (PP_FP32* batches whose spectra exceed the L2 together: as many branches
+ * as keep about 48 MB of spectra in flight, 3 at least), so kernels of different instances run
+ * concurrently.  With POISSON_BATCH_PERSISTENT (descs[0].flags)
  * and every instance a PP_FP32 plan with Nx/2 in {32,48,64,96,128,192}, Nz in
  * {64,96,128,192,256,384}, ny <= 256 and a warp-scan PDD partition (pdd_parts a power of two <= 32
  * with ny/pdd_parts in {2,3,4,6,8,12,16}; an automatic partition is chosen so), the graph is ONE
@@ -270,8 +272,8 @@ poisson_status poisson_autotune(const poisson_desc* desc, void* stream, int* pdd
  * by the plan (forked and joined with events, so the call stays stream-ordered on the caller's
  * stream).  slab_cols = 0 restores one pass over the whole spectrum.  Needs a PP_FP32 or
  * PP_FP32_REFINED plan whose blocks use the warp-scan PDD kernel (pdd_parts a power of two
- * <= 32 with ny/pdd_parts in {1,2,3,4,6,8,12,16,24}) and the specialised z-transform (nz in
- * {16,...,1024} of the form 2^a 3^b, no POISSON_GENERIC_FFT), slab_cols a multiple of the z tile
+ * <= 32 with ny/pdd_parts in {1,2,3,4,6,8,12,16,24}), nz in {16, 32, 48, 64, 96, 128, 192, 256,
+ * 384, 512, 768, 1024} without POISSON_GENERIC_FFT, slab_cols a multiple of the z tile
  * and of 256/pdd_parts and larger than fp64_low_modes (PS_EUNSUPPORTED otherwise).  Call with
  * the plan's device current (the second stream is created then); results are identical to the
  * whole-spectrum order. */

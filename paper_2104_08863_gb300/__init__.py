@@ -244,8 +244,9 @@ def autotune(nx, ny, nz, y_faces, lx=2 * np.pi, lz=np.pi, precision=PP_FP32, fp6
 
 
 class BatchPlan:
-    """Independent solves of uneven sizes run as one graph launch (poisson_solve_batched): one graph
-    branch per instance, or with persistent=True one persistent kernel over a device work queue.
+    """Independent solves of uneven sizes run as one graph launch (poisson_solve_batched): graph branches
+    that hold one instance each or, when FP32 spectra exceed the L2 together, several in turn; or with
+    persistent=True one persistent kernel over a device work queue.
 
     specs: sequence of dicts with keys nx, ny, nz, y_faces (and optional lx, lz, pdd_parts,
     flags).  With tune=True each distinct grid is autotuned once (partition count, FFT tiling).

@@ -14,8 +14,8 @@
 //
 // The tile functions are those of the standalone kernels (z_reg.cuh, k_fft_x_reg.cuh,
 // tridiag_scan.cuh), specialised for the batch sizes Nx/2 in {32, 48, 64, 96, 128, 192}, Nz in
-// {64, 96, 128, 192, 256, 384} and PDD blocks of {2, 3, 4, 6, 8, 12, 16, 24} rows (P a power of two
-// <= 32); other batches run as a graph of per-instance kernel branches (batch.cu).
+// {64, 96, 128, 192, 256, 384} and PDD blocks of {2, 3, 4, 6, 8, 12, 16} rows (P a power of two
+// <= 32); other batches run as a graph of kernel branches (batch.cu).
 #include "batch_persistent.h"
 #include "k_fft_x_reg.cuh"
 #include "tridiag_scan.cuh"

@@ -9,8 +9,11 @@
 // plain product, at any angle (at a quarter turn c is 6e-17 and t its inverse).
 // Per point a 512-point transform (8 x 8 x 8) takes 24.5 instructions instead of 31.  At 512x384x512
 // the FP64 passes went from 4.69 / 2.63 / 3.39 ms (divergence and x, z, inverse x) to 3.56 / 2.18 /
-// 2.52 ms; the error against 64 bits is no larger (velocity and pressure of a step 1.0e-14, before
-// 1.1e-14; 32x32x32 solve 8e-16, before 1.2e-15).
+// 2.52 ms.  The transform itself is the more accurate one: of random data (this code compiled for the
+// host, 40 lines a length) its rms error against an extended-precision DFT is 0.90 to 1.03 (mean 0.96)
+// times that of the plain butterflies with the same unit roots at 18 lengths from 16 to 1024 (512
+// points: 1.87e-16 and 2.01e-16; 108, the worst: 1.97e-16 and 1.93e-16).  A whole call's distance from another FP64 computation does not resolve that (two steps
+// at 512x384x512: 8.0e-15 to 9.6e-15 between seeds and runs, 9.0e-15 with the plain ones).
 #pragma once
 
 #include "fft_static.cuh"

@@ -31,8 +31,9 @@ namespace pp {
 
 // Rows per chunk: the split of the rows that minimises (CTAs on the busiest SM) x (rows + the
 // chunk's own start, worth about one row), so that small grids fill the SMs and large ones do not
-// repeat the start; at least 4 rows, at most 1024 (64 KB of coefficients).  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks
-// had at least 16 rows and filled 64 SMs.)
+// repeat the start; one chunk to four rows at most (5 or 9 rows: chunks of 3), at most 1024 rows to a
+// chunk (64 KB of coefficients).  (64x64x64 FP64: 45 us per stage on 152 SMs, 88 us when chunks had at
+// least 16 rows and filled 64 SMs.)
 int momentum_chunk_rows(long long tiles, int rows) {
   int best = rows;
   double cost = -1.0;

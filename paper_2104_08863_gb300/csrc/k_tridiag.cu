@@ -6,11 +6,11 @@
 // with a_0 = c_{ny-1} = 0 (zero wall flux).
 //
 // PDD (Sec. 2.2, Eqs. 10-21): each system is cut into P blocks of m = ny/P rows; one thread
-// owns one block, S systems share a CTA and a warp holds 32 consecutive systems of one block
-// index, so every row access is a coalesced 32-system segment.  Per block:
+// owns one block, S systems share a CTA and neighbouring threads hold consecutive systems of one
+// block index, so every row access is a coalesced segment of them.  Per block:
 //   1. forward elimination of the block matrix A_i (Eq. 20) for the data and for the spike
-//      a_1^i e_1, storing the eliminated data g_j in place and the pivots in shared memory;
-//   2. a backward recurrence that yields the block's first-row values of x~, v, w (Eq. 20);
+//      a_1^i e_1;
+//   2. the block's first-row values of x~, v, w (Eq. 20), summed up on the way;
 //   3. the reduced interface system Z (Eqs. 18, 21) solved EXACTLY, framed entries included,
 //      as a 2x2-block tridiagonal system over the P-1 interfaces by one thread per system;
 //   4. a final backward sweep that folds the two neighbour values into the right-hand side,
@@ -29,7 +29,7 @@
 
 namespace pp {
 
-// ---- PDD with per-mode factors (the production path) ----------------------------------------
+// ---- PDD with per-mode factors (FP64; FP32 blocks that do not fit in registers) ---------------
 // The RHS-independent part of each block's elimination (pivots, spikes, first-row weights)
 // depends only on the mode, so k_tridiag_setup computes it once per plan in FP64 and stores it
 // in the solve's precision.  Per solve a thread then runs, for its m rows,
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(64) k_tridiag_scan64(const __grid_constant__ G
   }
 }
 
-// ---- FP32 PDD with thread-private blocks (the FP32 production path) -------------------------
+// ---- FP32 PDD with thread-private blocks (P no power of two, or above 32) -------------------
 // One thread owns one block of M rows of one system.  It copies its M rows into a private slice
 // of shared memory with 8-byte cp.async (all M copies in flight, no register staging; layout
 // [row][thread], so every shared access of a warp is conflict-free), eliminates forward while
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(256, rows_min_ctas<M>())
 // What bounds it is the rate at which HBM serves row segments that lie nz pitch * 8 bytes apart
 // (6.4 MB at 1536x768x1024): an in-place copy in this order runs at 4.1 TB/s with 64-byte segments
 // and at 6.7 TB/s with 128-byte ones, so a CTA takes at least 16 systems: 512 threads at P = 32
-// (98 KB of shared memory, two CTAs per SM), else 256.  Per pass, against the rows kernel (4
+// (M = 24: 113,152 bytes of shared memory, 98,304 of them rows; two CTAs fill 224 of an SM's 228 KB), else 256.  Per pass, against the rows kernel (4
 // registers per row, 8 systems per CTA at P = 32): 1536x768x1024 2.13 against 2.58 ms,
 // 768x384x512 246 against 250 us; with 512 threads at P = 16 267 us.  Copies of 8 bytes cost half
 // as much again (3.0 ms), stores through shared memory 0.27 ms.  At P <= 8 the rows kernel's segments

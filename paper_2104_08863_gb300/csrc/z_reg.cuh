@@ -20,7 +20,10 @@ namespace pp {
 // Nz = 512 is split 16 x 32: CTAs of 128 threads with 32 values each in pass 1 and two rounds of 16 in
 // pass 2, four of them per SM where 32 x 16 has two of 256; the same loads are in flight, but the
 // phases of four CTAs overlap better (768x384x512: 215 us per pass, 241 before; a copy in the same
-// order takes 179).  At Nz = 1024 both factors are 32 and shared memory leaves room for three.
+// order takes 179).  Of the four lengths whose larger factor is 32 it is the only one that gains: 600 MB
+// of columns take 240 and 245 us at 768 (32 x 24 and 24 x 32), 247 and 248 us at 864 (32 x 27 and
+// 27 x 32), where the smaller CTAs leave fewer threads on an SM, against 232 and 205 us at 512; at 1024
+// both factors are 32.
 template <typename T, int NZ> struct ZReg {
   static constexpr int N1 = NZ == 512 ? 16 : split_n1(NZ), N2 = NZ / N1;
   static constexpr int WMIN = sizeof(T) == 4 ? 8 : 4;   // 64-byte row segments
