@@ -181,17 +181,17 @@ def measured_peaks():
 
 # DRAM bytes (read + write) of one fwd_x launch, from an ncu capture of the same kernel on the
 # 256x192x256 projection, scaled by the number of points (x 8.0) to the 512x384x512 launch; the
-# capture also shows the FP64 pipe 86 % busy.  Valid for the kernel as captured.
-FWD_X_FP64_TRAFFIC = {"bytes": 3.05e9, "ncu_fp64_pipe_active_pct": 85.9,
+# capture also shows the FP64 pipe 90 % busy.  Valid for the kernel as captured.
+FWD_X_FP64_TRAFFIC = {"bytes": 3.04e9, "ncu_fp64_pipe_active_pct": 90.1,
                       "source": "ncu capture at 256x192x256 scaled x8 by points"}
 
 # DRAM traffic of the momentum stages from an ncu capture of the same kernels on the 256x192x256
 # timestep, scaled by the number of points (x 8.0) to the 512x384x512 launches; the capture shows
 # the FP64 pipe 85 % busy.  Valid for the kernel as captured.
 KERNEL_TRAFFIC = {
-    "momentum_1": {"bytes": 4.74e9, "ncu_fp64_pipe_active_pct": 85.0,
+    "momentum_1": {"bytes": 4.74e9, "ncu_fp64_pipe_active_pct": 84.9,
                    "source": "ncu capture at 256x192x256 scaled x8 by points"},
-    "momentum_2": {"bytes": 7.30e9, "ncu_fp64_pipe_active_pct": 85.6,
+    "momentum_2": {"bytes": 7.29e9, "ncu_fp64_pipe_active_pct": 84.9,
                    "source": "ncu capture at 256x192x256 scaled x8 by points"},
 }
 

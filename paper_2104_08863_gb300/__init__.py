@@ -393,7 +393,7 @@ def _readable(plan: Plan, fields) -> bool:
     not for a lazily negated view or a zero tensor without storage)."""
     return plan.precision != PP_FP32_REFINED and all(
         t.is_cuda and t.dtype == plan.dtype and t.is_contiguous() and tuple(t.shape) == tuple(s)
-        and not t.is_neg() and not t._is_zerotensor() and t.data_ptr() % 16 == 0
+        and not t.is_neg() and (address := t.data_ptr()) and address % 16 == 0
         for t, s in zip(fields, (plan.cell_shape, plan.v_shape, plan.cell_shape)))
 
 
