@@ -492,6 +492,9 @@ void timer_end(Exec& ex, const char* name) {
     if (_e != cudaSuccess) return PS_ECUDA;               \
   } while (0)
 
+// After a wall-normal launch that carries the modes solved apart.
+#define PP_COUNT_SIDE() (ex.pl->launches += side_apart(ex.pl->g) ? 1 : 0)
+
 // Spectral middle of a solve on the x-transformed spectral buffer (Sec. 3.2 steps (4)-(6)):
 // forward z-transform, wall-normal systems (the (0, 0) mode and the FP64 low modes among them),
 // inverse z-transform.
@@ -506,6 +509,7 @@ poisson_status spectral_mid<double>(Exec& ex, cplx<double>* spec, GaugeMode gaug
   PP_TRY_N("fft_z_fwd", launch_fft_z<double>(g, ex.dt, pl->fz, -1, spec, st));
   PP_TRY_N("tridiag_pdd", launch_tridiag_factored(g, ex.dt, pl->parts, pl->tridiag == PT_PDD_TRUNCATED, spec,
                                                   side_args(ex.dt, -1, gauge), st));
+  PP_COUNT_SIDE();
   PP_TRY_N("fft_z_inv", launch_fft_z<double>(g, ex.dt, pl->fz, +1, spec, st));
   return PS_OK;
 }
@@ -558,6 +562,7 @@ poisson_status spectral_mid<float>(Exec& ex, cplx<float>* spec, GaugeMode gauge)
     PP_TRY_N("tridiag_pdd", launch_tridiag_factored_f32(g, ex.dt, pl->parts, pl->low, pl->tridiag == PT_PDD_TRUNCATED,
                                                         spec, side, st));
   else PP_TRY_N("tridiag_pdd", launch_tridiag_reg_f32(g, ex.dt, pl->parts, pl->low, spec, side, st));
+  PP_COUNT_SIDE();
   PP_TRY_N("fft_z_inv", launch_fft_z<float>(g, ex.dt, pl->fz, +1, spec, st));
   return PS_OK;
 }

@@ -206,6 +206,10 @@ cudaError_t launch_reduced_setup(const Geometry& g, const DevTables& tb, int par
 // rhs mean <f> in tb.acc[0]; GAUGE_OFFSET shifts the result so that the running pressure
 // total (weighted sum tb.acc[1]) plus this correction has zero weighted mean.
 enum GaugeMode { GAUGE_ZERO = 0, GAUGE_STORE_MEAN = 1, GAUGE_OFFSET = 2 };
+// Whether they are a launch of their own before the main pass: when a system's work area (16 bytes per
+// row) exceeds the 48 KB that every launch may ask for without lowering the main pass's occupancy.
+constexpr size_t kSideFusedBytes = 48 * 1024;
+inline bool side_apart(const Geometry& g) { return (size_t)16 * g.ny > kSideFusedBytes; }
 // The modes solved apart: the (0, 0) mode with the gauge, and the FP64 low modes (low >= 0).
 SideArgs side_args(const DevTables& tb, int low, GaugeMode gauge);
 // Their FP64 pivots tb.low_rb (once per plan; low >= 1).

@@ -838,11 +838,8 @@ static cudaError_t prep(K kernel, size_t smem) {
   return ensure_smem_limit((const void*)kernel, smem);
 }
 
-// The modes solved apart (low_modes.cuh): as extra CTAs of the main launch while a system's work
-// area (16 bytes per row) stays below the 48 KB that every launch may ask for without lowering the
-// main pass's occupancy, else (ny > 3072) as a launch of their own before it.
-static constexpr size_t kSideFusedBytes = 48 * 1024;
-
+// The modes solved apart (low_modes.cuh): as extra CTAs of the main launch, or (side_apart, ny > 3072) as a
+// launch of their own before it.
 template <typename TD>
 __global__ void __launch_bounds__(128) k_tridiag_side(const __grid_constant__ Geometry g,
                                                       const __grid_constant__ SideArgs sd,
@@ -871,7 +868,7 @@ static cudaError_t prepare_side(const Geometry& g, SideArgs& sd, int threads, si
                                 cudaStream_t st) {
   sd.n = 0;
   if (sd.nsys == 0) return cudaSuccess;
-  if ((size_t)16 * g.ny <= kSideFusedBytes) {
+  if (!side_apart(g)) {
     side_groups(g, sd, threads);
     const size_t need = (size_t)16 * g.ny * sd.per;
     if (smem < need) smem = need;

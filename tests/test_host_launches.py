@@ -128,3 +128,13 @@ def test_naming_the_automatic_partition_gives_the_automatic_plan(native, ny, pre
     same = [p for p in range(1, 257) if ny % p == 0 and (p <= 32 or (precision and ny // p in (1, 2, 3, 4, 6, 8)))
             and kernels(p) == auto]
     assert len(same) >= 1
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("nx,ny,nz", [(16, 8, 16), (162, 90, 108), (16, 3072, 16), (16, 3456, 16), (16, 8192, 16)])
+def test_launch_count_is_what_was_launched(native, nx, ny, nz, precision):
+    """Above 3072 rows the modes solved apart are a launch of their own."""
+    h, size = _plan(native, nx, ny, nz, precision, refine_steps=2)
+    kernels = _solve(native, h, size)
+    assert native[1].poisson_last_launch_count(h) == len(kernels)
+    native[1].poisson_plan_destroy(h)
